@@ -189,12 +189,17 @@ size_t recon_smem(const cgks_batch* b, int TA, int TB)
 
 // Set the tile shape of direction dir: the per-mesh tile counts of the work
 // list (host and device), the kernel's shared-memory limit and its persistent
-// grid at `threads` threads per block (slot dir).
+// grid at `threads` threads per block (slot dir).  The limit belongs to the
+// kernel, which every solver of the process shares: it is the largest tile's,
+// always, so that a solver tuned to a small tile leaves the launches of
+// another one, tuned to a large tile, in bounds.
 int set_tile(cgks_batch* b, int dir, int TA, int TB, int threads)
 {
     const void* fn = (const void*)b->k.recon[dir];
-    size_t smem = recon_smem(b, TA, TB);
-    CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    size_t smem = recon_smem(b, TA, TB), most = 0;
+    for (int sh = 0; sh < kNumTileShapes; ++sh)
+        most = std::max(most, recon_smem(b, kTileShapes[sh][0], kTileShapes[sh][1]));
+    CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess || occ < 1)
         return CGKS_ENOTSUP;

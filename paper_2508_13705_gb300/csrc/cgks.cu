@@ -414,6 +414,8 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
         g.dy = p->dim == 2 ? (ext[4 * k + 3] - ext[4 * k + 2]) / ny[k] : 1.0;
         g.gamma = p->gamma; g.K = K; g.thr = p->sigma_thres; g.ghi = p->gamma_hi; g.glo = p->gamma_lo;
         g.eps = p->weno_eps; g.c1 = p->tau_c1; g.c2 = p->tau_c2; g.cfl = p->cfl;
+        g.igamma = 1.0 / g.gamma; g.igm1 = 1.0 / (g.gamma - 1.0);
+        g.igf = (float)g.igamma; g.igm1f = (float)g.igm1;
         g.gf = (float)g.gamma; g.Kf = (float)g.K; g.c1f = (float)g.c1; g.c2f = (float)g.c2;
         g.idx = 1.0 / g.dx; g.idy = 1.0 / g.dy;
         g.mu = p->mu; g.muf = (float)p->mu;
@@ -1215,6 +1217,8 @@ extern "C" int cgks_step_1d_noalloc(const cgks_params* p, int nx, double x0, dou
     g.gamma = p->gamma; g.K = (3.0 - p->gamma) / (p->gamma - 1.0); g.thr = p->sigma_thres;
     g.ghi = p->gamma_hi; g.glo = p->gamma_lo; g.eps = p->weno_eps; g.c1 = p->tau_c1; g.c2 = p->tau_c2;
     g.cfl = p->cfl; g.plane = nx;
+    g.igamma = 1.0 / g.gamma; g.igm1 = 1.0 / (g.gamma - 1.0);
+    g.igf = (float)g.igamma; g.igm1f = (float)g.igm1;
     g.gf = (float)g.gamma; g.Kf = (float)g.K; g.c1f = (float)g.c1; g.c2f = (float)g.c2;
     g.idx = 1.0 / g.dx; g.idy = 1.0;
     g.mu = p->mu; g.muf = (float)p->mu;

@@ -73,6 +73,8 @@ struct Mesh {
     double bcx[4][2];               // split point along the side: bcx[0] + bcx[1] t
     float muf;
     float gf, Kf, c1f, c2f, idxf, idyf;  // FP32-bulk copies (no per-point conversions)
+    double igamma, igm1;            // 1 / gamma, 1 / (gamma - 1)
+    float igf, igm1f;
     float idxlo, idylo;             // low parts: idx = idxf + idxlo to float-float accuracy
     long long plane;                // nx * ny
     // state: planes of nx*ny doubles.  2-D: W[4] Wx[4] Wy[4] Wxl[m][4] Wyl[m][4];
@@ -144,6 +146,8 @@ template <typename R> struct MeshR;
 template <> struct MeshR<double> {
     __device__ static double gamma(const Mesh& g) { return g.gamma; }
     __device__ static double K(const Mesh& g) { return g.K; }
+    __device__ static double igamma(const Mesh& g) { return g.igamma; }
+    __device__ static double igm1(const Mesh& g) { return g.igm1; }
     __device__ static double c1(const Mesh& g) { return g.c1; }
     __device__ static double c2(const Mesh& g) { return g.c2; }
     __device__ static double mu(const Mesh& g) { return g.mu; }
@@ -153,6 +157,8 @@ template <> struct MeshR<double> {
 template <> struct MeshR<float> {
     __device__ static float gamma(const Mesh& g) { return g.gf; }
     __device__ static float K(const Mesh& g) { return g.Kf; }
+    __device__ static float igamma(const Mesh& g) { return g.igf; }
+    __device__ static float igm1(const Mesh& g) { return g.igm1f; }
     __device__ static float c1(const Mesh& g) { return g.c1f; }
     __device__ static float c2(const Mesh& g) { return g.c2f; }
     __device__ static float mu(const Mesh& g) { return g.muf; }
@@ -641,166 +647,187 @@ __device__ __forceinline__ void with_stencil(const DffR<R>& dff, Body&& body)
 
 
 // ------------------------------------------------------------------ kinetics
+//
+// Every moment the scheme needs of a micro-slope a (Eq. 2.8) is <a u^p v^q psi>
+// with <a psi> = dW prescribed: the change of rho <u^p v^q psi> of the
+// Maxwellian along dW.  The moments are known functions of (rho, U, V, theta),
+// theta = p / rho = 1 / (2 lambda), so that change is their differential: no
+// micro-slope is formed and no Gram matrix built.  Per derivative that is 7
+// operations to the variables (d rho, rho dU, rho dV, dp) and about 16 to a
+// half-range moment vector, where a slope solve (25) and a 4 x 4 Gram product
+// (20) did the same; full-range u- and v-moments are the Euler flux Jacobians,
+// which act on those variables in 7 operations each.  The FP64 flux kernel is
+// bound by the FP64 pipe: 512^2, order 9, tau = 0, two stages 11.46 -> 7.2 ms;
+// the FP32 one, bound by load latency, took 889 + 770 -> 768 + 680 us at 1024^2.
 
-// Maxwellian moments per unit density for one velocity range, with the
-// per-state factors the micro-slope solves reuse (1/rho, 1/(2 lambda),
-// 4 lambda^2 / (K + D), U^2 + V^2 + (K + D) / (2 lambda)).
+// The state variables of a Maxwellian: density, velocity, pressure, theta, and
+// the specific kinetic energy ek = (U^2 + V^2) / 2.
 template <typename R, int D>
-struct Mom {
-    R rho, U, V, lam;
-    R ir, il, c4, cs;
-    R mu[7];
-    R mv[6];
-    R x2, x4;
-};
+struct Gas { R rho, U, V, p, th, ek; };
 
-// range: 0 full, 1 u > 0, 2 u < 0.  Returns false if rho or p <= 0.
 template <typename R, int D>
-__device__ __forceinline__ bool maxwellian(const R* W, R gamma, R K, int range, Mom<R, D>& M)
+__device__ __forceinline__ Gas<R, D> gas_of(const R* W, R gm1)
 {
-    R rho = W[0];
-    R ir = (R)1 / rho;
-    R U = W[1] * ir;
-    R V = D == 2 ? W[2] * ir : (R)0;
-    R p = (gamma - (R)1) * (W[D + 1] - (R)0.5 * rho * (U * U + V * V));
-    R lam = (R)0.5 * rho / p;
-    R i2l = p * ir;  // 1 / (2 lambda)
-    M.rho = rho; M.U = U; M.V = V; M.lam = lam;
-    M.ir = ir; M.il = i2l;
-    M.c4 = (R)4 * lam * lam / (K + (R)D);
-    M.cs = U * U + V * V + (K + (R)D) * i2l;
-    if (range == 0) {
-        M.mu[0] = 1; M.mu[1] = U;
-    } else {
-        R sl = sqrt(lam);
-        R e = exp(-lam * U * U) * (R)0.28209479177387814 * rsqrt(lam);  // e^{-lam U^2} / (2 sqrt(pi lam))
-        if (range == 1) { M.mu[0] = (R)0.5 * erfc(-sl * U); M.mu[1] = U * M.mu[0] + e; }
-        else { M.mu[0] = (R)0.5 * erfc(sl * U); M.mu[1] = U * M.mu[0] - e; }
+    Gas<R, D> G;
+    G.rho = W[0];
+    const R ir = (R)1 / G.rho;
+    G.U = W[1] * ir;
+    G.V = D == 2 ? W[2] * ir : (R)0;
+    G.ek = (R)0.5 * (G.U * G.U + (D == 2 ? G.V * G.V : (R)0));
+    G.p = gm1 * (W[D + 1] - G.rho * G.ek);
+    G.th = G.p * ir;
+    return G;
+}
+
+// A derivative of the conservative variables at a state, in the variables the
+// differentials are short in: r = d rho, a = rho dU, b = rho dV, p = dp.
+template <typename R>
+struct Hat { R r, a, b, p; };
+
+template <typename R, int D>
+__device__ __forceinline__ Hat<R> hat_of(const Gas<R, D>& G, R gm1, const R* x)
+{
+    Hat<R> h;
+    h.r = x[0];
+    h.a = x[1] - G.U * x[0];
+    h.b = D == 2 ? x[2] - G.V * x[0] : (R)0;
+    R e = x[D + 1] - G.U * x[1] + G.ek * x[0];
+    if (D == 2) e -= G.V * x[2];
+    h.p = gm1 * e;
+    return h;
+}
+
+// back to conservative variables; igm1 = 1 / (gamma - 1)
+template <typename R, int D>
+__device__ __forceinline__ void unhat(const Gas<R, D>& G, R igm1, const Hat<R>& h, R* x)
+{
+    x[0] = h.r;
+    x[1] = h.a + G.U * h.r;
+    if (D == 2) x[2] = h.b + G.V * h.r;
+    R e = igm1 * h.p + G.U * h.a + G.ek * h.r;
+    if (D == 2) e += G.V * h.b;
+    x[D + 1] = e;
+}
+
+// y = F'(W) x + G'(W) z: the Jacobians of the Euler fluxes along u and v (the
+// full-range moments <a_x u psi> + <a_z v psi>); c2 = gamma theta
+template <typename R, int D>
+__device__ __forceinline__ Hat<R> euler_uv(const Gas<R, D>& G, R c2, const Hat<R>& x, const Hat<R>& z)
+{
+    Hat<R> y;
+    y.r = G.U * x.r + x.a;
+    y.a = G.U * x.a + x.p;
+    y.b = G.U * x.b;
+    y.p = G.U * x.p + c2 * x.a;
+    if (D == 2) {
+        y.r += G.V * z.r + z.b;
+        y.a += G.V * z.a;
+        y.b += G.V * z.b + z.p;
+        y.p += G.V * z.p + c2 * z.b;
     }
+    return y;
+}
+template <typename R, int D>
+__device__ __forceinline__ Hat<R> euler_u(const Gas<R, D>& G, R c2, const Hat<R>& x)
+{
+    return {G.U * x.r + x.a, G.U * x.a + x.p, G.U * x.b, G.U * x.p + c2 * x.a};
+}
+
+// Moments m[n] = <u^n> of the normal velocity over u > 0 (s = 1), u < 0 (s = -1)
+// or all of it, with their derivatives: d m_n / dU = n m_{n-1} and d m_n / dtheta
+// = n (n - 1) / 2 m_{n-2}, where the boundary at u = 0 of a half range gives
+// d m_0 / dU = k = s f(0), d m_0 / dtheta = -hk = -k U / (2 theta) and
+// d m_1 / dtheta = k / 2, f the normal distribution of mean U and variance theta.
+template <typename R, int NM>
+struct Range { R m[NM]; R k, hk; };
+
+// the cheap scaled complementary error function e^{x^2} erfc(x), x >= 0
+__device__ __forceinline__ double scaled_erfc(double x) { return erfcx(x); }
+__device__ __forceinline__ float scaled_erfc(float x) { return erfcxf(x); }
+
+// q = 1 / sqrt(theta).  One exponential serves f(0) and the error function.
+template <typename R, int D, int NM>
+__device__ __forceinline__ Range<R, NM> half_range(const Gas<R, D>& G, R q, bool left)
+{
+    Range<R, NM> H;
+    const R x = (R)0.70710678118654752 * G.U * q;  // U / sqrt(2 theta)
+    const R e = exp(-x * x);
+    const R c = (R)0.5 * e * scaled_erfc(fabs(x));   // erfc(|x|) / 2
+    H.k = (R)0.39894228040143268 * e * q;          // f(0)
+    if (!left) H.k = -H.k;
+    H.m[0] = (left ? x < (R)0 : x > (R)0) ? c : (R)1 - c;
+    H.m[1] = G.U * H.m[0] + G.th * H.k;
 #pragma unroll
-    for (int n = 0; n < 5; ++n) M.mu[n + 2] = U * M.mu[n + 1] + (R)(n + 1) * i2l * M.mu[n];
-    if (D == 2) {
-        M.mv[0] = 1; M.mv[1] = V;
+    for (int n = 0; n + 2 < NM; ++n) H.m[n + 2] = G.U * H.m[n + 1] + (R)(n + 1) * G.th * H.m[n];
+    H.hk = (R)0.5 * G.U * q * q * H.k;
+    return H;
+}
+template <typename R, int D, int NM>
+__device__ __forceinline__ Range<R, NM> full_range(const Gas<R, D>& G)
+{
+    Range<R, NM> H;
+    H.m[0] = (R)1;
+    H.m[1] = G.U;
 #pragma unroll
-        for (int n = 0; n < 4; ++n) M.mv[n + 2] = V * M.mv[n + 1] + (R)(n + 1) * i2l * M.mv[n];
-    }
-    M.x2 = K * i2l;
-    M.x4 = K * (K + (R)2) * i2l * i2l;
-    return rho > (R)0 && p > (R)0;
+    for (int n = 0; n + 2 < NM; ++n) H.m[n + 2] = G.U * H.m[n + 1] + (R)(n + 1) * G.th * H.m[n];
+    H.k = H.hk = (R)0;
+    return H;
 }
 
-// <a u^p v^q psi> per unit density, a = (a1, a2, a3, a4) on psi =
-// (1, u, v, (u^2+v^2+xi^2)/2) [2-D] or a = (a1, a2, a3) on (1, u, (u^2+xi^2)/2).
-template <typename R, int D>
-__device__ __forceinline__ void mom(const Mom<R, D>& M, const R* a, int p, int q, R* out)
+// rho <u^P psi> over the range
+template <int P, typename R, int D, int NM>
+__device__ __forceinline__ void moments(const Gas<R, D>& G, const Range<R, NM>& H, R Kx, R* out)
 {
+    const R g = (R)0.5 * (G.V * G.V + Kx * G.th);
+    const R w = G.rho * H.m[P];
+    out[0] = w;
+    out[1] = G.rho * H.m[P + 1];
+    if (D == 2) out[2] = G.V * w;
+    out[D + 1] = (R)0.5 * G.rho * H.m[P + 2] + g * w;
+}
+
+// d(rho m_n) along a derivative; t = rho d theta
+template <int N, typename R, int NM>
+__device__ __forceinline__ R dmom(const Range<R, NM>& H, const Hat<R>& h, R t)
+{
+    if (N == 0) return H.m[0] * h.r + H.k * h.a - H.hk * t;
+    if (N == 1) return H.m[1] * h.r + H.m[0] * h.a + (R)0.5 * H.k * t;
+    return H.m[N] * h.r + (R)N * H.m[N >= 1 ? N - 1 : 0] * h.a + (R)(N * (N - 1) / 2) * H.m[N >= 2 ? N - 2 : 0] * t;
+}
+
+// acc += d(rho <u^P psi>) along a derivative.  Kx = K + D - 1: the degrees of
+// freedom besides u and the mean tangential motion.
+template <int P, typename R, int D, int NM>
+__device__ __forceinline__ void add_dmoments_u(const Gas<R, D>& G, const Range<R, NM>& H, R Kx, const Hat<R>& h, R* acc)
+{
+    const R t = h.p - G.th * h.r;
+    const R g = (R)0.5 * (G.V * G.V + Kx * G.th);
+    const R d0 = dmom<P>(H, h, t);
+    acc[0] += d0;
+    acc[1] += dmom<P + 1>(H, h, t);
+    R e = (R)0.5 * dmom<P + 2>(H, h, t) + g * d0 + (R)0.5 * Kx * H.m[P] * t;
     if (D == 2) {
-        auto A = [&](int i, int j, bool xs) -> R {
-            R x0 = xs ? M.x2 : (R)1, x1 = xs ? M.x4 : M.x2;
-            R base = a[0] * M.mu[i] * M.mv[j] + a[1] * M.mu[i + 1] * M.mv[j] + a[2] * M.mu[i] * M.mv[j + 1]
-                   + (R)0.5 * a[3] * (M.mu[i + 2] * M.mv[j] + M.mu[i] * M.mv[j + 2]);
-            return x0 * base + (R)0.5 * a[3] * x1 * M.mu[i] * M.mv[j];
-        };
-        out[0] = A(p, q, false);
-        out[1] = A(p + 1, q, false);
-        out[2] = A(p, q + 1, false);
-        out[3] = (R)0.5 * (A(p + 2, q, false) + A(p, q + 2, false) + A(p, q, true));
-    } else {
-        auto A = [&](int i, bool xs) -> R {
-            R x0 = xs ? M.x2 : (R)1, x1 = xs ? M.x4 : M.x2;
-            return x0 * (a[0] * M.mu[i] + a[1] * M.mu[i + 1] + (R)0.5 * a[2] * M.mu[i + 2])
-                 + (R)0.5 * a[2] * x1 * M.mu[i];
-        };
-        out[0] = A(p, false);
-        out[1] = A(p + 1, false);
-        out[2] = (R)0.5 * (A(p + 2, false) + A(p, true));
+        const R bm = H.m[P] * h.b;
+        acc[2] += G.V * d0 + bm;
+        e += G.V * bm;
     }
+    acc[D + 1] += e;
 }
 
-// Closed-form solution of <a> = b (full-range moments, Eq. 2.8), using the
-// per-state factors of the Maxwellian.
-template <typename R, int D>
-__device__ __forceinline__ void slope(const Mom<R, D>& M, R K, const R* b, R* a)
+// acc += d(rho <u^P v psi>) along a derivative (2-D)
+template <int P, typename R, int NM>
+__device__ __forceinline__ void add_dmoments_v(const Gas<R, 2>& G, const Range<R, NM>& H, R Kx, const Hat<R>& h, R* acc)
 {
-    (void)K;
-    if (D == 2) {
-        R B0 = b[0] * M.ir, B1 = b[1] * M.ir, B2 = b[2] * M.ir, B3 = b[3] * M.ir;
-        R R2 = B1 - M.U * B0, R3 = B2 - M.V * B0;
-        R R4 = (R)2 * B3 - M.cs * B0;
-        R a4 = M.c4 * (R4 - (R)2 * M.U * R2 - (R)2 * M.V * R3);
-        R a3 = (R)2 * M.lam * R3 - M.V * a4;
-        R a2 = (R)2 * M.lam * R2 - M.U * a4;
-        a[0] = B0 - M.U * a2 - M.V * a3 - (R)0.5 * a4 * M.cs;
-        a[1] = a2; a[2] = a3; a[3] = a4;
-    } else {
-        R B0 = b[0] * M.ir, B1 = b[1] * M.ir, B2 = b[2] * M.ir;
-        R R2 = B1 - M.U * B0;
-        R R3 = (R)2 * B2 - M.cs * B0;
-        R a3 = M.c4 * (R3 - (R)2 * M.U * R2);
-        R a2 = (R)2 * M.lam * R2 - M.U * a3;
-        a[0] = B0 - M.U * a2 - (R)0.5 * a3 * M.cs;
-        a[1] = a2; a[2] = a3;
-    }
-}
-
-// Moments linear in the micro-slope: <a u^p v^q psi> = sum_k a_k G[k][i] with
-// the symmetric Gram matrix G[k][i] = <u^p v^q psi_k psi_i> per unit density.
-// A matrix serves every product with the same (p, q) and Maxwellian, which
-// costs a 4 x 4 multiply instead of a moment expansion each.  Stored as the
-// upper triangle: 2-D (00 01 02 03 11 12 13 22 23 33), 1-D (00 01 02 11 12 22).
-template <typename R, int D>
-struct Gram { R g[D == 2 ? 10 : 6]; };
-
-template <typename R, int D, int P, int Q>
-__device__ __forceinline__ void gram(const Mom<R, D>& M, Gram<R, D>& G)
-{
-    const R* m = M.mu + P;
-    if (D == 2) {
-        const R* v = M.mv + Q;
-        G.g[0] = m[0] * v[0];
-        G.g[1] = m[1] * v[0];
-        G.g[2] = m[0] * v[1];
-        G.g[3] = (R)0.5 * (m[2] * v[0] + m[0] * v[2] + M.x2 * G.g[0]);
-        G.g[4] = m[2] * v[0];
-        G.g[5] = m[1] * v[1];
-        G.g[6] = (R)0.5 * (m[3] * v[0] + m[1] * v[2] + M.x2 * G.g[1]);
-        G.g[7] = m[0] * v[2];
-        G.g[8] = (R)0.5 * (m[2] * v[1] + m[0] * v[3] + M.x2 * G.g[2]);
-        G.g[9] = (R)0.25 * (m[4] * v[0] + m[0] * v[4] + M.x4 * G.g[0]
-                            + (R)2 * (m[2] * v[2] + M.x2 * (G.g[4] + G.g[7])));
-    } else {
-        G.g[0] = m[0];
-        G.g[1] = m[1];
-        G.g[2] = (R)0.5 * (m[2] + M.x2 * m[0]);
-        G.g[3] = m[2];
-        G.g[4] = (R)0.5 * (m[3] + M.x2 * m[1]);
-        G.g[5] = (R)0.25 * (m[4] + (R)2 * M.x2 * m[2] + M.x4 * m[0]);
-    }
-}
-
-// out_i = s * sum_k a_k G[k][i]
-template <typename R, int D>
-__device__ __forceinline__ void gmul(const Gram<R, D>& G, const R* a, R s, R* out)
-{
-    if (D == 2) {
-        const R* g = G.g;
-        out[0] = s * (a[0] * g[0] + a[1] * g[1] + a[2] * g[2] + a[3] * g[3]);
-        out[1] = s * (a[0] * g[1] + a[1] * g[4] + a[2] * g[5] + a[3] * g[6]);
-        out[2] = s * (a[0] * g[2] + a[1] * g[5] + a[2] * g[7] + a[3] * g[8]);
-        out[3] = s * (a[0] * g[3] + a[1] * g[6] + a[2] * g[8] + a[3] * g[9]);
-    } else {
-        const R* g = G.g;
-        out[0] = s * (a[0] * g[0] + a[1] * g[1] + a[2] * g[2]);
-        out[1] = s * (a[0] * g[1] + a[1] * g[3] + a[2] * g[4]);
-        out[2] = s * (a[0] * g[2] + a[1] * g[4] + a[2] * g[5]);
-    }
-}
-// row 0 of G (the product with a = e_0), times s
-template <typename R, int D>
-__device__ __forceinline__ void grow0(const Gram<R, D>& G, R s, R* out)
-{
-    if (D == 2) { out[0] = s * G.g[0]; out[1] = s * G.g[1]; out[2] = s * G.g[2]; out[3] = s * G.g[3]; }
-    else { out[0] = s * G.g[0]; out[1] = s * G.g[1]; out[2] = s * G.g[2]; }
+    const R t = h.p - G.th * h.r;
+    const R g = (R)0.5 * (G.V * G.V + Kx * G.th);
+    const R d0 = dmom<P>(H, h, t), d1 = dmom<P + 1>(H, h, t);
+    const R bm = H.m[P] * h.b, tm = H.m[P] * t;
+    acc[0] += G.V * d0 + bm;
+    acc[1] += G.V * d1 + H.m[P + 1] * h.b;
+    acc[2] += (G.V * G.V + G.th) * d0 + (R)2 * G.V * bm + tm;
+    // energy: V times the differential of rho <u^P psi_4>, that moment times dV, and rho <u^P> V theta
+    const R de = (R)0.5 * dmom<P + 2>(H, h, t) + g * d0 + G.V * bm + (R)0.5 * Kx * tm;
+    acc[3] += G.V * (de + G.th * d0 + tm) + ((R)0.5 * H.m[P + 2] + g * H.m[P] + G.th * H.m[P]) * h.b;
 }
 
 } // namespace cgks

@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
         else if (dir == 0) { unsigned d = na + 1, q = r / d; f = (int)(r - q * d); b = (int)q; }
         else { unsigned d = nb, q = r / d; b = (int)(r - q * d); f = (int)q; }
         const R* FR = (const R*)g.FR[dir];
-        const R gm = MeshR<R>::gamma(g), K = MeshR<R>::K(g);
+        const R gm = MeshR<R>::gamma(g), gm1 = gm - (R)1, Kx = MeshR<R>::K(g) + (R)(D - 1);
         constexpr bool hgks = HG != 0;  // the collision-time terms of Eq. 2.6 (tau > 0)
         const long long npt = fr_npt(na, nb, M);
         const long long p00 = fr_row(dir, na, nb, b, f) * M;
@@ -544,7 +544,6 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
         // point fallback may still change the states
         bool lin = false;
         R Dl[4] = {0, 0, 0, 0};
-        R e1v[4] = {1, 0, 0, 0};
         R Q0[4] = {0, 0, 0, 0};
         R dQ[ND][4];
 #pragma unroll
@@ -553,7 +552,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
             for (int v = 0; v < 4; ++v) dQ[q][v] = 0;
         R T5[4] = {0, 0, 0, 0}, T6[4] = {0, 0, 0, 0}, S1h[4] = {0, 0, 0, 0};
         R pz[2], mn[2], mt[2];
-        bool bad = false, ok = true;
+        bool ok = true;
 #pragma unroll kSides
         for (int side = 0; side < 2; ++side) {
             // Step 2 data: W, W_n, W_nn (FP32 bulk: W as an increment over hb1);
@@ -597,32 +596,21 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
                     atomicAdd(g.nfall, 1ull);
                 }
             }
-            // Eq. 3.2 ingredients and the positivity test, in the precision the
-            // states carry (the face means, stencil sums and branch thresholds
-            // that use sigma are FP64)
-            {
-                R rho = ws[0];
-                R ir = (R)1 / rho;
-                R un = ws[1] * ir;
-                R ut = D == 2 ? ws[2] * ir : (R)0;
-                R p = (gm - (R)1) * (ws[NV - 1] - (R)0.5 * rho * (un * un + ut * ut));
-                R ic = (R)1 / sqrt(gm * p * ir);
-                pz[side] = p; mn[side] = un * ic; mt[side] = ut * ic;
-                bad |= !(rho > (R)0) || !(p > (R)0);
-            }
+            // the side's state variables serve Eq. 3.2 (in the precision the
+            // states carry: the face means, stencil sums and branch thresholds
+            // that use sigma are FP64), the positivity test and the moments
+            const Gas<R, D> Gs = gas_of<R, D>(ws, gm1);
+            const R q = rsqrt(Gs.th);
+            pz[side] = Gs.p; mn[side] = Gs.U * q; mt[side] = Gs.V * q;
+            ok &= Gs.rho > (R)0 && Gs.p > (R)0;
             // kinetic weighting (Eq. 2.7): this side's half-range integrals
-            Mom<R, D> Ms;
-            ok &= maxwellian<R, D>(ws, gm, K, side == 0 ? 1 : 2, Ms);
-            Gram<R, D> Gs;  // half-range <psi psi> of this side
-            gram<R, D, 0, 0>(Ms, Gs);
-            R t[4], z[4];
-            grow0<R, D>(Gs, Ms.rho, t);
+            const Range<R, hgks ? 5 : 3> Hs = half_range<R, D, hgks ? 5 : 3>(Gs, q, side == 0);
             if (BULK32 && side == 0) {
                 // Q0 = W_r + (H(W_l) - H(W_r)), H the u > 0 half-range moments;
                 // for a small jump, H(W_l) - H(W_r) = dH/dW (W_l - W_r) to second
-                // order, where dH/dW dW = <psi a>_{u > 0} with <a> = dW: the
-                // rounding then stays relative to the jump.  W_l - W_r is the
-                // difference of the two increments (a face's states share a base).
+                // order: the rounding then stays relative to the jump.  W_l - W_r
+                // is the difference of the two increments (a face's states share
+                // a base).
                 R e1[4], dW[4];
                 ld4(FR + npt * 12 + (p00 + rs + l) * 8, e1);
                 const R sc = fabs(hb1[0]) + fabs(hb1[NV - 1]);
@@ -632,38 +620,36 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
                     dW[v] = d0[v] - e1[v];
                     lin &= fabs(dW[v]) <= (R)2.5e-4 * sc;
                 }
-                if (NV < 4) dW[3] = (R)0;
-                if (lin) {
-                    R aa[4];
-                    slope<R, D>(Ms, K, dW, aa);
-                    gmul<R, D>(Gs, aa, Ms.rho, PF ? Dl : Q0);
-                }
+                if (lin) add_dmoments_u<0>(Gs, Hs, Kx, hat_of<R, D>(Gs, gm1, dW), PF ? Dl : Q0);
             }
+            R t[4];
             if (!(BULK32 && lin && !PF)) {
+                moments<0>(Gs, Hs, Kx, t);
 #pragma unroll
                 for (int v = 0; v < NV; ++v) Q0[v] += t[v];
             }
             if (hgks) {
-                mom<R, D>(Ms, e1v, 1, 0, t);
+                moments<1>(Gs, Hs, Kx, t);
 #pragma unroll
-                for (int v = 0; v < NV; ++v) T5[v] += Ms.rho * t[v];
+                for (int v = 0; v < NV; ++v) T5[v] += t[v];
             }
-            // one derivative: its micro-slope (<a> = dW of this side, Eq. 2.8)
-            // into the weighted derivative dQ[q], and for q = 0 (n) and 2 (t) the
-            // half-range (a_n u + a_t v) terms of Eq. 2.6 with and without the
-            // flux's u
-            auto fold = [&](int q, const R dv[4]) {
-                R a_[4];
-                slope<R, D>(Ms, K, dv, a_);
-                gmul<R, D>(Gs, a_, Ms.rho, t);
-#pragma unroll
-                for (int v = 0; v < NV; ++v) dQ[q][v] += t[v];
-                if (hgks && (q == 0 || (D == 2 && q == 2))) {
-                    int pu = q == 0 ? 1 : 0, pv = q == 0 ? 0 : 1;
-                    mom<R, D>(Ms, a_, pu, pv, t);
-                    mom<R, D>(Ms, a_, pu + 1, pv, z);
-#pragma unroll
-                    for (int v = 0; v < NV; ++v) { S1h[v] += Ms.rho * t[v]; T6[v] += Ms.rho * z[v]; }
+            // one derivative into the weighted derivative dQ[q], and for q = 0 (n)
+            // and 2 (t) the half-range (a_n u + a_t v) terms of Eq. 2.6 without
+            // and with the flux's u
+            auto fold = [&](int q, const R* dv) {
+                const Hat<R> h = hat_of<R, D>(Gs, gm1, dv);
+                add_dmoments_u<0>(Gs, Hs, Kx, h, dQ[q]);
+                if constexpr (hgks) {
+                    if (q == 0) {
+                        add_dmoments_u<1>(Gs, Hs, Kx, h, S1h);
+                        add_dmoments_u<2>(Gs, Hs, Kx, h, T6);
+                    }
+                    if constexpr (D == 2) {
+                        if (q == 2) {
+                            add_dmoments_v<0>(Gs, Hs, Kx, h, S1h);
+                            add_dmoments_v<1>(Gs, Hs, Kx, h, T6);
+                        }
+                    }
                 }
             };
             fold(0, dn[0]);
@@ -748,81 +734,44 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
         double sig;
         {
             R dpz = fabs(pz[0] - pz[1]);
-            sig = (double)(dpz / pz[0] + dpz / pz[1] + (mn[0] - mn[1]) * (mn[0] - mn[1]) + (mt[0] - mt[1]) * (mt[0] - mt[1]));
+            sig = (double)(dpz / pz[0] + dpz / pz[1]
+                           + MeshR<R>::igamma(g) * ((mn[0] - mn[1]) * (mn[0] - mn[1]) + (mt[0] - mt[1]) * (mt[0] - mt[1])));
         }
-        // equilibrium state g0 and its micro-slopes, time derivatives (Eq. 2.8)
+        // equilibrium state g0 (Eq. 2.8): derivatives in the variables of its
+        // Euler Jacobians, S1 = <a_n u + a_t v>, A = -S1, the time derivatives
+        // y1, y2 of W_n and W_t, S2 = <A1t u + A2t v>, and <A u>
         const R Dt = MeshR<R>::dt(g);
-        Mom<R, D> M0;
-        ok &= maxwellian<R, D>(Q0, gm, K, 0, M0);
-        // <u psi psi> and <v psi psi> of g0 serve every u- and v-weighted moment below
-        Gram<R, D> Gu, Gv;
-        gram<R, D, 1, 0>(M0, Gu);
-        if (D == 2) gram<R, D, 0, 1>(M0, Gv);
-        R S1[4], S2[4], z[4], rhs[4], Ab[4], A1t[4], A2t[4] = {0, 0, 0, 0};
-        R an[4], at2[4];
-        slope<R, D>(M0, K, dQ[0], an);
-        gmul<R, D>(Gu, an, (R)1, S1);
-        if (D == 2) {
-            slope<R, D>(M0, K, dQ[2], at2);
-            gmul<R, D>(Gv, at2, (R)1, z);
+        const Gas<R, D> G0 = gas_of<R, D>(Q0, gm1);
+        ok &= G0.rho > (R)0 && G0.p > (R)0;
+        const R igm1 = MeshR<R>::igm1(g), cs2 = gm * G0.th;
+        Hat<R> hx[ND];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) S1[v] += z[v];
-        }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) { S1[v] *= M0.rho; rhs[v] = -S1[v]; }
-        slope<R, D>(M0, K, rhs, Ab);
-        {
-            R ann[4];
-            slope<R, D>(M0, K, dQ[1], ann);
-            gmul<R, D>(Gu, ann, (R)1, rhs);
-        }
-        if (D == 2) {
-            R ant[4];
-            slope<R, D>(M0, K, dQ[4], ant);
-            gmul<R, D>(Gv, ant, (R)1, z);
-#pragma unroll
-            for (int v = 0; v < NV; ++v) rhs[v] += z[v];
-            R s2[4];
-            gmul<R, D>(Gu, ant, (R)1, s2);
-#pragma unroll
-            for (int v = 0; v < NV; ++v) rhs[v] *= -M0.rho;
-            slope<R, D>(M0, K, rhs, A1t);
-            R att[4];
-            slope<R, D>(M0, K, dQ[3], att);
-            gmul<R, D>(Gv, att, (R)1, z);
-#pragma unroll
-            for (int v = 0; v < NV; ++v) rhs[v] = -M0.rho * (s2[v] + z[v]);
-            slope<R, D>(M0, K, rhs, A2t);
-        } else {
-#pragma unroll
-            for (int v = 0; v < NV; ++v) rhs[v] *= -M0.rho;
-            slope<R, D>(M0, K, rhs, A1t);
-        }
-        gmul<R, D>(Gu, A1t, (R)1, S2);
-        if (D == 2) {
-            gmul<R, D>(Gv, A2t, (R)1, z);
-#pragma unroll
-            for (int v = 0; v < NV; ++v) S2[v] += z[v];
-        }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) S2[v] *= M0.rho;
+        for (int q = 0; q < ND; ++q) hx[q] = hat_of<R, D>(G0, gm1, dQ[q]);
+        const Hat<R> s1 = euler_uv<R, D>(G0, cs2, hx[0], hx[D == 2 ? 2 : 0]);
+        Hat<R> y1 = euler_uv<R, D>(G0, cs2, hx[1], hx[D == 2 ? 4 : 0]);
+        Hat<R> y2 = {0, 0, 0, 0};
+        if (D == 2) y2 = euler_uv<R, D>(G0, cs2, hx[D == 2 ? 4 : 0], hx[D == 2 ? 3 : 0]);
+        y1 = {-y1.r, -y1.a, -y1.b, -y1.p};
+        y2 = {-y2.r, -y2.a, -y2.b, -y2.p};
+        const Hat<R> s2 = euler_uv<R, D>(G0, cs2, y1, y2);
+        const Hat<R> ft = euler_u<R, D>(G0, cs2, s1);  // <A u> = -ft
         // flux terms <u> and <A u>; the linear / quadratic fits of Eq. 2.19-2.20
         // and 2.29 reduce to F = <u>, F_t = <A u>, W_t = -S1, W_tt = -S2 at tau = 0
         R F[4], Ft[4], Wt[4], Wtt[4];
-        grow0<R, D>(Gu, (R)1, F);
-        gmul<R, D>(Gu, Ab, (R)1, Ft);
+        F[0] = Q0[1];
+        F[1] = Q0[1] * G0.U + G0.p;
+        if (D == 2) F[2] = Q0[1] * G0.V;
+        F[NV - 1] = G0.U * (Q0[NV - 1] + G0.p);
+        unhat<R, D>(G0, igm1, ft, Ft);
+        unhat<R, D>(G0, igm1, s1, Wt);
+        unhat<R, D>(G0, igm1, s2, Wtt);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            F[v] *= M0.rho;
-            Ft[v] *= M0.rho;
-            Wt[v] = -S1[v];
-            Wtt[v] = -S2[v];
-        }
+        for (int v = 0; v < NV; ++v) { Ft[v] = -Ft[v]; Wt[v] = -Wt[v]; Wtt[v] = -Wtt[v]; }
         // the flux carried out: F itself (FP64), or its increment over the Euler
         // flux of hb1 (FP32 bulk; that flux is added in the update): the Euler
         // flux of Q0 = hb1 + qv taken as a difference
         R Fo[4];
-        if (BULK32) euler_flux_delta<D>(hb1, qv, gm - (R)1, Fo);
+        if (BULK32) euler_flux_delta<D>(hb1, qv, gm1, Fo);
         else {
 #pragma unroll
             for (int v = 0; v < 4; ++v) Fo[v] = F[v];
@@ -830,23 +779,17 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
         if (hgks) {
             // inviscid: c1 dt; viscous (Sec. 4): mu / p with p the pressure of
             // the equilibrium state at the face point
-            R base = g.tau_mode == 2 ? MeshR<R>::mu(g) / (M0.rho * M0.il) : MeshR<R>::c1(g) * Dt;
+            R base = g.tau_mode == 2 ? MeshR<R>::mu(g) / G0.p : MeshR<R>::c1(g) * Dt;
             R tau = base + MeshR<R>::c2(g) * fabs(pz[0] - pz[1]) / (pz[0] + pz[1]) * Dt;
             // collision and non-equilibrium terms of Eq. 2.6, fitted analytically
-            R Att[4], T2[4], T3[4], T4[4];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) rhs[v] = -S2[v];
-            slope<R, D>(M0, K, rhs, Att);
-            gmul<R, D>(Gu, Att, (R)1, T2);
-            mom<R, D>(M0, an, 2, 0, T3);
-            mom<R, D>(M0, A1t, 2, 0, T4);
-            if (D == 2) {
-                mom<R, D>(M0, at2, 1, 1, z);
-#pragma unroll
-                for (int v = 0; v < NV; ++v) T3[v] += z[v];
-                mom<R, D>(M0, A2t, 1, 1, z);
-#pragma unroll
-                for (int v = 0; v < NV; ++v) T4[v] += z[v];
+            R T2[4], T3[4] = {0, 0, 0, 0}, T4[4] = {0, 0, 0, 0};
+            unhat<R, D>(G0, igm1, euler_u<R, D>(G0, cs2, s2), T2);  // <Att u> = -T2
+            const Range<R, 5> H0 = full_range<R, D, 5>(G0);
+            add_dmoments_u<2>(G0, H0, Kx, hx[0], T3);
+            add_dmoments_u<2>(G0, H0, Kx, y1, T4);
+            if constexpr (D == 2) {
+                add_dmoments_v<1>(G0, H0, Kx, hx[2], T3);
+                add_dmoments_v<1>(G0, H0, Kx, y2, T4);
             }
             R ed = exp(-Dt / tau), eh = exp((R)-0.5 * Dt / tau);
             R h = (R)0.5 * Dt;
@@ -856,12 +799,12 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
             R f1 = ((R)4 * E1h - E1d) / Dt, g1 = (R)4 * (E1d - (R)2 * E1h) / (Dt * Dt);
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                R T3s = T3[v] * M0.rho, T4s = T4[v] * M0.rho, T2s = T2[v] * M0.rho;
+                const R T3s = T3[v], T4s = T4[v], T2s = -T2[v];
                 R T0v = F[v], T1v = Ft[v];
                 // F = T0 + (the terms below); FP32 bulk adds them to the increment
                 Fo[v] += -f0 * T0v - tau * T1v + (f1 - tau) * T3s + f0 * T5[v] - f1 * T6[v];
                 Ft[v] = -g0 * T0v + T1v - tau * T2s + g1 * T3s - tau * T4s + g0 * T5[v] - g1 * T6[v];
-                R dS = S1[v] - S1h[v];
+                R dS = -Wt[v] - S1h[v];  // S1 - S1h
                 Wt[v] += ((R)2 * eh - ed) * dS;
                 Wtt[v] += (R)4 * (ed - eh) / Dt * dS;
             }
@@ -896,7 +839,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
             st4(FO + fo_off(nf, M, q, l, face), o[q]);
         }
         if (STAGE == 1) g.SP[dir][pt] = sig;
-        if (bad || !ok || !finite) flag_bad(g, pt);
+        if (!ok || !finite) flag_bad(g, pt);
     }
 }
 

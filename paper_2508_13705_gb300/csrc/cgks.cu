@@ -54,8 +54,13 @@ int load_tables()
         for (int a = 0; a < 4; ++a) {
             f[k].gx[a] = (float)t[k].gx[a];
             f[k].gw[a] = (float)t[k].gw[a];
-            for (int b = 0; b < 12; ++b) { f[k].d1[a][b] = (float)t[k].d1[a][b]; f[k].d2[a][b] = (float)t[k].d2[a][b]; }
         }
+        for (int a = 0; a < 2; ++a)
+            for (int b = 0; b < 2; ++b)
+                for (int c = 0; c < 7; ++c) {
+                    f[k].sd1[a][b][c] = (float)t[k].sd1[a][b][c];
+                    f[k].sd2[a][b][c] = (float)t[k].sd2[a][b][c];
+                }
     }
     // one upload per translation unit (its constant tables serve both kernel sets)
     Kfns all[8] = {kfns_1_1_d(true), kfns_1_1_f(true), kfns_2_2_d(true), kfns_2_3_d(true), kfns_2_4_d(true),
@@ -89,8 +94,8 @@ Kfns pick_kfns(int dim, int order, int prec, int tau_mode, const int bc[4], int 
 }
 
 // Work lists: tiles of the 2-D Steps 1-2 per direction (their counts follow
-// the tile shape of each direction), 1-D cells of Step 2, face points, cells,
-// faces.
+// the tile shape of each direction), 1-D cells of Step 2, strips of faces of the
+// flux (2-D: one step of a warp; 1-D: a face), cells, faces.
 enum { W_TILE0 = 0, W_TILE1, W_NORMAL, W_FLUX, W_CELLS, W_SIGINIT, W_COUNT };
 
 // Tile shapes (cells along the normal x across it) the autotuner tries for
@@ -156,15 +161,20 @@ long long tiles(int dir, int nx, int ny, int TA, int TB)
 
 long long items(int kind, int dim, int M, int nx, int ny)
 {
-    (void)M;
     switch (kind) {
     case W_TILE0: return dim == 2 ? tiles(0, nx, ny, kTileShapes[0][0], kTileShapes[0][1]) : 0;
     case W_TILE1: return dim == 2 ? tiles(1, nx, ny, kTileShapes[0][0], kTileShapes[0][1]) : 0;
     case W_NORMAL: return dim == 2 ? 0 : nx + 2;
-    case W_FLUX: return dim == 2 ? ((long long)(nx + 1) * ny + (long long)(ny + 1) * nx) * M : nx + 1;
+    case W_FLUX: return dim == 2 ? flux_steps(M, nx, ny) : nx + 1;
     case W_CELLS: return (long long)nx * ny;
     default: return dim == 2 ? (long long)(nx + 1) * ny + (long long)(ny + 1) * nx : nx + 1;
     }
+}
+
+// Dynamic shared memory of a launch: the 2-D flux keeps a ring per warp.
+size_t dyn_smem(const cgks_batch* b, int kind, int threads)
+{
+    return b->dim == 2 && kind == W_FLUX ? (size_t)(threads / 32) * b->k.flux_warp_bytes : 0;
 }
 
 int launch(cgks_batch* b, const void* fn, int kind, int gi, int stage, bool has_stage)
@@ -172,12 +182,14 @@ int launch(cgks_batch* b, const void* fn, int kind, int gi, int stage, bool has_
     Work w = work_of(b, kind);
     if (w.total == 0) return CGKS_OK;
     int threads = b->threads[gi];
-    long long need = (w.total + threads - 1) / threads;
+    // a work item takes a thread, in the 2-D flux a warp
+    const long long per = b->dim == 2 && kind == W_FLUX ? threads / 32 : threads;
+    long long need = (w.total + per - 1) / per;
     int grid = (int)std::min<long long>(need, (long long)b->grid[gi]);
     if (grid < 1) grid = 1;
     void* args2[] = {&w, &stage};
     void* args1[] = {&w};
-    CK(cudaLaunchKernel(fn, dim3(grid), dim3(threads), has_stage ? args2 : args1, 0, b->stream));
+    CK(cudaLaunchKernel(fn, dim3(grid), dim3(threads), has_stage ? args2 : args1, dyn_smem(b, kind, threads), b->stream));
     return CGKS_OK;
 }
 
@@ -335,7 +347,7 @@ Layout layout(int dim, int M, size_t rs, int nx, int ny)
     for (int d = 0; d < 2; ++d) {
         int na = d == 0 ? nx : ny, nb = d == 0 ? ny : nx;
         bool on = dim == 2 || d == 0;
-        L.FR[d] = o; o = align256(o + (on ? (size_t)(nb + 2) * (na + 1) * M * 24 * rs : 0));
+        L.FR[d] = o; o = align256(o + (on ? (size_t)fr_nrow(d, na, nb) * M * 24 * rs : 0));
         L.FO[d] = o; o = align256(o + (on ? (size_t)nb * (na + 1) * M * 16 * rs : 0));
         L.SP[d] = o; o = align256(o + (on ? (size_t)nb * (na + 1) * M * 8 : 0));
         L.AT[d] = o; o = align256(o + (on && dim == 2 ? (size_t)(nb + 2) * (na + 6) * rs : 0));
@@ -365,6 +377,8 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
         // the kernels index a mesh's work items in 32 bits
         for (int kind = 0; kind < W_COUNT; ++kind)
             if (items(kind, p->dim, (p->order - 1) / 2, nx[k], ny[k]) >= (1LL << 31)) return CGKS_EINVAL;
+        if (p->dim == 2 && ((long long)(nx[k] + 1) * ny[k] + (long long)(ny[k] + 1) * nx[k]) * ((p->order - 1) / 2) >= (1LL << 31))
+            return CGKS_EINVAL;
     }
     if ((r = load_tables())) return r;
     cgks_batch* b = new (std::nothrow) cgks_batch();
@@ -490,11 +504,22 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
             int occ = 1;
             int th = (q == 2 || q == 3) ? 128 : 256;
             b->threads[q] = th;
+            if (fns[q] && p->dim == 2 && (q == 2 || q == 3)) {
+                // every flux variant may launch blocks of up to 128 threads; the
+                // limit is the kernel's, shared by all solvers of the process
+                const KOne* var = q == 2 ? b->k.flux1v : b->k.flux2v;
+                for (int c = 0; c < 2; ++c)
+                    if (cudaFuncSetAttribute((const void*)var[c], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)dyn_smem(b, W_FLUX, 128)) != cudaSuccess)
+                        rr = CGKS_ECUDA;
+            }
+            const size_t smem = q == 2 || q == 3 ? dyn_smem(b, W_FLUX, th) : 0;
             if (fns[q]) {
-                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fns[q], th, 0) != cudaSuccess) occ = 1;
+                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fns[q], th, smem) != cudaSuccess) occ = 1;
             }
             b->grid[q] = std::max(1, occ) * b->nsm;
         }
+        if (rr) break;
         // 2-D Steps 1-2: the default tile shape in both directions
         if (p->dim == 2)
             for (int d = 0; d < 2; ++d)
@@ -612,10 +637,10 @@ int post_set(cgks_batch* b, bool init_sigma)
 namespace {
 
 // Persistent grid for a kernel at a given block size: SM count x resident blocks.
-int grid_for(cgks_batch* b, const void* fn, int threads)
+int grid_for(cgks_batch* b, const void* fn, int threads, size_t smem = 0)
 {
     int occ = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, 0) != cudaSuccess || occ < 1) occ = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess || occ < 1) occ = 1;
     return occ * b->nsm;
 }
 
@@ -703,7 +728,7 @@ int autotune(cgks_batch* b, int* out)
                 int th = cand[c];
                 if (th > at.maxThreadsPerBlock) continue;
                 b->threads[q] = th;
-                b->grid[q] = grid_for(b, var[vi], th);
+                b->grid[q] = grid_for(b, var[vi], th, dyn_smem(b, kinds[qq], th));
                 float acc = 0.f;
                 for (int rep = 0; rep < 4; ++rep) {
                     CK(cudaEventRecord(e0, b->stream));
@@ -1199,7 +1224,7 @@ extern "C" int cgks_step_1d_noalloc(const cgks_params* p, int nx, double x0, dou
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o = align256(o + bytes); return at; };
     size_t oS1 = take(6 * (size_t)nx * 8), oACC = take(6 * (size_t)nx * 8), oSN = take((size_t)(nx + 1) * 8);
-    size_t oFR = take(3 * (size_t)(nx + 1) * 24 * rs), oFO = take((size_t)(nx + 1) * 16 * rs);
+    size_t oFR = take((size_t)fr_nrow(0, nx, 1) * 24 * rs), oFO = take((size_t)(nx + 1) * 16 * rs);
     size_t oSP = take((size_t)(nx + 1) * 8), oSC = take(512), oM = take(sizeof(Mesh));
     size_t oOF = take(W_COUNT * 2 * sizeof(long long));
     size_t oF = take(rs == 4 ? 2 * 9 * (size_t)nx * 4 : 0);  // FP32-bulk float planes and low parts

@@ -44,7 +44,7 @@ struct TabF {
     float bm2[3][3];
     float bm4[5][5];
     float gx[4], gw[4];
-    float d1[4][12], d2[4][12];
+    float sd1[2][2][7], sd2[2][2][7];
 };
 
 static __constant__ CgksTables c_tab[3];  // orders 5, 7, 9 (one copy per translation unit)
@@ -351,6 +351,17 @@ __device__ __forceinline__ void st4(double* p, const double v[4])
     *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
 }
 
+__device__ __forceinline__ void ld2(const float* p, float v[2])
+{
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    v[0] = q.x; v[1] = q.y;
+}
+__device__ __forceinline__ void ld2(const double* p, double v[2])
+{
+    const double2 q = *reinterpret_cast<const double2*>(p);
+    v[0] = q.x; v[1] = q.y;
+}
+
 // ------------------------------------------------------------------ float-float
 // Unevaluated sums hi + lo of two floats (Dekker's double-length arithmetic,
 // with Knuth's two-sum and the FMA two-product), about 44 significant bits:
@@ -411,18 +422,21 @@ __device__ __forceinline__ void euler_flux_ff(const float* w, ff gm1, ff* F)
     F[D + 1] = ff_mul(u, ff_add(ff_of(E), p));
 }
 
+__device__ __forceinline__ double recip(double x);
+__device__ __forceinline__ float recip(float x);
+
 // F(w0 + q) - F(w0) of the Euler flux along the local normal, by algebra in
 // which every term is a product with a component of q (no difference of two
 // O(1) values), so the result keeps the relative accuracy of q.  w0: the base
-// state (floats), q: the increment; same layouts as euler_flux_ff.
+// state (floats), q: the increment; same layouts as euler_flux_ff; ir =
+// 1 / (w0[0] + q[0]).
 template <int D, typename R>
-__device__ __forceinline__ void euler_flux_delta(const R* w0, const R* q, R gm1, R* dF)
+__device__ __forceinline__ void euler_flux_delta(const R* w0, const R* q, R ir, R gm1, R* dF)
 {
     const R r0 = w0[0], mn0 = w0[1], mt0 = D == 2 ? w0[2] : (R)0, E0 = w0[D + 1];
     const R dr = q[0], dmn = q[1], dmt = D == 2 ? q[2] : (R)0, dE = q[D + 1];
-    const R ir0 = (R)1 / r0;
+    const R ir0 = recip(r0);
     const R u0 = mn0 * ir0, v0 = mt0 * ir0;
-    const R ir = (R)1 / (r0 + dr);
     const R du = (dmn - u0 * dr) * ir, dv = (dmt - v0 * dr) * ir;  // u - u0, v - v0
     const R u = u0 + du;
     // kinetic energy rho |U|^2 / 2: its change, product by product
@@ -656,26 +670,40 @@ __device__ __forceinline__ void with_stencil(const DffR<R>& dff, Body&& body)
 // operations to the variables (d rho, rho dU, rho dV, dp) and about 16 to a
 // half-range moment vector, where a slope solve (25) and a 4 x 4 Gram product
 // (20) did the same; full-range u- and v-moments are the Euler flux Jacobians,
-// which act on those variables in 7 operations each.  The FP64 flux kernel is
-// bound by the FP64 pipe: 512^2, order 9, tau = 0, two stages 11.46 -> 7.2 ms;
-// the FP32 one, bound by load latency, took 889 + 770 -> 768 + 680 us at 1024^2.
+// which act on those variables in 7 operations each.  Alone that took the FP64
+// flux kernel, bound by the FP64 pipe, from 11.46 to 7.2 ms at 512^2, order 9,
+// tau = 0 (two stages), and the FP32 one, then bound by load latency, from
+// 889 + 770 to 768 + 680 us at 1024^2.
 
-// The state variables of a Maxwellian: density, velocity, pressure, theta, and
-// the specific kinetic energy ek = (U^2 + V^2) / 2.
+// 1 / x.  FP32: the hardware's approximation (1 ulp) and one Newton step, r +
+// r (1 - x r) with fused operations, which leaves the correctly rounded value
+// but for rare last bits; the compiled division tests for subnormal operands
+// and results besides, a fifth of the flux kernel's integer instructions.
+// x = 0 and infinite x give NaN: no physical density or pressure.
+__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+__device__ __forceinline__ float recip(float x)
+{
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return __fmaf_rn(r, __fmaf_rn(-x, r, 1.0f), r);
+}
+
+// The state variables of a Maxwellian: density and its reciprocal, velocity,
+// pressure, theta, and the specific kinetic energy ek = (U^2 + V^2) / 2.
 template <typename R, int D>
-struct Gas { R rho, U, V, p, th, ek; };
+struct Gas { R rho, ir, U, V, p, th, ek; };
 
 template <typename R, int D>
 __device__ __forceinline__ Gas<R, D> gas_of(const R* W, R gm1)
 {
     Gas<R, D> G;
     G.rho = W[0];
-    const R ir = (R)1 / G.rho;
-    G.U = W[1] * ir;
-    G.V = D == 2 ? W[2] * ir : (R)0;
+    G.ir = recip(G.rho);
+    G.U = W[1] * G.ir;
+    G.V = D == 2 ? W[2] * G.ir : (R)0;
     G.ek = (R)0.5 * (G.U * G.U + (D == 2 ? G.V * G.V : (R)0));
     G.p = gm1 * (W[D + 1] - G.rho * G.ek);
-    G.th = G.p * ir;
+    G.th = G.p * G.ir;
     return G;
 }
 
@@ -691,10 +719,34 @@ __device__ __forceinline__ Hat<R> hat_of(const Gas<R, D>& G, R gm1, const R* x)
     h.r = x[0];
     h.a = x[1] - G.U * x[0];
     h.b = D == 2 ? x[2] - G.V * x[0] : (R)0;
-    R e = x[D + 1] - G.U * x[1] + G.ek * x[0];
-    if (D == 2) e -= G.V * x[2];
-    h.p = gm1 * e;
+    h.p = gm1 * x[D + 1];
+    h.p -= (gm1 * G.U) * x[1];
+    if (D == 2) h.p -= (gm1 * G.V) * x[2];
+    h.p += (gm1 * G.ek) * x[0];
     return h;
+}
+
+// The same with t = rho d theta = dp - theta d rho in the place of dp.
+template <typename R>
+struct Var { R r, a, b, t; };
+
+template <typename R, int D>
+__device__ __forceinline__ Var<R> var_of(const Gas<R, D>& G, R gm1, const R* x)
+{
+    Var<R> h;
+    h.r = x[0];
+    h.a = x[1] - G.U * x[0];
+    h.b = D == 2 ? x[2] - G.V * x[0] : (R)0;
+    h.t = gm1 * x[D + 1];
+    h.t -= (gm1 * G.U) * x[1];
+    if (D == 2) h.t -= (gm1 * G.V) * x[2];
+    h.t += (gm1 * G.ek - G.th) * x[0];
+    return h;
+}
+template <typename R, int D>
+__device__ __forceinline__ Var<R> var_of(const Gas<R, D>& G, const Hat<R>& h)
+{
+    return {h.r, h.a, h.b, h.p - G.th * h.r};
 }
 
 // back to conservative variables; igm1 = 1 / (gamma - 1)
@@ -741,18 +793,19 @@ __device__ __forceinline__ Hat<R> euler_u(const Gas<R, D>& G, R c2, const Hat<R>
 template <typename R, int NM>
 struct Range { R m[NM]; R k, hk; };
 
-// the cheap scaled complementary error function e^{x^2} erfc(x), x >= 0
-__device__ __forceinline__ double scaled_erfc(double x) { return erfcx(x); }
-__device__ __forceinline__ float scaled_erfc(float x) { return erfcxf(x); }
+// erfc(x) / 2 for x >= 0, e = exp(-x^2).  FP64: the scaled function takes the
+// exponential that f(0) needs anyway; FP32: erfcf alone is the shorter.
+__device__ __forceinline__ double half_erfc(double x, double e) { return 0.5 * e * erfcx(x); }
+__device__ __forceinline__ float half_erfc(float x, float) { return 0.5f * erfcf(x); }
 
-// q = 1 / sqrt(theta).  One exponential serves f(0) and the error function.
+// q = 1 / sqrt(theta)
 template <typename R, int D, int NM>
 __device__ __forceinline__ Range<R, NM> half_range(const Gas<R, D>& G, R q, bool left)
 {
     Range<R, NM> H;
     const R x = (R)0.70710678118654752 * G.U * q;  // U / sqrt(2 theta)
     const R e = exp(-x * x);
-    const R c = (R)0.5 * e * scaled_erfc(fabs(x));   // erfc(|x|) / 2
+    const R c = half_erfc(fabs(x), e);
     H.k = (R)0.39894228040143268 * e * q;          // f(0)
     if (!left) H.k = -H.k;
     H.m[0] = (left ? x < (R)0 : x > (R)0) ? c : (R)1 - c;
@@ -786,48 +839,68 @@ __device__ __forceinline__ void moments(const Gas<R, D>& G, const Range<R, NM>& 
     out[D + 1] = (R)0.5 * G.rho * H.m[P + 2] + g * w;
 }
 
-// d(rho m_n) along a derivative; t = rho d theta
+// d(rho m_n) along a derivative, and s times it added to acc
 template <int N, typename R, int NM>
-__device__ __forceinline__ R dmom(const Range<R, NM>& H, const Hat<R>& h, R t)
+__device__ __forceinline__ R dmom(const Range<R, NM>& H, const Var<R>& h)
 {
-    if (N == 0) return H.m[0] * h.r + H.k * h.a - H.hk * t;
-    if (N == 1) return H.m[1] * h.r + H.m[0] * h.a + (R)0.5 * H.k * t;
-    return H.m[N] * h.r + (R)N * H.m[N >= 1 ? N - 1 : 0] * h.a + (R)(N * (N - 1) / 2) * H.m[N >= 2 ? N - 2 : 0] * t;
+    if (N == 0) return H.m[0] * h.r + H.k * h.a - H.hk * h.t;
+    if (N == 1) return H.m[1] * h.r + H.m[0] * h.a + ((R)0.5 * H.k) * h.t;
+    return H.m[N] * h.r + ((R)N * H.m[N >= 1 ? N - 1 : 0]) * h.a + ((R)(N * (N - 1) / 2) * H.m[N >= 2 ? N - 2 : 0]) * h.t;
+}
+template <int N, typename R, int NM>
+__device__ __forceinline__ void add_dmom(const Range<R, NM>& H, const Var<R>& h, R& acc)
+{
+    acc += H.m[N] * h.r;
+    acc += ((R)N * H.m[N - 1]) * h.a;
+    if (N == 1) acc += ((R)0.5 * H.k) * h.t;
+    else acc += ((R)(N * (N - 1) / 2) * H.m[N >= 2 ? N - 2 : 0]) * h.t;
 }
 
-// acc += d(rho <u^P psi>) along a derivative.  Kx = K + D - 1: the degrees of
-// freedom besides u and the mean tangential motion.
+// acc += d(rho <u^P psi>) along a derivative, as chains of fused multiply-adds.
+// Kx = K + D - 1: the degrees of freedom besides u and the mean tangential
+// motion.
 template <int P, typename R, int D, int NM>
-__device__ __forceinline__ void add_dmoments_u(const Gas<R, D>& G, const Range<R, NM>& H, R Kx, const Hat<R>& h, R* acc)
+__device__ __forceinline__ void add_dmoments_u(const Gas<R, D>& G, const Range<R, NM>& H, R Kx, const Var<R>& h, R* acc)
 {
-    const R t = h.p - G.th * h.r;
     const R g = (R)0.5 * (G.V * G.V + Kx * G.th);
-    const R d0 = dmom<P>(H, h, t);
+    const R d0 = dmom<P>(H, h);
     acc[0] += d0;
-    acc[1] += dmom<P + 1>(H, h, t);
-    R e = (R)0.5 * dmom<P + 2>(H, h, t) + g * d0 + (R)0.5 * Kx * H.m[P] * t;
+    add_dmom<P + 1>(H, h, acc[1]);
     if (D == 2) {
-        const R bm = H.m[P] * h.b;
-        acc[2] += G.V * d0 + bm;
-        e += G.V * bm;
+        acc[2] += G.V * d0;
+        acc[2] += H.m[P] * h.b;
     }
-    acc[D + 1] += e;
+    R e = acc[D + 1];
+    e += ((R)0.5 * H.m[P + 2]) * h.r;
+    e += ((R)(0.5 * (P + 2)) * H.m[P + 1]) * h.a;
+    e += (((R)(0.25 * (P + 2) * (P + 1)) + (R)0.5 * Kx) * H.m[P]) * h.t;
+    e += g * d0;
+    if (D == 2) e += (G.V * H.m[P]) * h.b;
+    acc[D + 1] = e;
 }
 
 // acc += d(rho <u^P v psi>) along a derivative (2-D)
 template <int P, typename R, int NM>
-__device__ __forceinline__ void add_dmoments_v(const Gas<R, 2>& G, const Range<R, NM>& H, R Kx, const Hat<R>& h, R* acc)
+__device__ __forceinline__ void add_dmoments_v(const Gas<R, 2>& G, const Range<R, NM>& H, R Kx, const Var<R>& h, R* acc)
 {
-    const R t = h.p - G.th * h.r;
     const R g = (R)0.5 * (G.V * G.V + Kx * G.th);
-    const R d0 = dmom<P>(H, h, t), d1 = dmom<P + 1>(H, h, t);
-    const R bm = H.m[P] * h.b, tm = H.m[P] * t;
-    acc[0] += G.V * d0 + bm;
-    acc[1] += G.V * d1 + H.m[P + 1] * h.b;
-    acc[2] += (G.V * G.V + G.th) * d0 + (R)2 * G.V * bm + tm;
+    const R d0 = dmom<P>(H, h), d1 = dmom<P + 1>(H, h);
+    const R bm = H.m[P] * h.b, tm = H.m[P] * h.t;
+    acc[0] += G.V * d0;
+    acc[0] += bm;
+    acc[1] += G.V * d1;
+    acc[1] += H.m[P + 1] * h.b;
+    acc[2] += (G.V * G.V + G.th) * d0;
+    acc[2] += ((R)2 * G.V) * bm;
+    acc[2] += tm;
     // energy: V times the differential of rho <u^P psi_4>, that moment times dV, and rho <u^P> V theta
-    const R de = (R)0.5 * dmom<P + 2>(H, h, t) + g * d0 + G.V * bm + (R)0.5 * Kx * tm;
-    acc[3] += G.V * (de + G.th * d0 + tm) + ((R)0.5 * H.m[P + 2] + g * H.m[P] + G.th * H.m[P]) * h.b;
+    R e = (g + G.th) * d0;
+    e += ((R)0.5 * H.m[P + 2]) * h.r;
+    e += ((R)(0.5 * (P + 2)) * H.m[P + 1]) * h.a;
+    e += ((R)(0.25 * (P + 2) * (P + 1) + 1.0) + (R)0.5 * Kx) * tm;
+    e += G.V * bm;
+    acc[3] += G.V * e;
+    acc[3] += ((R)0.5 * H.m[P + 2] + (g + G.th) * H.m[P]) * h.b;
 }
 
 } // namespace cgks

@@ -9,12 +9,12 @@
 // Scratch layouts per mesh and direction (na, nb: cells along / across the
 // normal; M Gauss points per face).  Direction 0 as written; direction 1 with
 // the two spatial indices swapped, so the global x index is always fastest:
-//   FR  [2]{[nb+2][na+1][M][8], [nb+2][na+1][M][4]}
-//                                     face states: side 0 = left (from cell f-1),
-//                                     side 1 = right (from cell f); per side one
-//                                     plane of (W, W_n) pairs, which Step 3 reads
-//                                     together, and one plane of W_nn
-//   FO  [4][M][nb][na+1][4]           per-point stage outputs (global frame),
+//   FR  [2][3][M][nb+2][na+1][4]      face states: side 0 = left (from cell f-1),
+//                                     side 1 = right (from cell f); W, W_n and W_nn,
+//                                     one plane per Gauss line, so that the lanes of
+//                                     a warp, which cover consecutive faces, read a
+//                                     line's points as consecutive 16-byte groups
+//   FO  [4][M][nb][na+1][4]           per-point stage outputs (local frame),
 //                                     one plane per output quantity and line
 //   SP  [nb][na+1][M]                 sigma per face Gauss point (Eq. 3.2)
 //   AT  [nb+2][na+6]                  tangential r5 DFF of each cell (Step 3)
@@ -63,6 +63,13 @@ __device__ __forceinline__ T lcell(const Mesh& g, const T* S, int dir, int lkind
     return cell<D, M, T, WALLS>(g, S, kind, vglob(dir, v), l, i, j, tb);
 }
 
+// W of a ghost cell, out of line: the flux kernel reads few of them
+template <int M, typename R>
+__device__ __noinline__ R ghost_average(const Mesh& g, const R* S, int dir, int v, int a, int b, int stage)
+{
+    return lcell<2, M, R, true>(g, S, dir, 0, v, 0, a, b, stage_time(g, stage));
+}
+
 // sigma of normal faces (f, b) and of tangential faces of column a (a, f)
 template <int D, bool WALLS = true>
 __device__ __forceinline__ double lsigN(const Mesh& g, const double* sx, const double* sy, int dir, int f, int b)
@@ -86,20 +93,27 @@ __device__ __forceinline__ long long cell_idx(int dir, int na, int nb, int a, in
 {
     return dir == 0 ? (long long)(b + 1) * (na + 6) + (a + 3) : (long long)(a + 3) * (nb + 2) + (b + 1);
 }
+// FR rows are padded to 8 points (128 bytes of FP32), so that the strips of the
+// flux kernel start on whole memory sectors: unpadded, it read 1436 MB instead
+// of 917 at 1024^2
+__host__ __device__ __forceinline__ int fr_pitch(int n) { return (n + 7) & ~7; }
 __device__ __forceinline__ long long fr_row(int dir, int na, int nb, int bb, int f)
 {
-    return dir == 0 ? (long long)bb * (na + 1) + f : (long long)f * (nb + 2) + bb;
+    return dir == 0 ? (long long)bb * fr_pitch(na + 1) + f : (long long)f * fr_pitch(nb + 2) + bb;
 }
 __device__ __forceinline__ long long pt_idx(int dir, int na, int nb, int b, int f)
 {
     return dir == 0 ? (long long)b * (na + 1) + f : (long long)f * nb + b;
 }
-// element offsets of a 16-byte group: FR (point = fr_row * M + l, npt points a
-// side) and FO (face = pt_idx, nf faces a plane)
-__device__ __forceinline__ long long fr_npt(int na, int nb, int M) { return (long long)(nb + 2) * (na + 1) * M; }
-__device__ __forceinline__ long long fr_off(long long npt, long long pt, int side, int nd)
+// element offsets of a 4-value group: FR (row = fr_row of nrow rows) and FO
+// (face = pt_idx, nf faces a plane)
+__host__ __device__ __forceinline__ long long fr_nrow(int dir, int na, int nb)
 {
-    return side * npt * 12 + (nd < 2 ? pt * 8 + nd * 4 : npt * 8 + pt * 4);
+    return dir == 0 ? (long long)(nb + 2) * fr_pitch(na + 1) : (long long)(na + 1) * fr_pitch(nb + 2);
+}
+__device__ __forceinline__ long long fr_off(long long nrow, int M, int side, int nd, int l, long long row)
+{
+    return (((long long)(side * 3 + nd) * M + l) * nrow + row) * 4;
 }
 __device__ __forceinline__ long long fo_off(long long nf, int M, int q, int l, long long face)
 {
@@ -283,7 +297,7 @@ __global__ void __launch_bounds__(256) k_recon(Work w, int stage, int TA, int TB
         const R ih = (R)1 / hn;
         const R ghi = (R)g.ghi, glo = (R)g.glo, eps = (R)g.eps;
         R* FR = (R*)g.FR[DIR];
-        const long long npt = fr_npt(na, nb, M);
+        const long long nrow = fr_nrow(DIR, na, nb);
         const long long P = g.plane;
         const int nitem = TA * TB * M;
         for (int it = threadIdx.x; it < nitem; it += blockDim.x) {
@@ -355,15 +369,15 @@ __global__ void __launch_bounds__(256) k_recon(Work w, int stage, int TA, int TB
             });
             // side 0: left state of face a+1 (value at xi = +1/2)
             if (a + 1 <= na) {
-                long long pt = fr_row(DIR, na, nb, b + 1, a + 1) * M + l;
+                const long long row = fr_row(DIR, na, nb, b + 1, a + 1);
 #pragma unroll
-                for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(npt, pt, 0, nd), sideL[nd]);
+                for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(nrow, M, 0, nd, l, row), sideL[nd]);
             }
             // side 1: right state of face a (value at xi = -1/2)
             if (a >= 0) {
-                long long pt = fr_row(DIR, na, nb, b + 1, a) * M + l;
+                const long long row = fr_row(DIR, na, nb, b + 1, a);
 #pragma unroll
-                for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(npt, pt, 1, nd), sideR[nd]);
+                for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(nrow, M, 1, nd, l, row), sideR[nd]);
             }
         }
         __syncthreads();  // the next tile reuses the shared memory
@@ -433,18 +447,18 @@ __global__ void __launch_bounds__(256) k_normal1(Work w, int stage)
 #pragma unroll
         for (int nd = 0; nd < 3; ++nd) { sideL[nd][3] = (R)0; sideR[nd][3] = (R)0; }
         R* FR = (R*)g.FR[0];
-        const long long npt = fr_npt(na, 1, 1);
+        const long long nrow = fr_nrow(0, na, 1);
         // side 0: left state of face a+1 (value at xi = +1/2)
         if (a + 1 <= na) {
-            long long pt = fr_row(0, na, 1, 1, a + 1);
+            const long long row = fr_row(0, na, 1, 1, a + 1);
 #pragma unroll
-            for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(npt, pt, 0, nd), sideL[nd]);
+            for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(nrow, 1, 0, nd, 0, row), sideL[nd]);
         }
         // side 1: right state of face a (value at xi = -1/2)
         if (a >= 0) {
-            long long pt = fr_row(0, na, 1, 1, a);
+            const long long row = fr_row(0, na, 1, 1, a);
 #pragma unroll
-            for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(npt, pt, 1, nd), sideR[nd]);
+            for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(nrow, 1, 1, nd, 0, row), sideR[nd]);
         }
     }
     __syncthreads();
@@ -453,91 +467,191 @@ __global__ void __launch_bounds__(256) k_normal1(Work w, int stage)
 }
 
 // -------------------------------------------------------------- Step 3 + flux
-// One thread per face Gauss point.  The two sides stream through one at a
-// time: each side's reconstructed data (Step 2 values, Step 3 tangential
-// derivatives), its Maxwellian half-range moments and micro-slopes are folded
-// into the kinetic weighting Q0, dQ0 (Eq. 2.7) and the half-range terms of
-// Eq. 2.6 as soon as they are formed, so only one side is live at a time.
-// CAP = 1 asks for at least 4 resident blocks of 128 threads (<= 128 registers,
-// spilling the rest); CAP = 0 for 3 in FP32 (<= 170 registers) and 1 in FP64.
-// The autotuner times both variants in FP64, where they round alike; the
-// FP32-bulk form has the uncapped one only (a capped compilation may contract
-// its FP32 arithmetic differently, and results must not depend on tuning).  HG = 1 compiles the
-// collision-time terms (tau > 0); the tau = 0 instance leaves them out and
-// carries fewer live values.  PF = true compiles the first-order fallback at
-// face points whose reconstructed state is not physical (a flagged option).
-template <int D, int M, typename R, int STAGE, int CAP, int HG, bool PF, bool ONE>
-__global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) : 1)) k_flux(Work w)
+//
+// One thread per face Gauss point.  1-D: a grid-stride loop over the faces.
+// 2-D: each warp marches along the tangential direction b of a strip of faces
+// and keeps the face states that Step 3 reads of the segments b-1, b, b+1 in
+// its own ring in shared memory, which asynchronous copies fill one step ahead.
+// A step is 32 / M faces (dir 0: 32 / M columns f of row b; dir 1: 32 / M
+// consecutive b of face row f) and has two parts: Step 3 with a lane per
+// (side, face, variable), then the kinetic part with a lane per (face, line).
+//
+// Why: with every point summing its own 3 M segment points from global memory
+// the FP32 kernel waited on those loads (762 us for stage 1 at 1024^2, order 9;
+// 582 us when they hit in L1 always), and from shared memory it spent 400
+// shared-memory passes a step on them (780 us): a 16-byte load takes four,
+// whichever lanes read alike.  A lane per variable reads 4 bytes, one pass for
+// a whole segment point of 8 faces, serves all M lines from it with weights from
+// constant memory, and sums mirrored points once for mirrored lines.  Now FP32
+// takes 512 + 448 us for the two stages (start 889 + 770), bound by issue slots:
+// 1443 instructions a point, 955 of them FP32 arithmetic, 16 warps per SM.  FP64,
+// bound by the FP64 pipe, takes 3.35 + 3.10 ms at 512^2 (start 5.96 + 5.51).  The
+// steps of a mesh are dealt to the warps in equal contiguous runs: a run has one
+// prologue, the rest streams.
+template <int M> struct FluxStrip {
+    static constexpr int FW = 32 / M;    // faces per step
+    static constexpr int RING = 3 * FW;  // ring positions: rows or blocks of rows j, j + 1, j + 2
+};
+
+// Values of one warp in shared memory: the ring of W and W_n of both sides; the
+// tangential derivatives of the step; two slots of what only the step's own
+// points read: W_nn, and the bases of the face (hi of its right cell, TD, FP32
+// bulk) with the tangential DFF of its two cells.
+template <int M, typename R>
+struct FluxShared {
+    static constexpr int FW = FluxStrip<M>::FW, RING = FluxStrip<M>::RING;
+    static constexpr bool BULK32 = sizeof(R) == 4;
+    static constexpr int ring = 0;                                    // [side][W, W_n][M][RING][4]
+    static constexpr int tang = ring + 2 * 2 * M * RING * 4;          // [side][t, tt, nt][M][FW][4]
+    static constexpr int nn = tang + 2 * 3 * M * FW * 4;              // [slot][side][M][FW][4]
+    static constexpr int hb = nn + 2 * 2 * M * FW * 4;                // [slot][FW][4]
+    static constexpr int td = hb + (BULK32 ? 2 * FW * 4 : 0);         // [slot][FW][8]
+    static constexpr int at = td + (BULK32 ? 2 * FW * 8 : 0);         // [slot][side][FW]
+    static constexpr int total = at + (2 * 2 * FW + 3) / 4 * 4;
+};
+
+// Steps (strips of 32 / M faces) of an nx x ny mesh
+__host__ __device__ inline long long flux_steps(int M, int nx, int ny)
+{
+    const int fw = 32 / M;
+    return (long long)((nx + 1 + fw - 1) / fw) * ny + (long long)(ny + 1) * ((nx + fw - 1) / fw);
+}
+
+__device__ __forceinline__ void copy_async16(void* dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+template <typename R>
+__device__ __forceinline__ void copy_async1(R* dst, const R* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"(sizeof(R))
+                 : "memory");
+}
+__device__ __forceinline__ void copy_async4(float* dst, const float* src) { copy_async16(dst, src); }
+__device__ __forceinline__ void copy_async4(double* dst, const double* src)
+{
+    copy_async16(dst, src);
+    copy_async16(dst + 2, src + 2);
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Step 3 for one (side, face, variable): the derivatives t, tt and nt at the M
+// lines of the face, from the 3 M points of segments b-1, b, b+1 (W: value of
+// the variable at ring position p of line k is W[(k * RING + p) * 4], Wn the
+// normal derivative likewise; q: ring positions of the segments).  Lines l and
+// M-1-l mirror each other: first derivatives of the even part of the points and
+// second ones of the odd part change sign.  dm, dp (FP32 bulk): the segment
+// points' values are increments over hi of the right cells (f, b-1), (f, b),
+// (f, b+1); the bases' part comes from their differences (the weights of a
+// constant sum to zero).  out[(q * M + l) * FW * 4]: quantity q at line l.
+template <int M, typename R>
+__device__ __forceinline__ void step3(const R* W, const R* Wn, const int q[3], R dm, R dp, R c1, R c2, R* out)
+{
+    constexpr int K = 3 * M, H = K / 2, RING = FluxStrip<M>::RING, FW = FluxStrip<M>::FW;
+    constexpr bool BULK32 = sizeof(R) == 4;
+    const auto& T = Tab<R>::get(M - 2);
+    R e[H + 1], o[H];
+    auto split = [&](const R* P) {
+        R x[K];
+#pragma unroll
+        for (int s = 0; s < 3; ++s)
+#pragma unroll
+            for (int k = 0; k < M; ++k) x[s * M + k] = P[(k * RING + q[s]) * 4];
+#pragma unroll
+        for (int k = 0; k < H; ++k) { e[k] = x[k] + x[K - 1 - k]; o[k] = x[k] - x[K - 1 - k]; }
+        e[H] = K % 2 ? x[H] : (R)0;
+    };
+    auto sum = [&](const R* w, const R* v, int n) {
+        R r = w[0] * v[0];
+#pragma unroll
+        for (int k = 1; k < n; ++k) r += w[k] * v[k];
+        return r;
+    };
+    split(W);
+#pragma unroll
+    for (int l = 0; l < (M + 1) / 2; ++l) {
+        R te = sum(T.sd1[l][0], e, (K + 1) / 2), to = sum(T.sd1[l][1], o, H);
+        R se = sum(T.sd2[l][0], e, (K + 1) / 2), so = sum(T.sd2[l][1], o, H);
+        if (BULK32) {
+            te += T.sd1[l][0][6] * (dm + dp);
+            to += T.sd1[l][1][6] * (dm - dp);
+            se += T.sd2[l][0][6] * (dm + dp);
+            so += T.sd2[l][1][6] * (dm - dp);
+        }
+        out[(0 * M + l) * FW * 4] = c1 * (to + te);
+        out[(1 * M + l) * FW * 4] = c2 * (se + so);
+        if (M - 1 - l != l) {
+            out[(0 * M + M - 1 - l) * FW * 4] = c1 * (to - te);
+            out[(1 * M + M - 1 - l) * FW * 4] = c2 * (se - so);
+        }
+    }
+    split(Wn);
+#pragma unroll
+    for (int l = 0; l < (M + 1) / 2; ++l) {
+        R te = sum(T.sd1[l][0], e, (K + 1) / 2), to = sum(T.sd1[l][1], o, H);
+        out[(2 * M + l) * FW * 4] = c1 * (to + te);
+        if (M - 1 - l != l) out[(2 * M + M - 1 - l) * FW * 4] = c1 * (to - te);
+    }
+}
+
+// What a face point reads, from a warp's shared memory (2-D).
+template <int M, typename R>
+struct StripPoint {
+    using L = FluxShared<M, R>;
+    const R* s;       // the warp's values
+    int slot, own_q;  // slot of the step, ring position of the point's own segment
+    int x, l;
+    __device__ __forceinline__ void own(int side, int nd, R* v) const
+    {
+        if (nd < 2) ld4(s + L::ring + (((side * 2 + nd) * M + l) * L::RING + own_q) * 4, v);
+        else ld4(s + L::nn + (((slot * 2 + side) * M + l) * L::FW + x) * 4, v);
+    }
+    __device__ __forceinline__ void base(R* v) const { ld4(s + L::hb + (slot * L::FW + x) * 4, v); }
+    __device__ __forceinline__ void tangential(int side, int q, R* v) const
+    {
+        ld4(s + L::tang + (((side * 3 + q) * M + l) * L::FW + x) * 4, v);
+    }
+};
+
+// What a 1-D face reads, from global memory.
+template <typename R>
+struct LinePoint {
+    const R* FR;
+    long long nrow, row;
+    R h[4];
+    __device__ __forceinline__ void own(int side, int nd, R* v) const { ld4(FR + fr_off(nrow, 1, side, nd, 0, row), v); }
+    __device__ __forceinline__ void base(R* v) const { for (int q = 0; q < 4; ++q) v[q] = h[q]; }
+};
+
+// One face Gauss point.  Each side's reconstructed data (Step 2 values, Step 3
+// tangential derivatives) and the differentials of its half-range moments are
+// folded into the kinetic weighting Q0, dQ0 (Eq. 2.7) and the half-range terms
+// of Eq. 2.6 as soon as they are formed.  HG = 1 compiles the collision-time
+// terms (tau > 0); the tau = 0 instance leaves them out and carries fewer live
+// values.  PF = true compiles the first-order fallback at face points whose
+// reconstructed state is not physical (a flagged option).  Dt: the step, dt26 =
+// Dt^2 / 6.
+template <int D, int M, typename R, int STAGE, int HG, bool PF, typename Point>
+__device__ __forceinline__ void flux_point(const Mesh& g, int dir, int na, int nb, int f, int b, int l, const Point& in,
+                                           R Dt, R dt26)
 {
     constexpr int NV = D + 2;
     constexpr int ND = D == 2 ? 5 : 2;  // derivatives: n, nn (, t, tt, nt)
     constexpr bool BULK32 = sizeof(R) == 4;
-    // FP32 bulk: the two sides unrolled, so that their independent chains
-    // interleave, and Step 3's segment loop rolled, which keeps the tau = 0
-    // compilation within 128 registers without spills (4 blocks of 128
-    // threads per SM; the tau > 0 ones take 168, 3 blocks)
-    constexpr int kSides = BULK32 ? 2 : 1, kSegs = BULK32 ? 1 : 3;
-    // Step 3 weights in shared memory: the Gauss line differs across the lanes
-    // of a warp, which would serialise constant-memory reads.  FP32 bulk also
-    // keeps, per line and segment, the sum of the segment's weights, which
-    // multiplies the difference of the segment cell's hi from the centre's.
-    __shared__ R s_d1[4][12], s_d2[4][12];
-    __shared__ R s_c1[4][3], s_c2[4][3];
-    if (D == 2) {
-        const auto& T = Tab<R>::get((ONE ? w.m0 : w.mesh[0]).oi);  // a table shares one order
-        for (int q = threadIdx.x; q < 48; q += blockDim.x) {
-            s_d1[q / 12][q % 12] = T.d1[q / 12][q % 12];
-            s_d2[q / 12][q % 12] = T.d2[q / 12][q % 12];
-        }
-        if (BULK32)
-            for (int q = threadIdx.x; q < 12; q += blockDim.x) {
-                R c1 = 0, c2 = 0;
-                for (int kk = 0; kk < M; ++kk) { c1 += T.d1[q / 3][(q % 3) * M + kk]; c2 += T.d2[q / 3][(q % 3) * M + kk]; }
-                s_c1[q / 3][q % 3] = c1;
-                s_c2[q / 3][q % 3] = c2;
-            }
-        __syncthreads();
-    }
-    for (long long gi = blockIdx.x * (long long)blockDim.x + threadIdx.x; gi < w.total;
-         gi += (long long)gridDim.x * blockDim.x) {
-        long long lil;
-        const Mesh& g = mesh_of<ONE>(w, gi, lil);
-        unsigned li = (unsigned)lil;  // 32-bit local index (bounded on the host)
-        int dir = 0, na = g.nx, nb = 1;
-        if (D == 2) {
-            unsigned nxl = (unsigned)(g.nx + 1) * (unsigned)g.ny * M;
-            dir = li < nxl ? 0 : 1;
-            if (dir == 1) li -= nxl;
-            local_dims<M>(g, dir, na, nb);
-        }
-        int l = D == 2 ? (int)(li % M) : 0;
-        unsigned r = D == 2 ? li / M : li;
-        int f, b;
-        if (D == 1) { f = (int)r; b = 0; }
-        else if (dir == 0) { unsigned d = na + 1, q = r / d; f = (int)(r - q * d); b = (int)q; }
-        else { unsigned d = nb, q = r / d; b = (int)(r - q * d); f = (int)q; }
-        const R* FR = (const R*)g.FR[dir];
-        const R gm = MeshR<R>::gamma(g), gm1 = gm - (R)1, Kx = MeshR<R>::K(g) + (R)(D - 1);
-        constexpr bool hgks = HG != 0;  // the collision-time terms of Eq. 2.6 (tau > 0)
-        const long long npt = fr_npt(na, nb, M);
-        const long long p00 = fr_row(dir, na, nb, b, f) * M;
-        const long long rs = (dir == 0 ? (long long)(na + 1) : 1LL) * M;  // FR row stride of the segments
-        // FP32 bulk: the state planes of this stage, whose high part hi of the
-        // face's right cell f is the base of both face states (local frame)
+    // FP32 bulk: the two sides unrolled, so that their independent chains interleave
+    constexpr int kSides = BULK32 ? 2 : 1;
+    constexpr bool hgks = HG != 0;  // the collision-time terms of Eq. 2.6 (tau > 0)
+    const R gm = MeshR<R>::gamma(g), gm1 = gm - (R)1, Kx = MeshR<R>::K(g) + (R)(D - 1);
+    {
+        // FP32 bulk: hi of the face's right cell f (local frame), the base of
+        // both face states
         const R* SF = state_planes<R>(g, STAGE == 1 ? 0 : 1);
-        const double tb = stage_time(g, STAGE);
-        // hb1: hi of the right cell f, the base of both face states
+        const double tb = PF ? stage_time(g, STAGE) : 0.0;
         R hb1[4] = {0, 0, 0, 0};
-        if (BULK32) {
-            if (f < na && (D == 1 || b < nb)) {
-                long long ci = dir == 0 ? (long long)b * g.nx + f : (long long)f * g.nx + b;
-#pragma unroll
-                for (int v = 0; v < NV; ++v) hb1[v] = SF[vglob(dir, v) * g.plane + ci];
-            } else {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) hb1[v] = lcell<D, M, R, true>(g, SF, dir, 0, v, 0, f, b, tb);
-            }
-        }
+        if (BULK32) in.base(hb1);
         // FP32 bulk: whether the jump W_l - W_r is small enough for the kinetic
         // weighting to be taken to first order in it (decided with the left
         // state, below); the first-order term, held in Q0 itself unless the
@@ -556,14 +670,12 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
 #pragma unroll kSides
         for (int side = 0; side < 2; ++side) {
             // Step 2 data: W, W_n, W_nn (FP32 bulk: W as an increment over hb1);
-            // Step 3's tangential derivatives are formed later, right before
-            // their micro-slope solves, so that few derivatives are live at once
+            // Step 3's tangential derivatives are read when they are folded in
             R d0[4], dn[2][4];
             const int a = side == 0 ? f - 1 : f;  // the reconstructing cell
-            const R* Fs = FR + side * npt * 12 + p00 * 8;  // (W, W_n) of segment b - 1
-            ld4(Fs + (rs + l) * 8, d0);
-            ld4(Fs + (rs + l) * 8 + 4, dn[0]);
-            ld4(FR + side * npt * 12 + npt * 8 + (p00 + rs + l) * 4, dn[1]);
+            in.own(side, 0, d0);
+            in.own(side, 1, dn[0]);
+            in.own(side, 2, dn[1]);
             // the side's state
             R ws[4];
 #pragma unroll
@@ -612,7 +724,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
                 // is the difference of the two increments (a face's states share
                 // a base).
                 R e1[4], dW[4];
-                ld4(FR + npt * 12 + (p00 + rs + l) * 8, e1);
+                in.own(1, 0, e1);
                 const R sc = fabs(hb1[0]) + fabs(hb1[NV - 1]);
                 lin = true;
 #pragma unroll
@@ -620,7 +732,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
                     dW[v] = d0[v] - e1[v];
                     lin &= fabs(dW[v]) <= (R)2.5e-4 * sc;
                 }
-                if (lin) add_dmoments_u<0>(Gs, Hs, Kx, hat_of<R, D>(Gs, gm1, dW), PF ? Dl : Q0);
+                if (lin) add_dmoments_u<0>(Gs, Hs, Kx, var_of<R, D>(Gs, gm1, dW), PF ? Dl : Q0);
             }
             R t[4];
             if (!(BULK32 && lin && !PF)) {
@@ -637,7 +749,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
             // and 2 (t) the half-range (a_n u + a_t v) terms of Eq. 2.6 without
             // and with the flux's u
             auto fold = [&](int q, const R* dv) {
-                const Hat<R> h = hat_of<R, D>(Gs, gm1, dv);
+                const Var<R> h = var_of<R, D>(Gs, gm1, dv);
                 add_dmoments_u<0>(Gs, Hs, Kx, h, dQ[q]);
                 if constexpr (hgks) {
                     if (q == 0) {
@@ -654,64 +766,17 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
             };
             fold(0, dn[0]);
             fold(1, dn[1]);
-            if (D == 2) {
-                // Step 3: tangential derivatives from the 3M face points of
-                // segments b-1, b, b+1, scaled by the tangential r5 DFF of the
-                // reconstructing cell (a = f-1 for the left state, f for the right)
-                R at = ((const R*)g.AT[dir])[cell_idx(dir, na, nb, a, b)];
-                R iht = (R)1 / (R)(dir == 0 ? g.dy : g.dx);
-                R c1 = fb ? (R)0 : at * iht, c2 = fb ? (R)0 : at * iht * iht;
-                {
-                    // W_t and W_tt from the points' values
-                    R wt[4] = {0, 0, 0, 0}, wtt[4] = {0, 0, 0, 0};
-#pragma unroll kSegs
-                    for (int s = 0; s < 3; ++s)
+            if constexpr (D == 2) {
+                // Step 3's tangential derivatives of this side, t, tt and nt
 #pragma unroll
-                        for (int kk = 0; kk < M; ++kk) {
-                            R x0[4];
-                            ld4(Fs + (s * rs + kk) * 8, x0);
-                            R w1 = s_d1[l][s * M + kk], w2 = s_d2[l][s * M + kk];
+                for (int q = 0; q < 3; ++q) {
+                    R dv[4];
+                    in.tangential(side, q, dv);
+                    if (PF && fb) {
 #pragma unroll
-                            for (int v = 0; v < 4; ++v) {
-                                wt[v] += w1 * x0[v];
-                                wtt[v] += w2 * x0[v];
-                            }
-                        }
-                    if (BULK32) {
-                        // the segment points' values are increments over hi of the
-                        // right cells (f, b-1), (f, b), (f, b+1): add the bases' part
-                        // from their differences (the weights of a constant sum to zero)
-                        R dm[4], dpl[4];
-                        const R* td = (const R*)g.TD[dir] + cell_idx(dir, na, nb, f, b) * 8;
-                        ld4(td, dm);
-                        ld4(td + 4, dpl);
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            wt[v] += s_c1[l][0] * dm[v] + s_c1[l][2] * dpl[v];
-                            wtt[v] += s_c2[l][0] * dm[v] + s_c2[l][2] * dpl[v];
-                        }
+                        for (int v = 0; v < 4; ++v) dv[v] = (R)0;
                     }
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) { wt[v] *= c1; wtt[v] *= c2; }
-                    fold(2, wt);
-                    fold(3, wtt);
-                }
-                {
-                    // W_nt from the points' normal derivatives
-                    R wnt[4] = {0, 0, 0, 0};
-#pragma unroll kSegs
-                    for (int s = 0; s < 3; ++s)
-#pragma unroll
-                        for (int kk = 0; kk < M; ++kk) {
-                            R x1[4];
-                            ld4(Fs + (s * rs + kk) * 8 + 4, x1);
-                            R w1 = s_d1[l][s * M + kk];
-#pragma unroll
-                            for (int v = 0; v < 4; ++v) wnt[v] += w1 * x1[v];
-                        }
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) wnt[v] *= c1;
-                    fold(4, wnt);
+                    fold(2 + q, dv);
                 }
             }
         }
@@ -720,7 +785,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
         if (BULK32) {
             if (lin) {
                 R e1[4];
-                ld4(FR + npt * 12 + (p00 + rs + l) * 8, e1);
+                in.own(1, 0, e1);
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
                     qv[v] = e1[v] + (PF ? Dl[v] : Q0[v]);
@@ -734,13 +799,12 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
         double sig;
         {
             R dpz = fabs(pz[0] - pz[1]);
-            sig = (double)(dpz / pz[0] + dpz / pz[1]
+            sig = (double)(dpz * recip(pz[0]) + dpz * recip(pz[1])
                            + MeshR<R>::igamma(g) * ((mn[0] - mn[1]) * (mn[0] - mn[1]) + (mt[0] - mt[1]) * (mt[0] - mt[1])));
         }
         // equilibrium state g0 (Eq. 2.8): derivatives in the variables of its
         // Euler Jacobians, S1 = <a_n u + a_t v>, A = -S1, the time derivatives
         // y1, y2 of W_n and W_t, S2 = <A1t u + A2t v>, and <A u>
-        const R Dt = MeshR<R>::dt(g);
         const Gas<R, D> G0 = gas_of<R, D>(Q0, gm1);
         ok &= G0.rho > (R)0 && G0.p > (R)0;
         const R igm1 = MeshR<R>::igm1(g), cs2 = gm * G0.th;
@@ -771,7 +835,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
         // flux of hb1 (FP32 bulk; that flux is added in the update): the Euler
         // flux of Q0 = hb1 + qv taken as a difference
         R Fo[4];
-        if (BULK32) euler_flux_delta<D>(hb1, qv, gm1, Fo);
+        if (BULK32) euler_flux_delta<D>(hb1, qv, G0.ir, gm1, Fo);
         else {
 #pragma unroll
             for (int v = 0; v < 4; ++v) Fo[v] = F[v];
@@ -785,11 +849,11 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
             R T2[4], T3[4] = {0, 0, 0, 0}, T4[4] = {0, 0, 0, 0};
             unhat<R, D>(G0, igm1, euler_u<R, D>(G0, cs2, s2), T2);  // <Att u> = -T2
             const Range<R, 5> H0 = full_range<R, D, 5>(G0);
-            add_dmoments_u<2>(G0, H0, Kx, hx[0], T3);
-            add_dmoments_u<2>(G0, H0, Kx, y1, T4);
+            add_dmoments_u<2>(G0, H0, Kx, var_of<R, D>(G0, hx[0]), T3);
+            add_dmoments_u<2>(G0, H0, Kx, var_of<R, D>(G0, y1), T4);
             if constexpr (D == 2) {
-                add_dmoments_v<1>(G0, H0, Kx, hx[2], T3);
-                add_dmoments_v<1>(G0, H0, Kx, y2, T4);
+                add_dmoments_v<1>(G0, H0, Kx, var_of<R, D>(G0, hx[2]), T3);
+                add_dmoments_v<1>(G0, H0, Kx, var_of<R, D>(G0, y2), T4);
             }
             R ed = exp(-Dt / tau), eh = exp((R)-0.5 * Dt / tau);
             R h = (R)0.5 * Dt;
@@ -816,30 +880,206 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
         R o[4][4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            int gv = D == 2 ? vglob(dir, v) : v;
             if (v >= NV) { o[0][v] = o[1][v] = o[2][v] = o[3][v] = (R)0; continue; }
             // interface-state values: Q0 itself, or its increment over hb1 (FP32 bulk)
             const R Qv = BULK32 ? qv[v] : Q0[v];
             if (STAGE == 1) {
-                o[0][gv] = (R)0.5 * Dt * Fo[v] + (R)0.125 * Dt * Dt * Ft[v];
-                o[1][gv] = Dt * Fo[v] + Dt * Dt / (R)6 * Ft[v];
-                o[2][gv] = Qv + (R)0.5 * Dt * Wt[v] + (R)0.125 * Dt * Dt * Wtt[v];
-                o[3][gv] = Qv + Dt * Wt[v] + Dt * Dt / (R)6 * Wtt[v];
+                o[0][v] = (R)0.5 * Dt * Fo[v] + (R)0.125 * Dt * Dt * Ft[v];
+                o[1][v] = Dt * Fo[v] + dt26 * Ft[v];
+                o[2][v] = Qv + (R)0.5 * Dt * Wt[v] + (R)0.125 * Dt * Dt * Wtt[v];
+                o[3][v] = Qv + Dt * Wt[v] + dt26 * Wtt[v];
             } else {
-                o[0][gv] = Dt * Dt / (R)3 * Ft[v];
-                o[1][gv] = Dt * Dt / (R)3 * Wtt[v];
+                o[0][v] = (R)2 * dt26 * Ft[v];
+                o[1][v] = (R)2 * dt26 * Wtt[v];
             }
         }
-        bool finite = true;
+        // finite outputs: 0 * x is 0 for finite x only
+        R zero = (R)0;
         constexpr int NO = STAGE == 1 ? 4 : 2;
 #pragma unroll
         for (int q = 0; q < NO; ++q) {
 #pragma unroll
-            for (int v = 0; v < NV; ++v) finite &= isfinite(o[q][v]);
+            for (int v = 0; v < NV; ++v) zero += (R)0 * o[q][v];
             st4(FO + fo_off(nf, M, q, l, face), o[q]);
         }
         if (STAGE == 1) g.SP[dir][pt] = sig;
-        if (!ok || !finite) flag_bad(g, pt);
+        if (!ok || !(zero == (R)0)) flag_bad(g, pt);
+    }
+}
+
+// 1-D: one thread per face.  CAP = 1 asks for at least 4 resident blocks of 128
+// threads (<= 128 registers, spilling the rest); CAP = 0 for 4, or 3 with the
+// collision-time terms, in FP32 (<= 128, 168 registers) and 1 in FP64.  The
+// autotuner times both variants in FP64, where they round alike; the FP32-bulk
+// form has the uncapped one only (a capped compilation may contract its FP32
+// arithmetic differently, and results must not depend on tuning).
+template <typename R, int STAGE, int CAP, int HG, bool PF, bool ONE>
+__global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) : 1)) k_flux1(Work w)
+{
+    for (long long gi = blockIdx.x * (long long)blockDim.x + threadIdx.x; gi < w.total;
+         gi += (long long)gridDim.x * blockDim.x) {
+        long long li;
+        const Mesh& g = mesh_of<ONE>(w, gi, li);
+        const int f = (int)li, na = g.nx;
+        const R Dt = MeshR<R>::dt(g);
+        LinePoint<R> in;
+        in.FR = (const R*)g.FR[0];
+        in.nrow = fr_nrow(0, na, 1);
+        in.row = fr_row(0, na, 1, 1, f);
+        if (sizeof(R) == 4) {
+            const R* SF = state_planes<R>(g, STAGE == 1 ? 0 : 1);
+            const double tb = stage_time(g, STAGE);
+#pragma unroll
+            for (int v = 0; v < 3; ++v) in.h[v] = cell<1, 1, R, true>(g, SF, 0, v, 0, f, 0, tb);
+            in.h[3] = (R)0;
+        }
+        flux_point<1, 1, R, STAGE, HG, PF>(g, 0, na, 1, f, 0, 0, in, Dt, Dt * Dt / (R)6);
+    }
+}
+
+// 2-D: warps marching over strips of faces (above).  Dynamic shared memory:
+// FluxShared<M, R>::total values of R per warp.  Work offsets count steps.
+template <int M, typename R, int STAGE, int CAP, int HG, bool PF, bool ONE>
+__global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flux2(Work w)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    using L = FluxShared<M, R>;
+    constexpr bool BULK32 = sizeof(R) == 4;
+    constexpr int FW = L::FW, RING = L::RING;
+    const int lane = threadIdx.x & 31, x = lane / M, l = lane - x * M;
+    R* sm = (R*)smem_raw + (threadIdx.x >> 5) * L::total;
+    const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
+    const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    long long t = wid * w.total / nw;
+    const long long tend = (wid + 1) * w.total / nw;
+    while (t < tend) {
+        long long tl;
+        const Mesh& g = mesh_of<ONE>(w, t, tl);
+        // the run's direction, strip and steps [k0, kend)
+        const int nc0 = (g.nx + 1 + FW - 1) / FW, nc1 = (g.nx + FW - 1) / FW;
+        const long long n0 = (long long)nc0 * g.ny;
+        const int dir = tl < n0 ? 0 : 1;
+        if (dir == 1) tl -= n0;
+        int na, nb;
+        local_dims<M>(g, dir, na, nb);
+        const int nk = dir == 0 ? nb : nc1;
+        const int outer = (int)(tl / nk);  // dir 0: strip of faces; dir 1: face row f
+        const int k0 = (int)(tl - (long long)outer * nk);
+        const int kend = (int)min((long long)nk, k0 + (tend - t));
+        t += kend - k0;
+        const R Dt = MeshR<R>::dt(g);
+        const R dt26 = Dt * Dt / (R)6, iht = (R)1 / (R)(dir == 0 ? g.dy : g.dx);
+        const int f = dir == 0 ? outer * FW + x : outer;
+        // this lane's sources of the next row (dir 0) or block of rows (dir 1) of
+        // face states, advanced by `step` values a row or block; its copies stop at
+        // row bb = nb + 1
+        const bool mine = lane < FW * M && f <= na;
+        const long long plane = M * fr_nrow(dir, na, nb) * 4;  // values of a quantity's M line planes
+        const long long step = dir == 0 ? (long long)fr_pitch(na + 1) * 4 : FW * 4;
+        int bs = dir == 0 ? k0 : k0 * FW + x;  // row bb of the next states
+        const R* ps = (const R*)g.FR[dir] + fr_off(fr_nrow(dir, na, nb), M, 0, 0, l, fr_row(dir, na, nb, bs, mine ? f : 0));
+        int slot3 = 0;                          // ring slot of the next states
+        auto load_states = [&]() {
+            if (mine && bs <= nb + 1) {
+                R* dst = sm + L::ring + (l * RING + slot3 * FW + x) * 4;
+#pragma unroll
+                for (int side = 0; side < 2; ++side)
+#pragma unroll
+                    for (int nd = 0; nd < 2; ++nd)
+                        copy_async4(dst + (side * 2 + nd) * M * RING * 4, ps + (side * 3 + nd) * plane);
+            }
+            ps += step;
+            bs += dir == 0 ? 1 : FW;
+            slot3 = slot3 == 2 ? 0 : slot3 + 1;
+        };
+        // and of what only a step's own points read, for step kn: W_nn, and the
+        // face's items dealt to its M lanes: hi of the right cell by variable, TD
+        // by halves, the tangential DFF of its two cells
+        int kn = k0;
+        const int b0 = dir == 0 ? k0 : k0 * FW + x;
+        const R* pn = (const R*)g.FR[dir] + fr_off(fr_nrow(dir, na, nb), M, 0, 2, l, fr_row(dir, na, nb, b0 + 1, mine ? f : 0));
+        long long ci = dir == 0 ? (long long)b0 * g.nx + f : (long long)f * g.nx + b0;
+        long long cidx = cell_idx(dir, na, nb, f, b0);
+        const long long prev = dir == 0 ? 1 : nb + 2;
+        auto load_own = [&]() {
+            const int b = dir == 0 ? kn : kn * FW + x;
+            if (mine && b < nb) {
+                const int slot = kn & 1;
+#pragma unroll
+                for (int side = 0; side < 2; ++side)
+                    copy_async4(sm + L::nn + (((slot * 2 + side) * M + l) * FW + x) * 4, pn + side * 3 * plane);
+                if (BULK32) {
+                    const R* SF = state_planes<R>(g, STAGE == 1 ? 0 : 1);
+                    for (int v = l; v < 4; v += M) {
+                        R* dst = sm + L::hb + (slot * FW + x) * 4 + v;
+                        if (f < na) copy_async1(dst, SF + vglob(dir, v) * g.plane + ci);
+                        else *dst = ghost_average<M, R>(g, SF, dir, v, f, b, STAGE);
+                    }
+                    if (l < 2) copy_async4(sm + L::td + (slot * FW + x) * 8 + l * 4, (const R*)g.TD[dir] + cidx * 8 + l * 4);
+                }
+                if (l == M - 1) {
+                    copy_async1(sm + L::at + (slot * 2 + 0) * FW + x, (const R*)g.AT[dir] + cidx - prev);
+                    copy_async1(sm + L::at + (slot * 2 + 1) * FW + x, (const R*)g.AT[dir] + cidx);
+                }
+            }
+            pn += step;
+            ci += dir == 0 ? g.nx : FW;
+            cidx += dir == 0 ? na + 6 : FW;
+            ++kn;
+        };
+        __syncwarp();  // the last run's reads are done
+        load_states();
+        if (dir == 0) load_states();
+        load_states();
+        load_own();
+        copy_commit();
+        int r0 = 0;  // ring slot of row or block k
+        for (int k = k0; k < kend; ++k) {
+            copy_wait<0>();
+            __syncwarp();
+            const int r1 = r0 == 2 ? 0 : r0 + 1, r2 = r1 == 2 ? 0 : r1 + 1, slot = k & 1;
+            // Step 3: items (side, face, variable)
+#pragma unroll 1
+            for (int it = lane; it < 2 * FW * 4; it += 32) {
+                const int v = it & 3, xi = (it >> 2) % FW, side = (it >> 2) / FW;
+                int q[3];
+                if (dir == 0) {
+                    q[0] = r0 * FW + xi; q[1] = r1 * FW + xi; q[2] = r2 * FW + xi;
+                } else {
+                    q[0] = r0 * FW + xi;
+                    q[1] = xi + 1 < FW ? r0 * FW + xi + 1 : r1 * FW;
+                    q[2] = xi + 2 < FW ? r0 * FW + xi + 2 : r1 * FW + xi + 2 - FW;
+                }
+                R dm = (R)0, dp = (R)0;
+                if (BULK32) {
+                    dm = sm[L::td + (slot * FW + xi) * 8 + v];
+                    dp = sm[L::td + (slot * FW + xi) * 8 + 4 + v];
+                }
+                // scaled by the tangential r5 DFF of the reconstructing cell
+                // (f-1 for the left state, f for the right)
+                const R c1 = sm[L::at + (slot * 2 + side) * FW + xi] * iht;
+                step3<M, R>(sm + L::ring + side * 2 * M * RING * 4 + v, sm + L::ring + (side * 2 + 1) * M * RING * 4 + v, q,
+                            dm, dp, c1, c1 * iht, sm + L::tang + (side * 3 * M * FW + xi) * 4 + v);
+            }
+            __syncwarp();
+            // the next step's copies; ring row k is free now
+            if (k + 1 < kend) {
+                load_states();
+                load_own();
+            }
+            copy_commit();
+            const int b = dir == 0 ? k : k * FW + x;
+            if (mine && b < nb) {
+                StripPoint<M, R> in;
+                in.s = sm;
+                in.slot = slot;
+                in.own_q = dir == 0 ? r1 * FW + x : (x + 1 < FW ? r0 * FW + x + 1 : r1 * FW);
+                in.x = x;
+                in.l = l;
+                flux_point<2, M, R, STAGE, HG, PF>(g, dir, na, nb, f, b, l, in, Dt, dt26);
+            }
+            r0 = r1;
+        }
     }
 }
 
@@ -941,6 +1181,9 @@ __global__ void __launch_bounds__(256) k_update2(Work w)
                 ld4(FX + fo_off(nfx, M, q, l, fxl), bq);
                 ld4(FY + fo_off(nfy, M, q, l, fyl + g.nx), cq);
                 ld4(FY + fo_off(nfy, M, q, l, fyl), dq);
+                // y-faces: local frame (rho, m_y, m_x, E) to global order
+                { const R z = cq[1]; cq[1] = cq[2]; cq[2] = z; }
+                { const R z = dq[1]; dq[1] = dq[2]; dq[2] = z; }
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     R dx_ = a[v] - bq[v];

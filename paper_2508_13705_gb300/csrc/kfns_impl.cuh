@@ -13,6 +13,14 @@ int upload_tables(const CgksTables* t3, const TabF* f3)
 }
 }  // namespace
 
+// The flux instance of a dimension
+template <int D, int M, typename R, int STAGE, int CAP, int HG, bool PF, bool ONE>
+constexpr KOne flux_fn()
+{
+    if constexpr (D == 2) return k_flux2<M, R, STAGE, CAP, HG, PF, ONE>;
+    else return k_flux1<R, STAGE, CAP, HG, PF, ONE>;
+}
+
 template <int D, int M, typename R, bool ONE>
 Kfns make_kfns_one()
 {
@@ -28,30 +36,31 @@ Kfns make_kfns_one()
         k.normal = k_normal1<R, false, ONE>;
         k.normalw = k_normal1<R, true, ONE>;
     }
-    k.flux1v[0] = k_flux<D, M, R, 1, 0, 0, false, ONE>;
-    k.flux2v[0] = k_flux<D, M, R, 2, 0, 0, false, ONE>;
-    k.flux1h[0] = k_flux<D, M, R, 1, 0, 1, false, ONE>;
-    k.flux2h[0] = k_flux<D, M, R, 2, 0, 1, false, ONE>;
+    k.flux1v[0] = flux_fn<D, M, R, 1, 0, 0, false, ONE>();
+    k.flux2v[0] = flux_fn<D, M, R, 2, 0, 0, false, ONE>();
+    k.flux1h[0] = flux_fn<D, M, R, 1, 0, 1, false, ONE>();
+    k.flux2h[0] = flux_fn<D, M, R, 2, 0, 1, false, ONE>();
     // the register-capped variants round exactly like the uncapped ones in
     // FP64 only (the compiler may contract the FP32 arithmetic differently),
     // so the FP32-bulk form offers the autotuner one variant
     if constexpr (sizeof(R) == 8) {
-        k.flux1v[1] = k_flux<D, M, R, 1, 1, 0, false, ONE>;
-        k.flux2v[1] = k_flux<D, M, R, 2, 1, 0, false, ONE>;
-        k.flux1h[1] = k_flux<D, M, R, 1, 1, 1, false, ONE>;
-        k.flux2h[1] = k_flux<D, M, R, 2, 1, 1, false, ONE>;
+        k.flux1v[1] = flux_fn<D, M, R, 1, 1, 0, false, ONE>();
+        k.flux2v[1] = flux_fn<D, M, R, 2, 1, 0, false, ONE>();
+        k.flux1h[1] = flux_fn<D, M, R, 1, 1, 1, false, ONE>();
+        k.flux2h[1] = flux_fn<D, M, R, 2, 1, 1, false, ONE>();
     } else {
         k.flux1v[1] = k.flux1v[0];
         k.flux2v[1] = k.flux2v[0];
         k.flux1h[1] = k.flux1h[0];
         k.flux2h[1] = k.flux2h[0];
     }
-    k.flux1p = k_flux<D, M, R, 1, 0, 1, true, ONE>;
-    k.flux2p = k_flux<D, M, R, 2, 0, 1, true, ONE>;
+    k.flux1p = flux_fn<D, M, R, 1, 0, 1, true, ONE>();
+    k.flux2p = flux_fn<D, M, R, 2, 0, 1, true, ONE>();
     k.flux1 = k.flux1v[0];
     k.flux2 = k.flux2v[0];
-    if (D == 2) { k.upd1 = (KOne)k_update2<M, R, 1, ONE>; k.upd2 = (KOne)k_update2<M, R, 2, ONE>; }
+    if constexpr (D == 2) { k.upd1 = (KOne)k_update2<M, R, 1, ONE>; k.upd2 = (KOne)k_update2<M, R, 2, ONE>; }
     else { k.upd1 = (KOne)k_update1<R, 1, ONE>; k.upd2 = (KOne)k_update1<R, 2, ONE>; }
+    k.flux_warp_bytes = D == 2 ? (int)(FluxShared<(D == 2 ? M : 4), R>::total * sizeof(R)) : 0;
     k.cfl = k_cfl<D, R>;
     k.siginit = k_sigma_init<D>;
     k.check = k_check_state<D>;

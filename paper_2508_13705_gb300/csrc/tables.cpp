@@ -194,5 +194,20 @@ extern "C" __attribute__((visibility("hidden"))) int cgks_build_tables(int order
         for (int l = 0; l < m; ++l) nodes[s * m + l] = (s - 1) + gx[l];
     int deg = 3 * m - 1 < 8 ? 3 * m - 1 : 8;
     for (int l = 0; l < m; ++l) lsq_derivative_weights(nodes, 3 * m, deg, gx[l], t->d1[l], t->d2[l]);
+    for (int l = 0; l < (m + 1) / 2; ++l)
+        for (int q = 0; q < 2; ++q) {
+            const double* d = q == 0 ? t->d1[l] : t->d2[l];
+            double(*sd)[7] = q == 0 ? t->sd1[l] : t->sd2[l];
+            const int n = 3 * m;
+            for (int k = 0; k < n / 2; ++k) {
+                sd[0][k] = (double)((LD)0.5 * ((LD)d[k] + d[n - 1 - k]));
+                sd[1][k] = (double)((LD)0.5 * ((LD)d[k] - d[n - 1 - k]));
+            }
+            if (n % 2) sd[0][n / 2] = d[n / 2];
+            LD lo = 0, hi = 0;
+            for (int k = 0; k < m; ++k) { lo += d[k]; hi += d[2 * m + k]; }
+            sd[0][6] = (double)((LD)0.5 * (lo + hi));
+            sd[1][6] = (double)((LD)0.5 * (lo - hi));
+        }
     return 0;
 }

@@ -14,6 +14,11 @@ struct CgksTables {
     double gx[4], gw[4];
     // Step 3 first / second derivative weights over the 3m face points
     double d1[4][12], d2[4][12];
+    // the same for the line pairs (l, m-1-l), l = 0 .. (m-1)/2, which mirror each
+    // other, on the sums [0] and differences [1] of mirrored points k and 3m-1-k
+    // (an odd rule's middle point stands alone in the sums), k = 0 .. 5; entry 6: on
+    // the sum and difference of what is common to all points of segments b-1, b+1
+    double sd1[2][2][7], sd2[2][2][7];
     int m;
 };
 

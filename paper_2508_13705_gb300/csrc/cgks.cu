@@ -55,6 +55,9 @@ int load_tables()
             f[k].gx[a] = (float)t[k].gx[a];
             f[k].gw[a] = (float)t[k].gw[a];
         }
+        for (int a = 0; a < 3; ++a)
+            for (int b = 0; b < 10; ++b)
+                for (int c = 0; c < 10; ++c) f[k].row2[a][b][c] = make_float2(f[k].row[3 + a][b][c], f[k].row[3 + a][b][c]);
         for (int a = 0; a < 2; ++a)
             for (int b = 0; b < 2; ++b)
                 for (int c = 0; c < 7; ++c) {
@@ -98,11 +101,6 @@ Kfns pick_kfns(int dim, int order, int prec, int tau_mode, const int bc[4], int 
 // flux (2-D: one step of a warp; 1-D: a face), cells, faces.
 enum { W_TILE0 = 0, W_TILE1, W_NORMAL, W_FLUX, W_CELLS, W_SIGINIT, W_COUNT };
 
-// Tile shapes (cells along the normal x across it) the autotuner tries for
-// the 2-D Steps 1-2; the first is the default.
-const int kTileShapes[][2] = {{28, 8}, {60, 4}, {12, 16}, {28, 4}, {12, 8}, {124, 2}};
-const int kNumTileShapes = 6;
-
 } // namespace
 
 struct cgks_batch {
@@ -120,7 +118,6 @@ struct cgks_batch {
     Kfns k;
     int grid[16];
     int threads[16];  // threads per block of each kernel slot (autotuned)
-    int tile[2][2];   // 2-D Steps 1-2: tile shape (TA, TB) per direction (autotuned)
     int nsm = 0;
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // [0] fixed dt, [1] CFL dt
     int kernels_per_step = 0;
@@ -159,11 +156,12 @@ long long tiles(int dir, int nx, int ny, int TA, int TB)
     return ((na + 2 + TA - 1) / TA) * ((nb + 2 + TB - 1) / TB);
 }
 
-long long items(int kind, int dim, int M, int nx, int ny)
+// Work items of a mesh; k: the kernels of its configuration
+long long items(const Kfns& k, int kind, int dim, int M, int nx, int ny)
 {
     switch (kind) {
-    case W_TILE0: return dim == 2 ? tiles(0, nx, ny, kTileShapes[0][0], kTileShapes[0][1]) : 0;
-    case W_TILE1: return dim == 2 ? tiles(1, nx, ny, kTileShapes[0][0], kTileShapes[0][1]) : 0;
+    case W_TILE0: return dim == 2 ? tiles(0, nx, ny, k.recon_tile[0][0], k.recon_tile[0][1]) : 0;
+    case W_TILE1: return dim == 2 ? tiles(1, nx, ny, k.recon_tile[1][0], k.recon_tile[1][1]) : 0;
     case W_NORMAL: return dim == 2 ? 0 : nx + 2;
     case W_FLUX: return dim == 2 ? flux_steps(M, nx, ny) : nx + 1;
     case W_CELLS: return (long long)nx * ny;
@@ -193,50 +191,15 @@ int launch(cgks_batch* b, const void* fn, int kind, int gi, int stage, bool has_
     return CGKS_OK;
 }
 
-// Dynamic shared memory of the 2-D Steps 1-2 for a tile shape.
-size_t recon_smem(const cgks_batch* b, int TA, int TB)
-{
-    return (size_t)(TA + 4) * TB * (4 * b->M + 8) * b->rsize;
-}
-
-// Set the tile shape of direction dir: the per-mesh tile counts of the work
-// list (host and device), the kernel's shared-memory limit and its persistent
-// grid at `threads` threads per block (slot dir).  The limit belongs to the
-// kernel, which every solver of the process shares: it is the largest tile's,
-// always, so that a solver tuned to a small tile leaves the launches of
-// another one, tuned to a large tile, in bounds.
-int set_tile(cgks_batch* b, int dir, int TA, int TB, int threads)
-{
-    const void* fn = (const void*)b->k.recon[dir];
-    size_t smem = recon_smem(b, TA, TB), most = 0;
-    for (int sh = 0; sh < kNumTileShapes; ++sh)
-        most = std::max(most, recon_smem(b, kTileShapes[sh][0], kTileShapes[sh][1]));
-    CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess || occ < 1)
-        return CGKS_ENOTSUP;
-    b->tile[dir][0] = TA;
-    b->tile[dir][1] = TB;
-    b->threads[dir] = threads;
-    b->grid[dir] = occ * b->nsm;
-    const int kind = dir == 0 ? W_TILE0 : W_TILE1;
-    long long* o = b->off.data() + (size_t)kind * (b->n + 1);
-    o[0] = 0;
-    for (int k = 0; k < b->n; ++k) o[k + 1] = o[k] + tiles(dir, b->host[k].nx, b->host[k].ny, TA, TB);
-    CK(cudaMemcpy(b->doff + (size_t)kind * (b->n + 1), o, (b->n + 1) * sizeof(long long), cudaMemcpyHostToDevice));
-    return CGKS_OK;
-}
-
 // One launch of the 2-D Steps 1-2 of direction dir (tiles as work items).
 int launch_recon(cgks_batch* b, int dir, int stage)
 {
     Work w = work_of(b, dir == 0 ? W_TILE0 : W_TILE1);
     if (w.total == 0) return CGKS_OK;
-    int TA = b->tile[dir][0], TB = b->tile[dir][1];
-    int grid = (int)std::max<long long>(1, std::min<long long>(w.total, (long long)b->grid[dir]));
-    void* args[] = {&w, &stage, &TA, &TB};
+    const int grid = (int)w.total;  // a block per tile
+    void* args[] = {&w, &stage};
     CK(cudaLaunchKernel((const void*)b->k.recon[dir], dim3(grid), dim3(b->threads[dir]), args,
-                        recon_smem(b, TA, TB), b->stream));
+                        (size_t)b->k.recon_bytes[dir], b->stream));
     return CGKS_OK;
 }
 
@@ -351,8 +314,8 @@ Layout layout(int dim, int M, size_t rs, int nx, int ny)
         L.FO[d] = o; o = align256(o + (on ? (size_t)nb * (na + 1) * M * 16 * rs : 0));
         L.SP[d] = o; o = align256(o + (on ? (size_t)nb * (na + 1) * M * 8 : 0));
         L.AT[d] = o; o = align256(o + (on && dim == 2 ? (size_t)(nb + 2) * (na + 6) * rs : 0));
-        // FP32 bulk: each cell's tangential differences of hi, for Step 3
-        L.TD[d] = o; o = align256(o + (on && dim == 2 && rs == 4 ? (size_t)(nb + 2) * (na + 6) * 8 * rs : 0));
+        // FP32 bulk: each cell's hi and its tangential differences, for the flux
+        L.TD[d] = o; o = align256(o + (on && dim == 2 && rs == 4 ? (size_t)(nb + 2) * (na + 6) * 12 * rs : 0));
     }
     L.scal = o; o = align256(o + 512);
     L.total = o;
@@ -375,8 +338,7 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
         bool wy = p->dim == 2 && (p->bc[2] >= CGKS_BC_REFLECTIVE || p->bc[3] >= CGKS_BC_REFLECTIVE);
         if ((wx && nx[k] < 3) || (wy && ny[k] < 3)) return CGKS_EINVAL;
         // the kernels index a mesh's work items in 32 bits
-        for (int kind = 0; kind < W_COUNT; ++kind)
-            if (items(kind, p->dim, (p->order - 1) / 2, nx[k], ny[k]) >= (1LL << 31)) return CGKS_EINVAL;
+        if ((p->dim == 2 ? (long long)nx[k] * ny[k] : nx[k] + 2LL) >= (1LL << 31)) return CGKS_EINVAL;
         if (p->dim == 2 && ((long long)(nx[k] + 1) * ny[k] + (long long)(ny[k] + 1) * nx[k]) * ((p->order - 1) / 2) >= (1LL << 31))
             return CGKS_EINVAL;
     }
@@ -471,7 +433,7 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
     b->off.assign((size_t)W_COUNT * (n + 1), 0);
     for (int kind = 0; kind < W_COUNT; ++kind)
         for (int k = 0; k < n; ++k)
-            b->off[(size_t)kind * (n + 1) + k + 1] = b->off[(size_t)kind * (n + 1) + k] + items(kind, p->dim, b->M, nx[k], ny[k]);
+            b->off[(size_t)kind * (n + 1) + k + 1] = b->off[(size_t)kind * (n + 1) + k] + items(b->k, kind, p->dim, b->M, nx[k], ny[k]);
     int rr = CGKS_OK;
     do {
         if (cudaMalloc(&b->dmesh, n * sizeof(Mesh)) != cudaSuccess) { rr = CGKS_ENOMEM; break; }
@@ -482,7 +444,7 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
             std::vector<long long> one((size_t)n * W_COUNT * 2, 0);
             for (int k = 0; k < n; ++k)
                 for (int kind = 0; kind < W_COUNT; ++kind)
-                    one[((size_t)k * W_COUNT + kind) * 2 + 1] = items(kind, p->dim, b->M, nx[k], ny[k]);
+                    one[((size_t)k * W_COUNT + kind) * 2 + 1] = items(b->k, kind, p->dim, b->M, nx[k], ny[k]);
             if (cudaMalloc(&b->doff1, one.size() * sizeof(long long)) != cudaSuccess) { rr = CGKS_ENOMEM; break; }
             if (cudaMemcpy(b->doff1, one.data(), one.size() * sizeof(long long), cudaMemcpyHostToDevice) != cudaSuccess) { rr = CGKS_ECUDA; break; }
         }
@@ -520,10 +482,14 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
             b->grid[q] = std::max(1, occ) * b->nsm;
         }
         if (rr) break;
-        // 2-D Steps 1-2: the default tile shape in both directions
+        // 2-D Steps 1-2: fixed tiles
         if (p->dim == 2)
-            for (int d = 0; d < 2; ++d)
-                if ((rr = set_tile(b, d, kTileShapes[0][0], kTileShapes[0][1], 256))) break;
+            for (int d = 0; d < 2; ++d) {
+                const void* fn = (const void*)b->k.recon[d];
+                b->threads[d] = b->k.recon_threads[d];
+                if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, b->k.recon_bytes[d]) != cudaSuccess)
+                    rr = CGKS_ECUDA;
+            }
     } while (0);
     if (rr) { cgks_batch_destroy(b); return rr; }
     *out = b;
@@ -590,7 +556,7 @@ int launch_one(cgks_batch* b, int k, const void* fn, int kind, int arg, bool has
     w.m0 = b->host[k];
     w.off = b->doff1 + ((size_t)k * W_COUNT + kind) * 2;
     w.n = 1;
-    w.total = items(kind, b->dim, b->M, b->host[k].nx, b->host[k].ny);
+    w.total = items(b->k, kind, b->dim, b->M, b->host[k].nx, b->host[k].ny);
     if (w.total == 0) return CGKS_OK;
     int threads = 256;
     long long need = (w.total + threads - 1) / threads;
@@ -654,7 +620,7 @@ int autotune(cgks_batch* b, int* out)
     if (!b->state_set) return CGKS_EINVAL;
     // tuning order: each kernel runs after the producers of its inputs (the
     // stage-2 flux last: it reads the stage-1 state W* that the update writes);
-    // the 2-D Steps 1-2 are tuned first, over tile shapes and block sizes
+    // the 2-D Steps 1-2 have one shape
     const void* fns[4] = {b->dim == 1 ? (const void*)b->k.normal : nullptr, (const void*)b->k.flux1,
                           (const void*)b->k.upd1, (const void*)b->k.flux2};
     const int slots[4] = {1, 2, 4, 3};
@@ -686,28 +652,9 @@ int autotune(cgks_batch* b, int* out)
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    for (int dir = 0; dir < (b->dim == 2 ? 2 : 0); ++dir) {
-        float best = 1e30f;
-        int bt = b->tile[dir][0], bb = b->tile[dir][1], bth = b->threads[dir];
-        const int thr[2] = {128, 256};
-        for (int sh = 0; sh < kNumTileShapes; ++sh)
-            for (int c = 0; c < 2; ++c) {
-                int TA = kTileShapes[sh][0], TB = kTileShapes[sh][1];
-                if (set_tile(b, dir, TA, TB, thr[c]) != CGKS_OK) continue;  // no room on an SM
-                float acc = 0.f;
-                for (int rep = 0; rep < 4; ++rep) {
-                    CK(cudaEventRecord(e0, b->stream));
-                    if ((r = launch_recon(b, dir, 1))) return r;
-                    CK(cudaEventRecord(e1, b->stream));
-                    CK(cudaEventSynchronize(e1));
-                    float ms = 0.f;
-                    CK(cudaEventElapsedTime(&ms, e0, e1));
-                    if (rep > 0) acc += ms;  // the first launch warms caches
-                }
-                if (acc < best) { best = acc; bt = TA; bb = TB; bth = thr[c]; }
-            }
-        if ((r = set_tile(b, dir, bt, bb, bth))) return r;
-    }
+    // the 2-D Steps 1-2 have one shape: run them for the flux's inputs
+    for (int dir = 0; dir < (b->dim == 2 ? 2 : 0); ++dir)
+        if ((r = launch_recon(b, dir, 1))) return r;
     for (int qq = 0; qq < 4; ++qq) {
         if (!fns[qq]) continue;
         int q = slots[qq];
@@ -768,7 +715,7 @@ int autotune(cgks_batch* b, int* out)
         if (b->k.flux1v[1] != b->k.flux1v[0] && b->k.flux1 == b->k.flux1v[1]) out[2] = -out[2];
         if (b->k.flux2v[1] != b->k.flux2v[0] && b->k.flux2 == b->k.flux2v[1]) out[3] = -out[3];
         for (int d = 0; d < 2; ++d)
-            for (int e = 0; e < 2; ++e) out[6 + 2 * d + e] = b->dim == 2 ? b->tile[d][e] : 0;
+            for (int e = 0; e < 2; ++e) out[6 + 2 * d + e] = b->dim == 2 ? b->k.recon_tile[d][e] : 0;
     }
     return CGKS_OK;
 }
@@ -1268,7 +1215,7 @@ extern "C" int cgks_step_1d_noalloc(const cgks_params* p, int nx, double x0, dou
     std::memset(&init, 0, sizeof(init));
     init.g = g;
     const long long* off = init.off;
-    for (int kind = 0; kind < W_COUNT; ++kind) { init.off[2 * kind] = 0; init.off[2 * kind + 1] = items(kind, 1, 1, nx, 1); }
+    for (int kind = 0; kind < W_COUNT; ++kind) { init.off[2 * kind] = 0; init.off[2 * kind + 1] = items(Kfns(), kind, 1, 1, nx, 1); }
     init.dt = dt;
     Mesh* dmesh = (Mesh*)(base + oM);
     long long* doff = (long long*)(base + oOF);

@@ -1,22 +1,22 @@
 // Device code of the ASE-DFF compact gas-kinetic scheme (sm_103a).
 //
-// One stage of the S2O4 step (Sec. 2.2) runs as four kernels, each a
-// grid-stride ("persistent") loop over the work items of every mesh in a
-// descriptor table (one mesh, or a batch of uneven meshes):
+// One stage of the S2O4 step (Sec. 2.2) runs as four kernels over the work
+// items of every mesh in a descriptor table (one mesh, or a batch of uneven
+// meshes):
 //
-//   k_lines   Sec. 3.3 Step 1: tangential ASE-DFF reconstruction of every cell
-//             (plus a ghost halo), evaluated at the m Gauss lines of the
-//             faces normal to x and to y -> line averages.
-//   k_normal  Sec. 3.3 Step 2: normal ASE-DFF reconstruction of every
-//             (cell, Gauss line) from line averages and line-averaged slopes
-//             -> W, W_n, W_nn at the cell's two faces (Algorithm 1).
-//   k_flux    Sec. 3.3 Step 3 (tangential W_t, W_tt, W_nt from the face values
+//   k_recon   (one launch per direction) Sec. 3.3 Step 1: tangential ASE-DFF
+//             reconstruction of every cell (plus a ghost halo), evaluated at the
+//             m Gauss lines of the faces -> line averages; Step 2: normal
+//             ASE-DFF reconstruction of every (cell, Gauss line) from line
+//             averages and line-averaged slopes -> W, W_n, W_nn at the cell's
+//             two faces (Algorithm 1).  1-D: k_normal1, Step 2 alone.
+//   k_flux1/2 Sec. 3.3 Step 3 (tangential W_t, W_tt, W_nt from the face values
 //             of three face segments), Eq. 3.2 (sigma), Step 4 (kinetic
 //             weighting, Eq. 2.7-2.8) and the time-integrated flux and
 //             interface state of Eq. 2.6, 2.11, 2.12, 2.15 with the linear /
 //             quadratic fits of Eq. 2.19-2.20 and 2.29 done analytically per
 //             term; emits the per-point quantities the update needs.
-//   k_update  Eq. 2.21-2.25, 2.30 and the Gauss-theorem slope update of
+//   k_update1/2  Eq. 2.21-2.25, 2.30 and the Gauss-theorem slope update of
 //             Sec. 3.3: cell averages, cell slopes and line slopes; the FP64
 //             accumulator makes stage 2 need no stage-1 face data; face
 //             sigma (Eq. 3.1) for the next step.
@@ -45,6 +45,7 @@ struct TabF {
     float bm4[5][5];
     float gx[4], gw[4];
     float sd1[2][2][7], sd2[2][2][7];
+    float2 row2[3][10][10];  // rows of r5, r7, r9, each coefficient twice, for two-wide FMAs
 };
 
 static __constant__ CgksTables c_tab[3];  // orders 5, 7, 9 (one copy per translation unit)
@@ -90,8 +91,8 @@ struct Mesh {
     const double* ghost;            // 1-D fixed BC ghost cells
     void *FR[2], *FO[2];            // scratch per direction (R typed)
     void* AT[2];                    // tangential r5 DFF per cell (R typed)
-    void* TD[2];                    // FP32 bulk: hi(a, b-1) - hi(a, b), hi(a, b+1) - hi(a, b)
-                                    // of each cell, local frame, [8] floats
+    void* TD[2];                    // FP32 bulk: hi(a, b), hi(a, b-1) - hi(a, b), hi(a, b+1) - hi(a, b)
+                                    // of each cell, local frame, [12] floats
     double* SP[2];                  // sigma per face Gauss point
     double* dt;                     // device scalar (this mesh's step)
     float* dtf;                     // the same in FP32: [0] float(dt), [1] float(dt - [0])
@@ -222,74 +223,102 @@ template <typename T> __device__ __forceinline__ T prescribed(double x, int kind
     return kind == 0 ? (T)x : (kind == 5 ? low_part<T>(x) : (T)0);
 }
 
-// kind: 0 W, 1 Wx, 2 Wy, 3 Wx_line, 4 Wy_line (global orientation), 5 the low
-// part of W (FP32-bulk float planes only); tb: the
-// stage's time, read by inflow sides only.  Ghost rules apply x first, then y.
-// WALLS = false compiles the wall and inflow branches out: the stencil kernels
-// have an instance for meshes without them, whose hot loops the (never
-// taken) code would otherwise slow down.
-template <int D, int M, typename T, bool WALLS = true>
-__device__ __forceinline__ T cell(const Mesh& g, const T* S, int kind, int v, int l, int i, int j, double tb)
+// Where the data of cell (i, j) come from.  Ghost rules apply x first, then y: a
+// prescribed state, or cell idx with slopes along x / y zeroed and with the
+// mirror images at walls normal to x / y (the wall's boundary code, or 0).
+struct CellMap {
+    long long idx;
+    int zx, zy, wx, wy;
+    const double* state;  // prescribed state (inflow), or null
+};
+
+// tb: the stage's time, read by inflow sides only.  WALLS = false compiles the
+// wall and inflow branches out: the stencil kernels have an instance for meshes
+// without them.
+template <bool WALLS>
+__device__ __forceinline__ CellMap cell_map(const Mesh& g, int i, int j, double tb, bool two = true)
 {
-    bool zero = false, neg = false;
+    CellMap c = {0, 0, 0, 0, 0, nullptr};
     if (i < 0 || i >= g.nx) {
-        int side = i < 0 ? 0 : 1;
-        int bc = g.bc[side];
+        const int side = i < 0 ? 0 : 1, bc = g.bc[side];
         if (bc == BC_PERIODIC) {
             i = imod(i, g.nx);
-        } else if (bc == BC_FIXED) {
-            int layer = side == 0 ? (-1 - i) : (i - g.nx);
-            double gv = g.ghost[((side * 3 + layer) * 2 + (kind == 0 || kind == 5 ? 0 : 1)) * 3 + v];
-            return kind == 5 ? low_part<T>(gv) : (T)gv;
         } else if (WALLS && (bc == BC_INFLOW || (bc == BC_INFLOW_REFLECTIVE && below_split(g, side, j, tb)))) {
-            // prescribed state by the row's centre, zero slopes
-            return prescribed<T>(g.bcs[side][below_split(g, side, j, tb) ? 0 : 1][v], kind);
+            // by the row's centre
+            c.state = g.bcs[side][below_split(g, side, j, tb) ? 0 : 1];
+            return c;
         } else if (WALLS && is_mirror(bc)) {
-            // ghost cell -1-k mirrors cell k; lines across x (Wy_line) swap ends
+            // ghost cell -1-k mirrors cell k
             i = i < 0 ? -1 - i : 2 * g.nx - 1 - i;
-            neg = wall_flip<D>(kind, v, 0, bc);
-            if (kind == 4) l = M - 1 - l;
+            c.wx = bc;
         } else {
             i = i < 0 ? 0 : g.nx - 1;
-            zero = (kind == 1 || kind == 3);
+            c.zx = 1;
         }
     }
-    if (D == 2 && (j < 0 || j >= g.ny)) {
-        int side = j < 0 ? 2 : 3;
-        int bc = g.bc[side];
+    if (two && (j < 0 || j >= g.ny)) {
+        const int side = j < 0 ? 2 : 3, bc = g.bc[side];
         if (WALLS && (bc == BC_INFLOW || (bc == BC_INFLOW_REFLECTIVE && below_split(g, side, i, tb)))) {
-            // prescribed state by the column's centre (after the x rule), zero slopes
-            T val = prescribed<T>(g.bcs[side][below_split(g, side, i, tb) ? 0 : 1][v], kind);
-            return neg ? -val : val;
+            // by the column's centre (after the x rule)
+            c.state = g.bcs[side][below_split(g, side, i, tb) ? 0 : 1];
+            return c;
         }
         if (bc == BC_PERIODIC) {
             j = imod(j, g.ny);
         } else if (WALLS && is_mirror(bc)) {
             j = j < 0 ? -1 - j : 2 * g.ny - 1 - j;
-            neg = neg != wall_flip<D>(kind, v, 1, bc);
-            if (kind == 3) l = M - 1 - l;
+            c.wy = bc;
         } else {
             j = j < 0 ? 0 : g.ny - 1;
-            zero = zero || (kind == 2 || kind == 4);
+            c.zy = 1;
         }
     }
-    if (zero) return (T)0;
-    long long idx = (long long)j * g.nx + i;
-    int p;
-    if (D == 1) {
-        p = kind == 0 ? v : (kind == 5 ? 6 + v : 3 + v);
-    } else {
-        switch (kind) {
-        case 0: p = v; break;
-        case 1: p = 4 + v; break;
-        case 2: p = 8 + v; break;
-        case 3: p = 12 + 4 * l + v; break;
-        case 5: p = 12 + 8 * M + v; break;
-        default: p = 12 + 4 * M + 4 * l + v; break;
-        }
+    c.idx = (long long)j * g.nx + i;
+    return c;
+}
+
+// The plane of a value.  kind: 0 W, 1 Wx, 2 Wy, 3 Wx_line, 4 Wy_line (global
+// orientation), 5 the low part of W (FP32-bulk float planes only).
+template <int D, int M>
+__device__ __forceinline__ int value_plane(int kind, int v, int l)
+{
+    if (D == 1) return kind == 0 ? v : (kind == 5 ? 6 + v : 3 + v);
+    switch (kind) {
+    case 0: return v;
+    case 1: return 4 + v;
+    case 2: return 8 + v;
+    case 3: return 12 + 4 * l + v;
+    case 5: return 12 + 8 * M + v;
+    default: return 12 + 4 * M + 4 * l + v;
     }
-    T val = S[p * g.plane + idx];
-    return neg ? -val : val;
+}
+
+// One value of a mapped cell
+template <int D, int M, typename T, bool WALLS>
+__device__ __forceinline__ T mapped(const Mesh& g, const T* S, const CellMap& c, int kind, int v, int l)
+{
+    const bool nx = WALLS && c.wx && wall_flip<D>(kind, v, 0, c.wx), ny = WALLS && c.wy && wall_flip<D>(kind, v, 1, c.wy);
+    if (WALLS && c.state) {
+        const T val = prescribed<T>(c.state[v], kind);  // zero slopes
+        return nx ? -val : val;
+    }
+    if ((c.zx && (kind == 1 || kind == 3)) || (c.zy && (kind == 2 || kind == 4))) return (T)0;
+    // lines across a mirrored side swap ends
+    if (WALLS && ((c.wx && kind == 4) != (c.wy && kind == 3))) l = M - 1 - l;
+    const T val = S[value_plane<D, M>(kind, v, l) * g.plane + c.idx];
+    return nx != ny ? -val : val;
+}
+
+// One value of cell (i, j), ghost rules applied
+template <int D, int M, typename T, bool WALLS = true>
+__device__ __forceinline__ T cell(const Mesh& g, const T* S, int kind, int v, int l, int i, int j, double tb)
+{
+    if (D == 1 && (i < 0 || i >= g.nx) && g.bc[i < 0 ? 0 : 1] == BC_FIXED) {
+        const int side = i < 0 ? 0 : 1, layer = side == 0 ? (-1 - i) : (i - g.nx);
+        const double gv = g.ghost[((side * 3 + layer) * 2 + (kind == 0 || kind == 5 ? 0 : 1)) * 3 + v];
+        return kind == 5 ? low_part<T>(gv) : (T)gv;
+    }
+    return mapped<D, M, T, WALLS>(g, S, cell_map<WALLS>(g, i, j, tb, D == 2), kind, v, l);
 }
 
 // sigma of x-face f (between cells f-1 and f) in row j; ghost faces: periodic
@@ -506,24 +535,20 @@ __device__ __forceinline__ DffR<R> dff_r(const Dff& d)
     return r;
 }
 
-// Packed form for a per-cell buffer: (a0, a1, a3, stencil code)
-template <typename R>
-__device__ __forceinline__ void dff_pack(const DffR<R>& d, R out[4])
+// The taps of dp that sub-stencil k of HWENO-AO uses (S0, S1, S2, r5; the own
+// average enters through the differences only)
+__host__ __device__ constexpr bool ao_tap(int k, int q)
 {
-    out[0] = d.a[0]; out[1] = d.a[1]; out[2] = d.a[3]; out[3] = (R)d.st;
-}
-template <typename R>
-__device__ __forceinline__ DffR<R> dff_unpack(const R in[4])
-{
-    DffR<R> d;
-    d.a[0] = in[0]; d.a[1] = in[1]; d.a[2] = d.a[3] = in[2];
-    d.st = (int)in[3];
-    return d;
+    return k == 0 ? (q == 1 || q == 6)
+         : k == 1 ? (q == 3 || q == 8)
+         : k == 2 ? (q == 1 || q == 3)
+         : (q == 1 || q == 3 || q == 6 || q == 8);
 }
 
 // HWENO-AO(5,3) with DFF-scaled sub-polynomials (Eq. 3.11-3.17, 3.19) for
 // NOUT consecutive functional rows starting at row0.  Kept out of line: the
 // branch is rare, and inlining it in every variable's loop bloats the kernels.
+// Only the taps a sub-stencil has are summed (10 of 40 a row).
 template <typename R, int NOUT>
 __device__ __noinline__ void recon_ao(const R* al, int oi, int row0, const R* dp, R* out, R ghi, R glo, R eps)
 {
@@ -531,12 +556,16 @@ __device__ __noinline__ void recon_ao(const R* al, int oi, int row0, const R* dp
     R beta[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
+        constexpr int kDeg[4] = {3, 3, 3, 5};
         R c[5];
 #pragma unroll
-        for (int n = 0; n < 5; ++n) {
+        for (int n = 1; n < 5; ++n) {
             R s = 0;
+            if (n < kDeg[k]) {
 #pragma unroll
-            for (int q = 0; q < 10; ++q) s += T.cpoly[k][n][q] * dp[q];
+                for (int q = 0; q < 10; ++q)
+                    if (ao_tap(k, q)) s += T.cpoly[k][n][q] * dp[q];
+            }
             c[n] = s;
         }
         R b = 0;
@@ -565,9 +594,10 @@ __device__ __noinline__ void recon_ao(const R* al, int oi, int row0, const R* dp
     }
     R inv = (R)1 / ws;
     R c3 = w[3] * inv / g3;
-    R ck[3];
+    R ck[4];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) ck[k] = w[k] * inv - w[3] * inv * gk[k] / g3;
+    for (int k = 0; k < 3; ++k) ck[k] = (w[k] * inv - w[3] * inv * gk[k] / g3) * al[k];
+    ck[3] = c3 * al[3];
 #pragma unroll
     for (int r = 0; r < NOUT; ++r) {
         R s = 0;
@@ -575,8 +605,9 @@ __device__ __noinline__ void recon_ao(const R* al, int oi, int row0, const R* dp
         for (int k = 0; k < 4; ++k) {
             R p = 0;
 #pragma unroll
-            for (int q = 0; q < 10; ++q) p += T.row[k][row0 + r][q] * dp[q];
-            s += (k == 3 ? c3 : ck[k]) * al[k] * p;
+            for (int q = 0; q < 10; ++q)
+                if (ao_tap(k, q)) p += T.row[k][row0 + r][q] * dp[q];
+            s += ck[k] * p;
         }
         out[r] = s;
     }
@@ -613,52 +644,69 @@ __host__ __device__ constexpr bool st_tap(int st, int k)
 {
     return st == ST_R9 ? (k != 2 && k != 7)
          : st == ST_R7 ? (k == 0 || k == 1 || k == 3 || k == 4 || k == 6 || k == 8)
-         : st == ST_R5 ? (k == 1 || k == 3 || k == 6 || k == 8)
-         : true;
+         : (k == 1 || k == 3 || k == 6 || k == 8);
 }
 
-// A linear stencil with the order (table index OI), the stencil and the first
-// output row fixed at compile time, for the 2-D kernels, whose instantiation
-// fixes the order: the stencil row comes from a constant address, so the
-// coefficients enter the FMAs as constant-bank operands instead of loads.
-template <typename R, int NOUT, int OI, int ST, int ROW0>
-__device__ __forceinline__ void recon_lin(const R dp[10], R out[NOUT])
+// FP32: a linear stencil's functional rows tap by tap, on two data sets at once
+// (two lines, or two variables) with two-wide FMAs; Steps 1-2 are bound by issue
+// slots.  The order (table OI), the stencil and the row are fixed at compile time.
+template <int OI, int ST, int ROW>
+__device__ __forceinline__ float2 row_taps(const float2 dp[10])
 {
-    const auto& T = Tab<R>::get(OI);
+    const auto& c = c_tabf[OI].row2[ST - ST_R5][ROW];
+    float2 r = __fmul2_rn(c[1], dp[1]);
 #pragma unroll
-    for (int r = 0; r < NOUT; ++r) {
-        R s = 0;
+    for (int k = 0; k < 10; ++k)
+        if (k != 1 && st_tap(ST, k)) r = __ffma2_rn(c[k], dp[k], r);
+    return r;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float a, float2 b) { return __fmul2_rn(make_float2(a, a), b); }
+
+// FP64: the rows in mirrored pairs: on the sums e and differences o of the averages
+// of cells i+j and i-j (relative to cell i's) and the sums E and differences O
+// of their slopes, j = 1, 2, a functional at place xi is even + odd with even =
+// c0 e1 + c1 e2 + c2 O1 + c3 O2 and odd = c4 o1 + c5 o2 + c6 E1 + c7 E2, and the
+// same functional at -xi is +-(even - odd): half the multiplications of both.
+// The FP64 pipe bounds its Steps 1-2 (0.73 -> 0.57 ms per direction at 512^2,
+// order 9); FP32 keeps the taps, whose rounding is a third smaller (order 9
+// density wave on 20^2 to t = 2: 1.35e-8 against 1.99e-8).
+template <int ST, typename R>
+__device__ __forceinline__ void sym_row(const R c[8], const R e[2], const R o[2], const R E[2], const R O[2], R& even,
+                                        R& odd)
+{
+    constexpr bool a2 = ST != ST_R5, s2 = ST == ST_R9;
+    even = c[0] * e[0] + c[2] * O[0];
+    odd = c[4] * o[0] + c[6] * E[0];
+    if (a2) { even += c[1] * e[1]; odd += c[5] * o[1]; }
+    if (s2) { even += c[3] * O[1]; odd += c[7] * E[1]; }
+}
+
+template <typename R>
+__device__ __forceinline__ void sym_data(const R dp[10], R e[2], R o[2], R E[2], R O[2])
+{
 #pragma unroll
-        for (int k = 0; k < 10; ++k)
-            if (st_tap(ST, k)) s += T.row[ST][ROW0 + r][k] * dp[k];
-        out[r] = s;
+    for (int j = 0; j < 2; ++j) {
+        e[j] = dp[3 + j] + dp[1 - j];
+        o[j] = dp[3 + j] - dp[1 - j];
+        E[j] = dp[8 + j] + dp[6 - j];
+        O[j] = dp[8 + j] - dp[6 - j];
     }
 }
 
-// Compile-time stencil tag (-1: HWENO-AO) for branch-hoisted reconstruction
-// loops: the branch on a cell's stencil is taken once, outside the loop over
-// variables, so each branch is one straight run of code.
+// Calls body(StTag<st>()) for a stencil code (-1: HWENO-AO); the order bounds
+// the linear stencils that occur.  The branch is taken once, outside the loop
+// over lines or variables, so that each branch is one straight run of code.
 template <int V> struct StTag { static constexpr int value = V; };
-
-// Reconstruction with the stencil fixed at compile time (ST = -1: HWENO-AO).
-template <typename R, int NOUT, int OI, int ST, int ROW0>
-__device__ __forceinline__ void recon_st(const DffR<R>& dff, const R dp[10], R out[NOUT], R ghi, R glo, R eps)
+template <int M, typename Body>
+__device__ __forceinline__ void with_stencil(int st, Body&& body)
 {
-    if constexpr (ST >= 0) recon_lin<R, NOUT, OI, ST, ROW0>(dp, out);
-    else recon_ao<R, NOUT>(dff.a, OI, ROW0, dp, out, ghi, glo, eps);
-}
-
-// Calls body(StTag<st>()) for the stencil of dff; the order (table index OI)
-// bounds the linear stencils that can occur.
-template <int OI, typename R, typename Body>
-__device__ __forceinline__ void with_stencil(const DffR<R>& dff, Body&& body)
-{
-    if (OI == 2 && dff.st == ST_R9) body(StTag<(OI == 2 ? ST_R9 : ST_R5)>());
-    else if (OI >= 1 && dff.st == ST_R7) body(StTag<(OI >= 1 ? ST_R7 : ST_R5)>());
-    else if (dff.st == ST_R5) body(StTag<ST_R5>());
+    if (M == 4 && st == ST_R9) body(StTag<(M == 4 ? ST_R9 : ST_R5)>());
+    else if (M >= 3 && st == ST_R7) body(StTag<(M >= 3 ? ST_R7 : ST_R5)>());
+    else if (st == ST_R5) body(StTag<ST_R5>());
     else body(StTag<-1>());
 }
-
 
 // ------------------------------------------------------------------ kinetics
 //

@@ -18,9 +18,10 @@
 //                                     one plane per output quantity and line
 //   SP  [nb][na+1][M]                 sigma per face Gauss point (Eq. 3.2)
 //   AT  [nb+2][na+6]                  tangential r5 DFF of each cell (Step 3)
-//   TD  [nb+2][na+6][8]               FP32 bulk: the cell's tangential differences of hi,
-//                                     hi(a, b-1) - hi(a, b) and hi(a, b+1) - hi(a, b), for
-//                                     the bases of the Step 3 segments
+//   TD  [nb+2][na+6][12]              FP32 bulk: the cell's hi (the base of the face
+//                                     states) and its tangential differences hi(a, b-1) -
+//                                     hi(a, b), hi(a, b+1) - hi(a, b), for the bases of the
+//                                     Step 3 segments
 //
 // FP32-bulk form: a cell average W (FP64) is held in the float planes as
 // hi = float(W) and lo = float(W - hi), and every reconstructed quantity that
@@ -61,13 +62,6 @@ __device__ __forceinline__ T lcell(const Mesh& g, const T* S, int dir, int lkind
     else kind = dir == 0 ? 3 : 4;
     int i = dir == 0 ? a : b, j = dir == 0 ? b : a;
     return cell<D, M, T, WALLS>(g, S, kind, vglob(dir, v), l, i, j, tb);
-}
-
-// W of a ghost cell, out of line: the flux kernel reads few of them
-template <int M, typename R>
-__device__ __noinline__ R ghost_average(const Mesh& g, const R* S, int dir, int v, int a, int b, int stage)
-{
-    return lcell<2, M, R, true>(g, S, dir, 0, v, 0, a, b, stage_time(g, stage));
 }
 
 // sigma of normal faces (f, b) and of tangential faces of column a (a, f)
@@ -126,262 +120,438 @@ __device__ __forceinline__ void flag_bad(const Mesh& g, long long idx)
     atomicMin((unsigned long long*)g.bad, (unsigned long long)idx);
 }
 
-// -------------------------------------------------------------- Steps 1-2 (2-D)
-// Step 1 of one cell (a, b) of direction dir: the tangential ASE-DFF
-// reconstruction from the five cells b-2..b+2, evaluated at the M Gauss lines
-// -> res (line averages; FP32 bulk: lo + the increment over the cell's hi);
-// hi: the cell's average (FP32 bulk: its high part).  For the cells whose
-// faces this stage evaluates (core), also the tangential r5 DFF (AT, Step 3),
-// the tangential differences of hi (TD, FP32 bulk) and the packed DFF of the
-// normal stencil (dn, Step 2).
-template <int M, typename R, bool WALLS>
-__device__ __forceinline__ void step1_cell(const Mesh& g, const R* S, int dir, int na, int nb, int a, int b, double tb,
-                                           const double* SX, const double* SY, bool core, R res[M][4], R hi[4],
-                                           R dn[4])
+// Asynchronous copies from global to shared memory: one value, 4 values
+__device__ __forceinline__ void copy_async16(void* dst, const void* src)
 {
-    constexpr bool BULK32 = sizeof(R) == 4;
-    // the tangential stencil: a direct walk for interior cells, whose loads
-    // are issued before the DFF selections so that their latencies overlap
-    bool inner = a >= 0 && a < na && b >= 2 && b + 2 < nb;
-    long long P = g.plane;
-    long long ci = dir == 0 ? (long long)b * g.nx + a : (long long)a * g.nx + b;
-    long long st = dir == 0 ? g.nx : 1;  // tangential neighbour stride
-    int pt = dir == 0 ? 8 : 4;           // plane of the tangential cell slope
-    R sw[4][5], swt[4][5], slo[4][BULK32 ? 5 : 1];  // slo: low parts of the averages (FP32 bulk)
-    if (inner) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            int gv = vglob(dir, v);
-            const R* w0 = S + gv * P + ci;
-            const R* wt = S + (pt + gv) * P + ci;
-            const R* wl = S + (12 + 8 * M + gv) * P + ci;
-#pragma unroll
-            for (int q = 0; q < 5; ++q) {
-                sw[v][q] = w0[(q - 2) * st];
-                swt[v][q] = wt[(q - 2) * st];
-                if (BULK32) slo[v][BULK32 ? q : 0] = wl[(q - 2) * st];
-            }
-        }
-    } else {
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-#pragma unroll
-            for (int q = 0; q < 5; ++q) {
-                sw[v][q] = lcell<2, M, R, WALLS>(g, S, dir, 0, v, 0, a, b + q - 2, tb);
-                swt[v][q] = lcell<2, M, R, WALLS>(g, S, dir, 2, v, 0, a, b + q - 2, tb);
-                if (BULK32) slo[v][BULK32 ? q : 0] = lcell<2, M, R, WALLS>(g, S, dir, 5, v, 0, a, b + q - 2, tb);
-            }
-    }
-    // face sigma of the tangential stencil: a direct walk for interior cells
-    double s6[6];
-    if (inner) {
-        const double* sp = dir == 0 ? SY + (long long)(b - 2) * g.nx + a : SX + (long long)a * (g.nx + 1) + (b - 2);
-        const long long ss = dir == 0 ? g.nx : 1;
-#pragma unroll
-        for (int q = 0; q < 6; ++q) s6[q] = sp[q * ss];
-    } else {
-#pragma unroll
-        for (int q = 0; q < 6; ++q) s6[q] = lsigT<WALLS>(g, SX, SY, dir, a, b - 2 + q);
-    }
-    DffR<R> dff = dff_r<R>(dff_select(g.order, s6, g.thr));
-    R ht = (R)(dir == 0 ? g.dy : g.dx);
-    if (core) {
-        long long cidx = cell_idx(dir, na, nb, a, b);
-        // tangential r5 DFF of this cell, reused by Step 3 in k_flux
-        ((R*)g.AT[dir])[cidx] = (R)dff.a[3];
-        if (BULK32) {
-            // the tangential differences of hi, for the bases of Step 3's segments
-            R tdm[4], tdp[4];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) { tdm[v] = sw[v][1] - sw[v][2]; tdp[v] = sw[v][3] - sw[v][2]; }
-            st4((R*)g.TD[dir] + cidx * 8, tdm);
-            st4((R*)g.TD[dir] + cidx * 8 + 4, tdp);
-        }
-        // the DFF of the normal stencil, used by every Gauss line in Step 2
-        double n6[6];
-        if (a >= 2 && a + 3 <= na && b >= 0 && b < nb) {
-            const double* sp = dir == 0 ? SX + (long long)b * (g.nx + 1) + (a - 2) : SY + (long long)(a - 2) * g.nx + b;
-            const long long ss = dir == 0 ? 1 : g.nx;
-#pragma unroll
-            for (int q = 0; q < 6; ++q) n6[q] = sp[q * ss];
-        } else {
-#pragma unroll
-            for (int q = 0; q < 6; ++q) n6[q] = lsigN<2, WALLS>(g, SX, SY, dir, a - 2 + q, b);
-        }
-        dff_pack<R>(dff_r<R>(dff_select(g.order, n6, g.thr)), dn);
-    }
-#pragma unroll
-    for (int v = 0; v < 4; ++v) hi[v] = sw[v][2];
-    const R ghi = (R)g.ghi, glo = (R)g.glo, eps = (R)g.eps;
-    with_stencil<M - 2>(dff, [&](auto tag) {
-        constexpr int ST = decltype(tag)::value;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            // FP32 bulk: differences of averages as (hi - hi) + (lo - lo), and
-            // the line average kept as lo + increment (over the cell's hi)
-            R qi = sw[v][2], dp[10];
-#pragma unroll
-            for (int q = 0; q < 5; ++q) {
-                dp[q] = BULK32 ? (sw[v][q] - qi) + (slo[v][BULK32 ? q : 0] - slo[v][BULK32 ? 2 : 0]) : sw[v][q] - qi;
-                dp[5 + q] = ht * swt[v][q];
-            }
-            R out[M];
-            recon_st<R, M, M - 2, ST, 6>(dff, dp, out, ghi, glo, eps);
-            const R base = BULK32 ? slo[v][BULK32 ? 2 : 0] : qi;
-#pragma unroll
-            for (int l = 0; l < M; ++l) res[l][v] = base + out[l];
-        }
-    });
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+template <typename R>
+__device__ __forceinline__ void copy_async1(R* dst, const R* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"(sizeof(R))
+                 : "memory");
+}
+__device__ __forceinline__ void copy_async4(float* dst, const float* src) { copy_async16(dst, src); }
+__device__ __forceinline__ void copy_async4(double* dst, const double* src)
+{
+    copy_async16(dst, src);
+    copy_async16(dst + 2, src + 2);
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// -------------------------------------------------------------- Steps 1-2 (2-D)
+//
+// One launch per direction over tiles of TA x TB cells (a along the face
+// normal, b across it) of the range a in [-1, na], b in [-1, nb] whose faces
+// the stage evaluates (ghost columns and rows included: Step 3 reads the face
+// states of the rows beside the mesh).  A tile goes through shared memory in
+// four parts:
+//   stage  asynchronous copies of what the tile reads: averages (FP32 bulk: hi
+//          and lo) and tangential slopes of the tile and two halo layers each
+//          way, line slopes of the tile and its halo along a, and the face sigma;
+//          ghost values are resolved here, once each;
+//   0      per cell: the DFFs of the tangential and the normal stencil;
+//   1      Step 1 per cell, a variable at a time: the tangential reconstruction at the M
+//          Gauss lines -> line averages; for the cells whose faces this tile
+//          evaluates also AT and TD (Step 3);
+//   2      Step 2 (Algorithm 1) per (cell, variable), all M lines: both face
+//          states with their derivatives.
+// A lane per (cell, variable) needs a quarter of the registers of a lane per
+// cell and line, so that more warps hide each other's latencies, and the M lines
+// share the cell's differences of averages; 8 cells x 4 variables a warp write
+// whole 128-byte groups of FR.  The tile shape is fixed at compile time (index
+// arithmetic was a third of the instructions): along x 32 cells with the halo
+// (28 + 4 in direction 0, 12 + 4 by 16 in direction 1), and a block's cells fill
+// its threads.
+//
+// Before, a lane took a cell (Step 1) or a cell and line (Step 2) and loaded its
+// 60 or 20 stencil values from global memory, resolving ghosts at each; 128
+// registers, 16 warps per SM, waiting on those loads and on barriers.  FP32,
+// 1024^2, order 9, per launch: 288 -> 163 us (x), 317 -> 175 us (y), now bound by
+// issue slots and latency together (87 M warp instructions; the DRAM traffic
+// alone would take 80 us); FP64 512^2: 730 -> 558 us, near the FP64 pipe's
+// bound; 47 x 33, order 5: 38 -> 12 us, where the ghosts' serial loads had been
+// the time.
+template <typename R, int DIR>
+struct ReconTile {
+    static constexpr int TA = DIR == 0 ? 28 : 12, TB = DIR == 0 ? 4 : (sizeof(R) == 4 ? 16 : 8);
+    static constexpr int threads = (TA + 4) * TB;
+};
+
+template <int M, typename R, int DIR>
+struct ReconShared {
+    using T = ReconTile<R, DIR>;
+    static constexpr bool BULK32 = sizeof(R) == 4;
+    static constexpr int TA = T::TA, TB = T::TB, TAH = TA + 4;
+    static constexpr int NA = BULK32 ? 12 : 8;  // planes of A: W (hi), W_t, lo
+    // plane strides = 8 mod 32, so that lanes of 8 cells x 4 variables touch every bank once
+    static constexpr int pad(int n) { return ((n + 23) & ~31) + 8; }
+    static constexpr int nc = TAH * TB;                                   // cells with their halo along a
+    static constexpr int nA = TAH * (TB + 4);                             // and along b
+    static constexpr int sA = pad(nA), sB = pad(nc);                      // plane strides
+    static constexpr int nst = TAH * (TB + 5), nsn = (TA + 5) * TB;       // faces across b, along a
+    // offsets in bytes
+    static constexpr int st = 0, sn = st + nst * 8, A = sn + nsn * 8;     // sigma; averages and slopes
+    static constexpr int B = A + NA * sA * (int)sizeof(R);                // line slopes [M * 4][sB]
+    static constexpr int la = B + 4 * M * sB * (int)sizeof(R);            // line averages [M * 4][sB]
+    static constexpr int at = la + 4 * M * sB * (int)sizeof(R);           // DFFs of S0, S1, r5 [3][nc]: tangential
+    static constexpr int an = at + 3 * nc * (int)sizeof(R);               // and normal
+    static constexpr int ct = an + 3 * nc * (int)sizeof(R);               // stencil codes: tangential
+    static constexpr int cn = ct + nc * 4;                                // and normal
+    static constexpr int bytes = cn + nc * 4;
+};
+
+// A ghost cell's value into shared memory
+template <int M, typename R, bool WALLS>
+__device__ __forceinline__ void ghost_into(R* d, const Mesh& g, const R* S, const CellMap& c, int kind, int v, int l)
+{
+    if (WALLS && (c.state || c.wx || c.wy)) *d = mapped<2, M, R, WALLS>(g, S, c, kind, v, l);
+    else if ((c.zx && (kind == 1 || kind == 3)) || (c.zy && (kind == 2 || kind == 4))) *d = (R)0;
+    else copy_async1(d, S + value_plane<2, M>(kind, v, l) * g.plane + c.idx);
 }
 
-// Steps 1-2 of one direction, fused through shared memory.  A tile is TA x TB
-// cells (a along the face normal, b across it) of the range a in [-1, na],
-// b in [-1, nb] whose faces the stage evaluates (ghost columns and rows
-// included: Step 3 reads the face states of the rows beside the mesh).  Phase
-// 1 runs Step 1 for the tile and two halo columns on each side along a and
-// keeps each cell's M line averages, its average and the DFF of its normal
-// stencil in shared memory; phase 2 runs Step 2 (Algorithm 1) for every
-// (cell, Gauss line) of the tile from there and writes both face states.
-// The line averages never reach global memory; the halo costs 4 / TA more
-// Step 1 work.  Shared memory per CTA: (TA + 4) TB (4 M + 8) values of R,
-// launched as dynamic shared memory.  Shared-memory and thread layouts keep
-// the global x index fastest.  Work items are tiles (Work offsets count
-// tiles per mesh for the tile shape of the launch).
+// body(StTag<0>()) .. body(StTag<N - 1>())
+template <int N, int K = 0, typename Body>
+__device__ __forceinline__ void for_rows(Body&& body)
+{
+    if constexpr (K < N) {
+        body(StTag<K>());
+        for_rows<N, K + 1>(body);
+    }
+}
+
+// (quotient, remainder) by a compile-time extent
+template <int N>
+__device__ __forceinline__ void split(int t, int& q, int& r) { q = t / N; r = t - q * N; }
+
 template <int M, typename R, bool WALLS, int DIR, bool ONE>
-__global__ void __launch_bounds__(256) k_recon(Work w, int stage, int TA, int TB)
+__global__ void __launch_bounds__(ReconTile<R, DIR>::threads, sizeof(R) == 4 ? 768 / ReconTile<R, DIR>::threads : 1)
+k_recon(Work w, int stage)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned long long cnt[4];
+    using L = ReconShared<M, R, DIR>;
     constexpr bool BULK32 = sizeof(R) == 4;
-    constexpr int NV = 4;
+    constexpr int TA = L::TA, TB = L::TB, TAH = L::TAH, nc = L::nc, sA = L::sA, sB = L::sB;
+    constexpr int NT = ReconTile<R, DIR>::threads;
     if (threadIdx.x < 4) cnt[threadIdx.x] = 0;
-    const int TAH = TA + 4;
-    const int ncs = TAH * TB;                       // cells held per tile
-    R* s_la = (R*)smem_raw;                         // [M][ncs][4] line averages
-    R* s_hi = s_la + (size_t)M * ncs * 4;           // [ncs][4] averages (FP32 bulk: hi)
-    R* s_dn = s_hi + (size_t)ncs * 4;               // [ncs][4] packed normal DFF (tile cells)
-    const int sa = DIR == 0 ? 1 : TB;               // shared-memory stride of a
-    for (long long tile = blockIdx.x; tile < w.total; tile += gridDim.x) {
+    double* s_st = (double*)(smem_raw + L::st);
+    double* s_sn = (double*)(smem_raw + L::sn);
+    R* s_A = (R*)(smem_raw + L::A);
+    R* s_B = (R*)(smem_raw + L::B);
+    R* s_la = (R*)(smem_raw + L::la);
+    R* s_at = (R*)(smem_raw + L::at);
+    R* s_an = (R*)(smem_raw + L::an);
+    int* s_ct = (int*)(smem_raw + L::ct);
+    int* s_cn = (int*)(smem_raw + L::cn);
+    // shared-memory strides of a and b: the global x index is fastest
+    constexpr int aA = DIR == 0 ? 1 : TB + 4, bA = DIR == 0 ? TAH : 1;  // of A
+    constexpr int aB = DIR == 0 ? 1 : TB, bB = DIR == 0 ? TAH : 1;      // of B, la and the cell arrays
+    constexpr int aT = DIR == 0 ? 1 : TB + 5, bT = DIR == 0 ? TAH : 1;  // of the tangential sigma
+    constexpr int aN = DIR == 0 ? 1 : TB, bN = DIR == 0 ? TA + 5 : 1;   // of the normal sigma
+    // this thread's cell of the tile and its halo
+    const int tc = threadIdx.x;
+    int ia, ib;
+    if (DIR == 0) split<TAH>(tc, ib, ia); else split<TB>(tc, ia, ib);
+    {
+        // one tile per block: the tiles along a shock take many times longer, and the
+        // hardware deals blocks to SMs as they come free (dealt in fixed strides, a
+        // 960 x 240 mesh put most of them on a few SMs: 2.29 instead of 0.9 ms)
         long long ltl;
-        const Mesh& g = mesh_of<ONE>(w, tile, ltl);
+        const Mesh& g = mesh_of<ONE>(w, blockIdx.x, ltl);
         int na, nb;
         local_dims<M>(g, DIR, na, nb);
         const int nta = (na + 2 + TA - 1) / TA;
         const int lt = (int)ltl;                    // 32-bit tile index (bounded on the host)
         const int a0 = -1 + (lt % nta) * TA, b0 = -1 + (lt / nta) * TB;
+        const int a = a0 - 2 + ia, b = b0 + ib;
+        const bool on = a <= na + 2 && b <= nb;                  // within the mesh's halo
+        const bool core = on && ia >= 2 && ia < TA + 2 && a <= na;  // evaluates its faces
         const R* S = state_planes<R>(g, stage == 1 ? 0 : 1);
         const double tb = WALLS ? stage_time(g, stage) : 0.0;  // inflow ghost states
-        // sigma of the DFF (Sec. 3.1): of step n-1 in both stages, or, in stage 2
-        // of the stage-lag reading, the face means of stage 1 of this step
-        const bool lag_stage = stage == 2 && g.dff_lag;
-        const double* SX = lag_stage ? g.sig_xn : g.sig_x;
-        const double* SY = lag_stage ? g.sig_yn : g.sig_y;
-        // ---- phase 1: Step 1 of the tile and its halo along a
-        for (int t = threadIdx.x; t < ncs; t += blockDim.x) {
-            int ia, ib;
-            if (DIR == 0) { ib = t / TAH; ia = t - ib * TAH; }
-            else { ia = t / TB; ib = t - ia * TB; }
-            const int a = a0 - 2 + ia, b = b0 + ib;
-            if (a > na + 2 || b > nb) continue;     // beyond the mesh's halo
-            const bool core = ia >= 2 && ia < TA + 2 && a <= na;
-            R res[M][4], hi[4], dn[4];
-            step1_cell<M, R, WALLS>(g, S, DIR, na, nb, a, b, tb, SX, SY, core, res, hi, dn);
-#pragma unroll
-            for (int l = 0; l < M; ++l) st4(s_la + ((size_t)l * ncs + t) * 4, res[l]);
-            st4(s_hi + (size_t)t * 4, hi);
-            if (core) st4(s_dn + (size_t)t * 4, dn);
-        }
-        __syncthreads();
-        // ---- phase 2: Step 2 of every (cell, Gauss line) of the tile
-        const R hn = (R)(DIR == 0 ? g.dx : g.dy);
-        const R ih = (R)1 / hn;
-        const R ghi = (R)g.ghi, glo = (R)g.glo, eps = (R)g.eps;
-        R* FR = (R*)g.FR[DIR];
-        const long long nrow = fr_nrow(DIR, na, nb);
         const long long P = g.plane;
-        const int nitem = TA * TB * M;
-        for (int it = threadIdx.x; it < nitem; it += blockDim.x) {
-            const int l = it % M, c = it / M;
+        // ---- stage
+        for (int t = threadIdx.x; t < L::nA; t += NT) {
             int ia, ib;
-            if (DIR == 0) { ib = c / TA; ia = c - ib * TA + 2; }
-            else { ia = c / TB + 2; ib = c - (ia - 2) * TB; }
-            const int a = a0 - 2 + ia, b = b0 + ib;
-            if (a > na || b > nb) continue;
-            const int tc = DIR == 0 ? ib * TAH + ia : ia * TB + ib;
-            R pk[4];
-            ld4(s_dn + (size_t)tc * 4, pk);
-            DffR<R> dff = dff_unpack<R>(pk);
-            {
-                // branch counts, aggregated per warp
-                int bi = dff.st < 0 ? 0 : dff.st - ST_R5 + 1;
-                unsigned act = __activemask();
-                unsigned same = __match_any_sync(act, bi);
-                if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&cnt[bi], (unsigned long long)__popc(same));
-            }
-            // the line averages and averages of the five stencil cells on this line
-            R la5[5][4], sh[5][4];
+            if (DIR == 0) split<TAH>(t, ib, ia); else split<TB + 4>(t, ia, ib);
+            const int a = a0 - 2 + ia, b = b0 - 2 + ib;
+            if (a > na + 2 || b > nb + 2) continue;
+            const int i = DIR == 0 ? a : b, j = DIR == 0 ? b : a;
+            R* d = s_A + t;
+            if ((unsigned)i < (unsigned)g.nx && (unsigned)j < (unsigned)g.ny) {
+                const R* p = S + (long long)j * g.nx + i;
 #pragma unroll
-            for (int q = 0; q < 5; ++q) {
-                ld4(s_la + ((size_t)l * ncs + tc + (q - 2) * sa) * 4, la5[q]);
-                ld4(s_hi + (size_t)(tc + (q - 2) * sa) * 4, sh[q]);
-            }
-            // the normal stencil of line slopes: a direct walk for interior cells
-            const bool inner = a >= 2 && a + 2 < na && b >= 0 && b < nb;
-            const long long ci = DIR == 0 ? (long long)b * g.nx + a : (long long)a * g.nx + b;
-            const long long sn = DIR == 0 ? 1 : g.nx;                  // normal neighbour stride
-            const int pl0 = (DIR == 0 ? 12 : 12 + 4 * M) + 4 * l;       // first line-slope plane of line l
-            R sl[NV][5];
-            if (inner) {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    const R* ws = S + (pl0 + vglob(DIR, v)) * P + ci;
-#pragma unroll
-                    for (int q = 0; q < 5; ++q) sl[v][q] = ws[(q - 2) * sn];
+                for (int v = 0; v < 4; ++v) {
+                    copy_async1(d + v * sA, p + vglob(DIR, v) * P);
+                    copy_async1(d + (4 + v) * sA, p + ((DIR == 0 ? 8 : 4) + vglob(DIR, v)) * P);
+                    if (BULK32) copy_async1(d + (8 + v) * sA, p + (12 + 8 * M + vglob(DIR, v)) * P);
                 }
             } else {
+                const CellMap c = cell_map<WALLS>(g, i, j, tb);
 #pragma unroll
-                for (int v = 0; v < NV; ++v)
-#pragma unroll
-                    for (int q = 0; q < 5; ++q) sl[v][q] = lcell<2, M, R, WALLS>(g, S, DIR, 3, v, l, a + q - 2, b, tb);
-            }
-            R sideL[3][4], sideR[3][4];
-            with_stencil<M - 2>(dff, [&](auto tag) {
-                constexpr int ST = decltype(tag)::value;
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    // FP32 bulk: la5 holds increments over the cells' hi, so a
-                    // difference of line averages is (hi - hi) + (la - la), and the
-                    // face values come out as increments over this cell's hi
-                    R qi = la5[2][v], dp[10];
-#pragma unroll
-                    for (int q = 0; q < 5; ++q) {
-                        dp[q] = BULK32 ? (sh[q][v] - sh[2][v]) + (la5[q][v] - qi) : la5[q][v] - qi;
-                        dp[5 + q] = hn * sl[v][q];
-                    }
-                    R out[6];
-                    recon_st<R, 6, M - 2, ST, 0>(dff, dp, out, ghi, glo, eps);
-                    // FP32 bulk: the left state of face a+1 over the hi of that face's
-                    // right cell a+1, like the right state: a face's two states share a base
-                    const R shift = BULK32 ? sh[2][v] - sh[3][v] : (R)0;
-                    sideL[0][v] = (qi + shift) + out[0]; sideL[1][v] = out[1] * ih; sideL[2][v] = out[2] * ih * ih;
-                    sideR[0][v] = qi + out[3]; sideR[1][v] = out[4] * ih; sideR[2][v] = out[5] * ih * ih;
+                for (int v = 0; v < 4; ++v) {
+                    ghost_into<M, R, WALLS>(d + v * sA, g, S, c, 0, vglob(DIR, v), 0);
+                    ghost_into<M, R, WALLS>(d + (4 + v) * sA, g, S, c, DIR == 0 ? 2 : 1, vglob(DIR, v), 0);
+                    if (BULK32) ghost_into<M, R, WALLS>(d + (8 + v) * sA, g, S, c, 5, vglob(DIR, v), 0);
                 }
-            });
-            // side 0: left state of face a+1 (value at xi = +1/2)
-            if (a + 1 <= na) {
-                const long long row = fr_row(DIR, na, nb, b + 1, a + 1);
-#pragma unroll
-                for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(nrow, M, 0, nd, l, row), sideL[nd]);
-            }
-            // side 1: right state of face a (value at xi = -1/2)
-            if (a >= 0) {
-                const long long row = fr_row(DIR, na, nb, b + 1, a);
-#pragma unroll
-                for (int nd = 0; nd < 3; ++nd) st4(FR + fr_off(nrow, M, 1, nd, l, row), sideR[nd]);
             }
         }
-        __syncthreads();  // the next tile reuses the shared memory
+        if (on) {
+            const int i = DIR == 0 ? a : b, j = DIR == 0 ? b : a;
+            R* d = s_B + tc;
+            if ((unsigned)i < (unsigned)g.nx && (unsigned)j < (unsigned)g.ny) {
+                const R* p = S + (DIR == 0 ? 12 : 12 + 4 * M) * P + (long long)j * g.nx + i;
+#pragma unroll
+                for (int l = 0; l < M; ++l)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) copy_async1(d + (4 * l + v) * sB, p + (4 * l + vglob(DIR, v)) * P);
+            } else {
+                const CellMap c = cell_map<WALLS>(g, i, j, tb);
+#pragma unroll
+                for (int l = 0; l < M; ++l)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v)
+                        ghost_into<M, R, WALLS>(d + (4 * l + v) * sB, g, S, c, DIR == 0 ? 3 : 4, vglob(DIR, v), l);
+            }
+        }
+        {
+            // sigma of the DFF (Sec. 3.1): of step n-1 in both stages, or, in stage 2
+            // of the stage-lag reading, the face means of stage 1 of this step
+            const bool lag_stage = stage == 2 && g.dff_lag;
+            const double* SX = lag_stage ? g.sig_xn : g.sig_x;
+            const double* SY = lag_stage ? g.sig_yn : g.sig_y;
+            for (int t = threadIdx.x; t < L::nst; t += NT) {
+                int ia, q;
+                if (DIR == 0) split<TAH>(t, q, ia); else split<TB + 5>(t, ia, q);
+                const int a = a0 - 2 + ia, f = b0 - 2 + q;  // tangential face f of column a
+                if (a > na + 2 || f > nb + 3) continue;
+                s_st[t] = lsigT<WALLS>(g, SX, SY, DIR, a, f);
+            }
+            for (int t = threadIdx.x; t < L::nsn; t += NT) {
+                int q, ib;
+                if (DIR == 0) split<TA + 5>(t, ib, q); else split<TB>(t, q, ib);
+                const int f = a0 - 2 + q, b = b0 + ib;      // normal face f of row b
+                if (f > na + 3 || b > nb) continue;
+                s_sn[t] = lsigN<2, WALLS>(g, SX, SY, DIR, f, b);
+            }
+        }
+        copy_commit();
+        copy_wait<0>();
+        __syncthreads();
+        // ---- 0: DFFs
+        if (on) {
+            double s6[6];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) s6[q] = s_st[ia * aT + (ib + q) * bT];
+            const Dff dt = dff_select(g.order, s6, g.thr);
+            s_ct[tc] = dt.st;
+            if (dt.st < 0) {
+                s_at[tc] = (R)dt.a[0]; s_at[nc + tc] = (R)dt.a[1]; s_at[2 * nc + tc] = (R)dt.a[3];
+            }
+            if (core) {
+                // tangential r5 DFF of this cell, reused by Step 3
+                ((R*)g.AT[DIR])[cell_idx(DIR, na, nb, a, b)] = (R)dt.a[3];
+#pragma unroll
+                for (int q = 0; q < 6; ++q) s6[q] = s_sn[(ia - 2 + q) * aN + ib * bN];
+                const Dff dn = dff_select(g.order, s6, g.thr);
+                s_cn[tc] = dn.st;
+                if (dn.st < 0) {
+                    s_an[tc] = (R)dn.a[0]; s_an[nc + tc] = (R)dn.a[1]; s_an[2 * nc + tc] = (R)dn.a[3];
+                }
+                // branch counts of the M lines, aggregated per warp
+                const int bi = dn.st < 0 ? 0 : dn.st - ST_R5 + 1;
+                const unsigned same = __match_any_sync(__activemask(), bi);
+                if ((int)(threadIdx.x & 31) == __ffs(same) - 1)
+                    atomicAdd(&cnt[bi], (unsigned long long)(M * __popc(same)));
+            }
+        }
+        __syncthreads();
+        const R ghi = (R)g.ghi, glo = (R)g.glo, eps = (R)g.eps;
+        // ---- 1: Step 1; a lane per cell, its variables in turn
+        if (on) {
+            const R ht = (R)(DIR == 0 ? g.dy : g.dx);
+            const R* A = s_A + ia * aA + (ib + 2) * bA;
+            with_stencil<M>(s_ct[tc], [&](auto tag) {
+                constexpr int ST = decltype(tag)::value;
+                if constexpr (ST >= 0 && BULK32) {
+                    // differences of averages as (hi - hi) + (lo - lo), and the line
+                    // average kept as lo + increment (over the cell's hi); two
+                    // variables at once
+#pragma unroll
+                    for (int v = 0; v < 4; v += 2) {
+                        const float* A0 = (const float*)A + v * sA;
+                        auto at2 = [&](int k) { return make_float2(A0[k], A0[k + sA]); };
+                        const float2 h0 = at2(0), l0 = at2(8 * sA);
+                        float2 dp[10];
+#pragma unroll
+                        for (int q = 0; q < 5; ++q) {
+                            if (st_tap(ST, q)) {
+                                dp[q] = add2(sub2(at2((q - 2) * bA), h0), sub2(at2(8 * sA + (q - 2) * bA), l0));
+                            }
+                            if (st_tap(ST, 5 + q)) dp[5 + q] = mul2(ht, at2(4 * sA + (q - 2) * bA));
+                        }
+                        for_rows<M>([&](auto row) {
+                            constexpr int l = decltype(row)::value;
+                            const float2 r = add2(l0, row_taps<M - 2, ST, 6 + l>(dp));
+                            s_la[(4 * l + v) * sB + tc] = r.x;
+                            s_la[(4 * l + v + 1) * sB + tc] = r.y;
+                        });
+                    }
+                } else {
+#pragma unroll(ST >= 0 ? 4 : 1)
+                    for (int v = 0; v < 4; ++v) {
+                        const R* Av = A + v * sA;
+                        R dp[10], out[M];
+#pragma unroll
+                        for (int q = 0; q < 5; ++q) {
+                            dp[q] = Av[(q - 2) * bA] - Av[0];
+                            if (BULK32) dp[q] += Av[8 * sA + (q - 2) * bA] - Av[8 * sA];
+                            dp[5 + q] = ht * Av[4 * sA + (q - 2) * bA];
+                        }
+                        if constexpr (ST >= 0) {
+                            const auto& T = c_tab[M - 2];
+                            double e[2], o[2], E[2], O[2];
+                            sym_data<double>((const double*)dp, e, o, E, O);
+#pragma unroll
+                            for (int l = 0; l < (M + 1) / 2; ++l) {
+                                double p, q;
+                                sym_row<ST, double>(T.sym[ST - ST_R5][3 + l], e, o, E, O, p, q);
+                                out[l] = (R)(M - 1 - l == l ? p : p + q);
+                                if (M - 1 - l != l) out[M - 1 - l] = (R)(p - q);
+                            }
+                        } else {
+                            const R al[4] = {s_at[tc], s_at[nc + tc], s_at[2 * nc + tc], s_at[2 * nc + tc]};
+                            recon_ao<R, M>(al, M - 2, 6, dp, out, ghi, glo, eps);
+                        }
+                        const R base = BULK32 ? Av[8 * sA] : Av[0];
+#pragma unroll
+                        for (int l = 0; l < M; ++l) s_la[(4 * l + v) * sB + tc] = base + out[l];
+                    }
+                }
+            });
+            if (BULK32 && core) {
+                // hi and its tangential differences: the bases of the face states
+                // and of Step 3's segments
+                R hi[4], tdm[4], tdp[4];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    hi[v] = A[v * sA];
+                    tdm[v] = A[v * sA - bA] - hi[v];
+                    tdp[v] = A[v * sA + bA] - hi[v];
+                }
+                R* td = (R*)g.TD[DIR] + cell_idx(DIR, na, nb, a, b) * 12;
+                st4(td, hi);
+                st4(td + 4, tdm);
+                st4(td + 8, tdp);
+            }
+        }
+        __syncthreads();
+        // ---- 2: Step 2; variable fastest
+        {
+            const R hn = (R)(DIR == 0 ? g.dx : g.dy);
+            const R ih = (R)1 / hn, ih2 = ih * ih;
+            const long long nrow = fr_nrow(DIR, na, nb) * 4;  // values of a line's plane
+            for (int it = threadIdx.x; it < 4 * TA * TB; it += NT) {
+                const int v = it & 3, c = it >> 2;
+                int ia, ib;
+                if (DIR == 0) split<TA>(c, ib, ia); else split<TB>(c, ia, ib);
+                ia += 2;
+                const int a = a0 - 2 + ia, b = b0 + ib;
+                if (a > na || b > nb) continue;
+                const int t = ia * aB + ib * bB;
+                // side 0: left state of face a+1 (value at xi = +1/2), side 1: right
+                // state of face a (xi = -1/2)
+                R* FR = (R*)g.FR[DIR];
+                R* fl = FR + fr_row(DIR, na, nb, b + 1, a + 1) * 4 + v;
+                R* fr = FR + 3 * M * nrow + fr_row(DIR, na, nb, b + 1, a >= 0 ? a : 0) * 4 + v;
+                const bool left = a + 1 <= na, right = a >= 0;
+                // value r (0..2 left state and its derivatives, 3..5 right) of line l
+                auto put = [&](int r, int l, R x) {
+                    if (r < 3) { if (left) fl[(r * M + l) * nrow] = x; }
+                    else { if (right) fr[((r - 3) * M + l) * nrow] = x; }
+                };
+                const R* A = s_A + v * sA + ia * aA + (ib + 2) * bA;
+                const R* la = s_la + v * sB + t;
+                const R* sl = s_B + v * sB + t;
+                // FP32 bulk: line averages are increments over the cells' hi, so a
+                // difference of them is (hi - hi) + (la - la), and the face values
+                // come out as increments over this cell's hi; the left state of face
+                // a+1 over the hi of that face's right cell a+1, like the right
+                // state: a face's two states share a base
+                R h5[5];
+#pragma unroll
+                for (int q = 0; q < 5; ++q) h5[q] = BULK32 ? A[(q - 2) * aA] - A[0] : (R)0;
+                with_stencil<M>(s_cn[t], [&](auto tag) {
+                    constexpr int ST = decltype(tag)::value;
+                    if constexpr (ST >= 0 && BULK32) {
+                        // two lines at once (the last of an odd number twice)
+                        constexpr int NP = (M + 1) / 2;
+                        float2 dp[NP][10], qi[NP];
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) {
+                            constexpr int step = 4 * sB;
+                            const int l0 = 2 * p, l1 = 2 * p + 1 < M ? 2 * p + 1 : 2 * p;
+                            auto two = [&](const R* x, int k) { return make_float2(x[l0 * step + k], x[l1 * step + k]); };
+                            qi[p] = two(la, 0);
+#pragma unroll
+                            for (int q = 0; q < 5; ++q) {
+                                if (st_tap(ST, q))
+                                    dp[p][q] = add2(make_float2(h5[q], h5[q]), sub2(two(la, (q - 2) * aB), qi[p]));
+                                if (st_tap(ST, 5 + q)) dp[p][5 + q] = mul2(hn, two(sl, (q - 2) * aB));
+                            }
+                        }
+                        for_rows<6>([&](auto row) {
+                            constexpr int r = decltype(row)::value;
+#pragma unroll
+                            for (int p = 0; p < NP; ++p) {
+                                float2 x = row_taps<M - 2, ST, r>(dp[p]);
+                                if (r == 0) x = add2(sub2(qi[p], make_float2(h5[3], h5[3])), x);
+                                else if (r == 3) x = add2(qi[p], x);
+                                else x = mul2(r % 3 == 1 ? ih : ih2, x);
+                                put(r, 2 * p, x.x);
+                                if (2 * p + 1 < M) put(r, 2 * p + 1, x.y);
+                            }
+                        });
+                    } else {
+#pragma unroll(ST >= 0 ? 2 : 1)
+                        for (int l = 0; l < M; ++l) {
+                            R qi = la[4 * l * sB], dp[10], out[6];
+#pragma unroll
+                            for (int q = 0; q < 5; ++q) {
+                                dp[q] = h5[q] + (la[4 * l * sB + (q - 2) * aB] - qi);
+                                dp[5 + q] = hn * sl[4 * l * sB + (q - 2) * aB];
+                            }
+                            if constexpr (ST >= 0) {
+                                const auto& T = c_tab[M - 2];
+                                double e[2], o[2], E[2], O[2];
+                                sym_data<double>((const double*)dp, e, o, E, O);
+#pragma unroll
+                                for (int nd = 0; nd < 3; ++nd) {
+                                    double p, q;
+                                    sym_row<ST, double>(T.sym[ST - ST_R5][nd], e, o, E, O, p, q);
+                                    out[nd] = (R)(p + q);
+                                    out[3 + nd] = (R)(nd == 1 ? q - p : p - q);
+                                }
+                            } else {
+                                const R al[4] = {s_an[t], s_an[nc + t], s_an[2 * nc + t], s_an[2 * nc + t]};
+                                recon_ao<R, 6>(al, M - 2, 0, dp, out, ghi, glo, eps);
+                            }
+                            put(0, l, (qi - h5[3]) + out[0]);
+                            put(1, l, out[1] * ih);
+                            put(2, l, out[2] * ih2);
+                            put(3, l, qi + out[3]);
+                            put(4, l, out[4] * ih);
+                            put(5, l, out[5] * ih2);
+                        }
+                    }
+                });
+            }
+        }
     }
+    __syncthreads();
     if (threadIdx.x < 4 && cnt[threadIdx.x] && w.n > 0)
         atomicAdd(&(ONE ? w.m0 : w.mesh[0]).branch[threadIdx.x], cnt[threadIdx.x]);
 }
@@ -495,7 +665,7 @@ template <int M> struct FluxStrip {
 
 // Values of one warp in shared memory: the ring of W and W_n of both sides; the
 // tangential derivatives of the step; two slots of what only the step's own
-// points read: W_nn, and the bases of the face (hi of its right cell, TD, FP32
+// points read: W_nn, and the bases of the face (TD of its right cell, FP32
 // bulk) with the tangential DFF of its two cells.
 template <int M, typename R>
 struct FluxShared {
@@ -504,9 +674,8 @@ struct FluxShared {
     static constexpr int ring = 0;                                    // [side][W, W_n][M][RING][4]
     static constexpr int tang = ring + 2 * 2 * M * RING * 4;          // [side][t, tt, nt][M][FW][4]
     static constexpr int nn = tang + 2 * 3 * M * FW * 4;              // [slot][side][M][FW][4]
-    static constexpr int hb = nn + 2 * 2 * M * FW * 4;                // [slot][FW][4]
-    static constexpr int td = hb + (BULK32 ? 2 * FW * 4 : 0);         // [slot][FW][8]
-    static constexpr int at = td + (BULK32 ? 2 * FW * 8 : 0);         // [slot][side][FW]
+    static constexpr int td = nn + 2 * 2 * M * FW * 4;                // [slot][FW][12]
+    static constexpr int at = td + (BULK32 ? 2 * FW * 12 : 0);        // [slot][side][FW]
     static constexpr int total = at + (2 * 2 * FW + 3) / 4 * 4;
 };
 
@@ -516,27 +685,6 @@ __host__ __device__ inline long long flux_steps(int M, int nx, int ny)
     const int fw = 32 / M;
     return (long long)((nx + 1 + fw - 1) / fw) * ny + (long long)(ny + 1) * ((nx + fw - 1) / fw);
 }
-
-__device__ __forceinline__ void copy_async16(void* dst, const void* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-template <typename R>
-__device__ __forceinline__ void copy_async1(R* dst, const R* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-                 "n"(sizeof(R))
-                 : "memory");
-}
-__device__ __forceinline__ void copy_async4(float* dst, const float* src) { copy_async16(dst, src); }
-__device__ __forceinline__ void copy_async4(double* dst, const double* src)
-{
-    copy_async16(dst, src);
-    copy_async16(dst + 2, src + 2);
-}
-__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Step 3 for one (side, face, variable): the derivatives t, tt and nt at the M
 // lines of the face, from the 3 M points of segments b-1, b, b+1 (W: value of
@@ -609,7 +757,7 @@ struct StripPoint {
         if (nd < 2) ld4(s + L::ring + (((side * 2 + nd) * M + l) * L::RING + own_q) * 4, v);
         else ld4(s + L::nn + (((slot * 2 + side) * M + l) * L::FW + x) * 4, v);
     }
-    __device__ __forceinline__ void base(R* v) const { ld4(s + L::hb + (slot * L::FW + x) * 4, v); }
+    __device__ __forceinline__ void base(R* v) const { ld4(s + L::td + (slot * L::FW + x) * 12, v); }
     __device__ __forceinline__ void tangential(int side, int q, R* v) const
     {
         ld4(s + L::tang + (((side * 3 + q) * M + l) * L::FW + x) * 4, v);
@@ -993,12 +1141,11 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flu
             slot3 = slot3 == 2 ? 0 : slot3 + 1;
         };
         // and of what only a step's own points read, for step kn: W_nn, and the
-        // face's items dealt to its M lanes: hi of the right cell by variable, TD
-        // by halves, the tangential DFF of its two cells
+        // face's items dealt to its M lanes: TD of the right cell in three parts,
+        // the tangential DFF of its two cells
         int kn = k0;
         const int b0 = dir == 0 ? k0 : k0 * FW + x;
         const R* pn = (const R*)g.FR[dir] + fr_off(fr_nrow(dir, na, nb), M, 0, 2, l, fr_row(dir, na, nb, b0 + 1, mine ? f : 0));
-        long long ci = dir == 0 ? (long long)b0 * g.nx + f : (long long)f * g.nx + b0;
         long long cidx = cell_idx(dir, na, nb, f, b0);
         const long long prev = dir == 0 ? 1 : nb + 2;
         auto load_own = [&]() {
@@ -1008,22 +1155,15 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flu
 #pragma unroll
                 for (int side = 0; side < 2; ++side)
                     copy_async4(sm + L::nn + (((slot * 2 + side) * M + l) * FW + x) * 4, pn + side * 3 * plane);
-                if (BULK32) {
-                    const R* SF = state_planes<R>(g, STAGE == 1 ? 0 : 1);
-                    for (int v = l; v < 4; v += M) {
-                        R* dst = sm + L::hb + (slot * FW + x) * 4 + v;
-                        if (f < na) copy_async1(dst, SF + vglob(dir, v) * g.plane + ci);
-                        else *dst = ghost_average<M, R>(g, SF, dir, v, f, b, STAGE);
-                    }
-                    if (l < 2) copy_async4(sm + L::td + (slot * FW + x) * 8 + l * 4, (const R*)g.TD[dir] + cidx * 8 + l * 4);
-                }
+                if (BULK32)
+                    for (int q = l; q < 3; q += M)
+                        copy_async4(sm + L::td + (slot * FW + x) * 12 + q * 4, (const R*)g.TD[dir] + cidx * 12 + q * 4);
                 if (l == M - 1) {
                     copy_async1(sm + L::at + (slot * 2 + 0) * FW + x, (const R*)g.AT[dir] + cidx - prev);
                     copy_async1(sm + L::at + (slot * 2 + 1) * FW + x, (const R*)g.AT[dir] + cidx);
                 }
             }
             pn += step;
-            ci += dir == 0 ? g.nx : FW;
             cidx += dir == 0 ? na + 6 : FW;
             ++kn;
         };
@@ -1052,8 +1192,8 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flu
                 }
                 R dm = (R)0, dp = (R)0;
                 if (BULK32) {
-                    dm = sm[L::td + (slot * FW + xi) * 8 + v];
-                    dp = sm[L::td + (slot * FW + xi) * 8 + 4 + v];
+                    dm = sm[L::td + (slot * FW + xi) * 12 + 4 + v];
+                    dp = sm[L::td + (slot * FW + xi) * 12 + 8 + v];
                 }
                 // scaled by the tangential r5 DFF of the reconstructing cell
                 // (f-1 for the left state, f for the right)

@@ -7,10 +7,11 @@
 namespace cgks {
 typedef void (*KStage)(Work, int);
 typedef void (*KOne)(Work);
-typedef void (*KTile)(Work, int, int, int);
 struct Kfns {
-    KTile recon[2];            // 2-D Steps 1-2 per direction (meshes without walls)
-    KTile reconw[2];           // the same with the wall ghost rules
+    KStage recon[2];           // 2-D Steps 1-2 per direction (meshes without walls)
+    KStage reconw[2];          // the same with the wall ghost rules
+    int recon_tile[2][2];      // their tile shapes (TA, TB), blocks and dynamic shared memory
+    int recon_threads[2], recon_bytes[2];
     KStage normal, normalw;    // 1-D Step 2, without and with the wall ghost rules
     KOne flux1, flux2, upd1, upd2, cfl, siginit, check;
     KStage convert;  // FP32-bulk state copies (to_float = 1: FP64 -> float planes)

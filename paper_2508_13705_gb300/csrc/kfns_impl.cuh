@@ -24,8 +24,14 @@ constexpr KOne flux_fn()
 template <int D, int M, typename R, bool ONE>
 Kfns make_kfns_one()
 {
-    Kfns k;
+    Kfns k = {};
     if constexpr (D == 2) {
+        using T0 = ReconShared<M, R, 0>;
+        using T1 = ReconShared<M, R, 1>;
+        k.recon_tile[0][0] = T0::TA; k.recon_tile[0][1] = T0::TB;
+        k.recon_tile[1][0] = T1::TA; k.recon_tile[1][1] = T1::TB;
+        k.recon_threads[0] = ReconTile<R, 0>::threads; k.recon_threads[1] = ReconTile<R, 1>::threads;
+        k.recon_bytes[0] = T0::bytes; k.recon_bytes[1] = T1::bytes;
         k.recon[0] = k_recon<M, R, false, 0, ONE>;
         k.recon[1] = k_recon<M, R, false, 1, ONE>;
         k.reconw[0] = k_recon<M, R, true, 0, ONE>;

@@ -186,6 +186,17 @@ extern "C" __attribute__((visibility("hidden"))) int cgks_build_tables(int order
             for (int k = 0; k < 5; ++k)
                 for (int d = 0; d < 10; ++d) t->cpoly[st][k][d] = (double)coef[k][d];
     }
+    for (int st = 3; st < 6; ++st)
+        for (int r = 0; r < 3 + (m + 1) / 2; ++r) {
+            const double* row = t->row[st][r < 3 ? r : 6 + (r - 3)];
+            double* c = t->sym[st - 3][r];
+            for (int j = 1; j <= 2; ++j) {
+                c[j - 1] = 0.5 * (row[2 + j] + row[2 - j]);
+                c[2 + j - 1] = 0.5 * (row[7 + j] - row[7 - j]);
+                c[4 + j - 1] = 0.5 * (row[2 + j] - row[2 - j]);
+                c[6 + j - 1] = 0.5 * (row[7 + j] + row[7 - j]);
+            }
+        }
     smoothness_matrix(2, &t->bm2[0][0]);
     smoothness_matrix(4, &t->bm4[0][0]);
     // Step 3: 3m nodes of segments b-1, b, b+1 (in units of the tangential h)

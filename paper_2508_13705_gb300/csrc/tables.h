@@ -19,6 +19,10 @@ struct CgksTables {
     // (an odd rule's middle point stands alone in the sums), k = 0 .. 5; entry 6: on
     // the sum and difference of what is common to all points of segments b-1, b+1
     double sd1[2][2][7], sd2[2][2][7];
+    // rows of r5, r7, r9 for mirrored places, on sums and differences of mirrored
+    // taps (see cgks_device.cuh): value, first and second derivative at xi = 1/2,
+    // then the value at Gauss nodes 0 and 1 (of m = 2: 0 only)
+    double sym[3][5][8];
     int m;
 };
 

@@ -1,7 +1,9 @@
 """The 2-D flux kernel marches warps over strips of 32 / m faces (16, 10, 8 for
-orders 5, 7, 9): meshes whose faces fill a strip exactly, fall one short or
-spill one over, in each direction, alone and as a batch (one work list over
-meshes of different sizes), against the oracle after one step.
+orders 5, 7, 9), and Steps 1-2 cover the mesh and a ring of ghost cells with
+tiles of 28 x 4 (x faces) and 12 x 16 (y faces; FP64 12 x 8) cells: meshes that
+fill strips or tiles exactly, fall one short or spill one over, in each
+direction, alone and as a batch (one work list over meshes of different sizes),
+against the oracle after one step.
 
 Tolerances: FP64 1e-12 relative L1 with every value within 1e-11 of the field's
 largest (the operation order differs); FP32 bulk 2e-7 for the averages and 1e-4
@@ -39,7 +41,8 @@ def check(got, orc, precision, what):
 
 def sizes(order):
     fw = 32 // {5: 2, 7: 3, 9: 4}[order]
-    return [(fw - 2, fw + 1), (fw - 1, fw), (fw, fw - 1), (fw + 1, 2 * fw), (2 * fw - 1, 3), (3, 2 * fw + 1)]
+    return [(fw - 2, fw + 1), (fw - 1, fw), (fw, fw - 1), (fw + 1, 2 * fw), (2 * fw - 1, 3), (3, 2 * fw + 1),
+            (26, 14), (27, 10), (25, 22), (54, 6)]
 
 
 @pytest.mark.parametrize("precision", [cgks.FP64, cgks.FP32_BULK])

@@ -736,6 +736,15 @@ __device__ __forceinline__ float recip(float x)
     return __fmaf_rn(r, __fmaf_rn(-x, r, 1.0f), r);
 }
 
+// 1 / sqrt(x).  FP32: the approximation (2 ulp) and one Newton step; without it
+// the half-range moments of a shock's two sides carry its error.
+__device__ __forceinline__ double recip_sqrt(double x) { return rsqrt(x); }
+__device__ __forceinline__ float recip_sqrt(float x)
+{
+    const float r = rsqrtf(x);
+    return __fmaf_rn(0.5f * r, __fmaf_rn(-x * r, r, 1.0f), r);
+}
+
 // The state variables of a Maxwellian: density and its reciprocal, velocity,
 // pressure, theta, and the specific kinetic energy ek = (U^2 + V^2) / 2.
 template <typename R, int D>
@@ -760,6 +769,16 @@ __device__ __forceinline__ Gas<R, D> gas_of(const R* W, R gm1)
 template <typename R>
 struct Hat { R r, a, b, p; };
 
+// the change of the internal energy density along a derivative, e = d(rho E)
+template <typename R, int D>
+__device__ __forceinline__ R internal(const Gas<R, D>& G, R e, R r, R a, R b)
+{
+    e -= G.ek * r;
+    e -= G.U * a;
+    if (D == 2) e -= G.V * b;
+    return e;
+}
+
 template <typename R, int D>
 __device__ __forceinline__ Hat<R> hat_of(const Gas<R, D>& G, R gm1, const R* x)
 {
@@ -767,10 +786,7 @@ __device__ __forceinline__ Hat<R> hat_of(const Gas<R, D>& G, R gm1, const R* x)
     h.r = x[0];
     h.a = x[1] - G.U * x[0];
     h.b = D == 2 ? x[2] - G.V * x[0] : (R)0;
-    h.p = gm1 * x[D + 1];
-    h.p -= (gm1 * G.U) * x[1];
-    if (D == 2) h.p -= (gm1 * G.V) * x[2];
-    h.p += (gm1 * G.ek) * x[0];
+    h.p = gm1 * internal(G, x[D + 1], h.r, h.a, h.b);
     return h;
 }
 
@@ -785,10 +801,7 @@ __device__ __forceinline__ Var<R> var_of(const Gas<R, D>& G, R gm1, const R* x)
     h.r = x[0];
     h.a = x[1] - G.U * x[0];
     h.b = D == 2 ? x[2] - G.V * x[0] : (R)0;
-    h.t = gm1 * x[D + 1];
-    h.t -= (gm1 * G.U) * x[1];
-    if (D == 2) h.t -= (gm1 * G.V) * x[2];
-    h.t += (gm1 * G.ek - G.th) * x[0];
+    h.t = gm1 * internal(G, x[D + 1], h.r, h.a, h.b) - G.th * h.r;
     return h;
 }
 template <typename R, int D>
@@ -875,16 +888,51 @@ __device__ __forceinline__ Range<R, NM> full_range(const Gas<R, D>& G)
     return H;
 }
 
-// rho <u^P psi> over the range
-template <int P, typename R, int D, int NM>
-__device__ __forceinline__ void moments(const Gas<R, D>& G, const Range<R, NM>& H, R Kx, R* out)
+// rho <psi> of the state W over its half range: m0 W plus what the cut at u = 0
+// carries, k (0, p, 0, p U / 2).  W enters with one rounding.
+template <typename R, int D, int NM>
+__device__ __forceinline__ void half_moments(const Gas<R, D>& G, const Range<R, NM>& H, const R* W, R* out)
 {
-    const R g = (R)0.5 * (G.V * G.V + Kx * G.th);
-    const R w = G.rho * H.m[P];
+    const R pk = G.p * H.k;
+    out[0] = H.m[0] * W[0];
+    out[1] = H.m[0] * W[1] + pk;
+    if (D == 2) out[2] = H.m[0] * W[2];
+    out[D + 1] = H.m[0] * W[D + 1] + (R)0.5 * G.U * pk;
+}
+// its half-range Euler flux rho <u psi>
+template <typename R, int D, int NM>
+__device__ __forceinline__ void half_flux(const Gas<R, D>& G, const Range<R, NM>& H, const R* W, R Kx, R* out)
+{
+    const R w = H.m[0] * W[1] + G.p * H.k;
     out[0] = w;
-    out[1] = G.rho * H.m[P + 1];
+    out[1] = G.U * w + G.p * H.m[0];
     if (D == 2) out[2] = G.V * w;
-    out[D + 1] = (R)0.5 * G.rho * H.m[P + 2] + g * w;
+    out[D + 1] = (R)0.5 * G.U * out[1] + ((R)0.5 * (G.V * G.V + Kx * G.th) + G.th) * w;
+}
+
+// acc += the differential of half_moments along a derivative x: m0 x plus the
+// change of m0 and of the cut's terms
+template <typename R, int D, int NM>
+__device__ __forceinline__ void add_dhalf(const Gas<R, D>& G, const Range<R, NM>& H, R Kx, const R* x, const Var<R>& h,
+                                          R* acc)
+{
+    const R z = H.k * h.a - H.hk * h.t;  // rho d m0
+    const R tk = G.th * H.k;
+    acc[0] += H.m[0] * x[0];
+    acc[0] += z;
+    acc[1] += H.m[0] * x[1];
+    acc[1] += tk * h.r;
+    acc[1] += ((R)0.5 * H.k) * h.t;
+    if (D == 2) {
+        acc[2] += H.m[0] * x[2];
+        acc[2] += G.V * z;
+    }
+    R e = acc[D + 1];
+    e += H.m[0] * x[D + 1];
+    e += ((R)0.5 * (G.V * G.V + Kx * G.th)) * z;
+    e += tk * h.a;
+    e += ((R)0.5 * G.U * tk) * h.r;
+    acc[D + 1] = e;
 }
 
 // d(rho m_n) along a derivative, and s times it added to acc

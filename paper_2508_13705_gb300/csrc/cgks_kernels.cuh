@@ -860,7 +860,7 @@ __device__ __forceinline__ void flux_point(const Mesh& g, int dir, int na, int n
             // states carry: the face means, stencil sums and branch thresholds
             // that use sigma are FP64), the positivity test and the moments
             const Gas<R, D> Gs = gas_of<R, D>(ws, gm1);
-            const R q = rsqrt(Gs.th);
+            const R q = recip_sqrt(Gs.th);
             pz[side] = Gs.p; mn[side] = Gs.U * q; mt[side] = Gs.V * q;
             ok &= Gs.rho > (R)0 && Gs.p > (R)0;
             // kinetic weighting (Eq. 2.7): this side's half-range integrals
@@ -880,16 +880,16 @@ __device__ __forceinline__ void flux_point(const Mesh& g, int dir, int na, int n
                     dW[v] = d0[v] - e1[v];
                     lin &= fabs(dW[v]) <= (R)2.5e-4 * sc;
                 }
-                if (lin) add_dmoments_u<0>(Gs, Hs, Kx, var_of<R, D>(Gs, gm1, dW), PF ? Dl : Q0);
+                if (lin) add_dhalf(Gs, Hs, Kx, dW, var_of<R, D>(Gs, gm1, dW), PF ? Dl : Q0);
             }
             R t[4];
             if (!(BULK32 && lin && !PF)) {
-                moments<0>(Gs, Hs, Kx, t);
+                half_moments(Gs, Hs, ws, t);
 #pragma unroll
                 for (int v = 0; v < NV; ++v) Q0[v] += t[v];
             }
             if (hgks) {
-                moments<1>(Gs, Hs, Kx, t);
+                half_flux(Gs, Hs, ws, Kx, t);
 #pragma unroll
                 for (int v = 0; v < NV; ++v) T5[v] += t[v];
             }
@@ -898,7 +898,7 @@ __device__ __forceinline__ void flux_point(const Mesh& g, int dir, int na, int n
             // and with the flux's u
             auto fold = [&](int q, const R* dv) {
                 const Var<R> h = var_of<R, D>(Gs, gm1, dv);
-                add_dmoments_u<0>(Gs, Hs, Kx, h, dQ[q]);
+                add_dhalf(Gs, Hs, Kx, dv, h, dQ[q]);
                 if constexpr (hgks) {
                     if (q == 0) {
                         add_dmoments_u<1>(Gs, Hs, Kx, h, S1h);

@@ -290,7 +290,7 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // per-mesh slab layout
 struct Layout {
-    size_t S, F, ACC, sigx, sigy, FR[2], FO[2], SP[2], AT[2], TD[2], scal, total;
+    size_t S, F, ACC, sigx, sigy, FR[2], FO[2], AT[2], TD[2], scal, total;
 };
 
 Layout layout(int dim, int M, size_t rs, int nx, int ny)
@@ -311,8 +311,8 @@ Layout layout(int dim, int M, size_t rs, int nx, int ny)
         int na = d == 0 ? nx : ny, nb = d == 0 ? ny : nx;
         bool on = dim == 2 || d == 0;
         L.FR[d] = o; o = align256(o + (on ? (size_t)fr_nrow(d, na, nb) * M * 24 * rs : 0));
-        L.FO[d] = o; o = align256(o + (on ? (size_t)nb * (na + 1) * M * 16 * rs : 0));
-        L.SP[d] = o; o = align256(o + (on ? (size_t)nb * (na + 1) * M * 8 : 0));
+        // 2-D: two interface states per point and two flux sums per face; 1-D: four quantities
+        L.FO[d] = o; o = align256(o + (on ? (size_t)nb * (na + 1) * (2 * M + 2) * 4 * rs : 0));
         L.AT[d] = o; o = align256(o + (on && dim == 2 ? (size_t)(nb + 2) * (na + 6) * rs : 0));
         // FP32 bulk: each cell's hi and its tangential differences, for the flux
         L.TD[d] = o; o = align256(o + (on && dim == 2 && rs == 4 ? (size_t)(nb + 2) * (na + 6) * 12 * rs : 0));
@@ -413,7 +413,6 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
         for (int d = 0; d < 2; ++d) {
             g.FR[d] = m0 + L[k].FR[d];
             g.FO[d] = m0 + L[k].FO[d];
-            g.SP[d] = (double*)(m0 + L[k].SP[d]);
             g.AT[d] = m0 + L[k].AT[d];
             g.TD[d] = m0 + L[k].TD[d];
         }
@@ -1167,12 +1166,12 @@ extern "C" int cgks_step_1d_noalloc(const cgks_params* p, int nx, double x0, dou
     if ((r = noalloc_setup(dev))) return r;
     cudaStream_t st = (cudaStream_t)stream;
     size_t rs = p->precision == CGKS_FP64 ? 8 : 4;
-    // carve the array: S1, ACC, sigma (new), FR, FO, SP, scalars, descriptor, offsets
+    // carve the array: S1, ACC, sigma (new), FR, FO, scalars, descriptor, offsets
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o = align256(o + bytes); return at; };
     size_t oS1 = take(6 * (size_t)nx * 8), oACC = take(6 * (size_t)nx * 8), oSN = take((size_t)(nx + 1) * 8);
     size_t oFR = take((size_t)fr_nrow(0, nx, 1) * 24 * rs), oFO = take((size_t)(nx + 1) * 16 * rs);
-    size_t oSP = take((size_t)(nx + 1) * 8), oSC = take(512), oM = take(sizeof(Mesh));
+    size_t oSC = take(512), oM = take(sizeof(Mesh));
     size_t oOF = take(W_COUNT * 2 * sizeof(long long));
     size_t oF = take(rs == 4 ? 2 * 9 * (size_t)nx * 4 : 0);  // FP32-bulk float planes and low parts
     if (o > CGKS_NOALLOC_SCRATCH_BYTES) return CGKS_EINVAL;
@@ -1205,7 +1204,7 @@ extern "C" int cgks_step_1d_noalloc(const cgks_params* p, int nx, double x0, dou
     g.ACC = (double*)(base + oACC);
     g.sig_x = sigma_out;
     g.sig_xn = (double*)(base + oSN);
-    g.FR[0] = base + oFR; g.FO[0] = base + oFO; g.SP[0] = (double*)(base + oSP);
+    g.FR[0] = base + oFR; g.FO[0] = base + oFO;
     unsigned char* sc = base + oSC;
     g.dt = (double*)sc; g.t = (double*)(sc + 8); g.status = (unsigned*)(sc + 16);
     g.bad = (long long*)(sc + 24); g.smax = (unsigned long long*)(sc + 32);

@@ -93,7 +93,6 @@ struct Mesh {
     void* AT[2];                    // tangential r5 DFF per cell (R typed)
     void* TD[2];                    // FP32 bulk: hi(a, b), hi(a, b-1) - hi(a, b), hi(a, b+1) - hi(a, b)
                                     // of each cell, local frame, [12] floats
-    double* SP[2];                  // sigma per face Gauss point
     double* dt;                     // device scalar (this mesh's step)
     float* dtf;                     // the same in FP32: [0] float(dt), [1] float(dt - [0])
     double* t;                      // device scalar (simulated time)
@@ -384,6 +383,11 @@ __device__ __forceinline__ void ld2(const float* p, float v[2])
 {
     const float2 q = *reinterpret_cast<const float2*>(p);
     v[0] = q.x; v[1] = q.y;
+}
+__device__ __forceinline__ void st2(float* p, const float v[2]) { *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]); }
+__device__ __forceinline__ void st2(double* p, const double v[2])
+{
+    *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
 }
 __device__ __forceinline__ void ld2(const double* p, double v[2])
 {

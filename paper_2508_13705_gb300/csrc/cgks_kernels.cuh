@@ -14,9 +14,11 @@
 //                                     one plane per Gauss line, so that the lanes of
 //                                     a warp, which cover consecutive faces, read a
 //                                     line's points as consecutive 16-byte groups
-//   FO  [4][M][nb][na+1][4]           per-point stage outputs (local frame),
-//                                     one plane per output quantity and line
-//   SP  [nb][na+1][M]                 sigma per face Gauss point (Eq. 3.2)
+//   FO  [NO][M][nb][na+1][4], [NO][nb][na+1][4]   stage outputs (local frame; NO = 2
+//                                     quantities of each kind in stage 1, 1 in stage 2):
+//                                     interface states per point, one plane per quantity
+//                                     and line, then the Gauss sums of the fluxes per face.
+//                                     1-D: [4][nx+1][4]
 //   AT  [nb+2][na+6]                  tangential r5 DFF of each cell (Step 3)
 //   TD  [nb+2][na+6][12]              FP32 bulk: the cell's hi (the base of the face
 //                                     states) and its tangential differences hi(a, b-1) -
@@ -82,7 +84,7 @@ __device__ __forceinline__ double lsigT(const Mesh& g, const double* sx, const d
 // SoA state planes with unit stride.
 //   cell_idx: a in [-3, na+2], b in [-1, nb]   (AT, TD)
 //   fr_row:   bb = b + 1 in [0, nb+1], f in [0, na]   (FR)
-//   pt_idx:   b in [0, nb), f in [0, na]       (FO, SP)
+//   pt_idx:   b in [0, nb), f in [0, na]       (FO)
 __device__ __forceinline__ long long cell_idx(int dir, int na, int nb, int a, int b)
 {
     return dir == 0 ? (long long)(b + 1) * (na + 6) + (a + 3) : (long long)(a + 3) * (nb + 2) + (b + 1);
@@ -112,6 +114,12 @@ __device__ __forceinline__ long long fr_off(long long nrow, int M, int side, int
 __device__ __forceinline__ long long fo_off(long long nf, int M, int q, int l, long long face)
 {
     return ((long long)(q * M + l) * nf + face) * 4;
+}
+
+// sums over a face's points, after the NO quantities of the points
+__device__ __forceinline__ long long fs_off(long long nf, int M, int NO, int q, long long face)
+{
+    return ((long long)NO * M * nf + q * nf + face) * 4;
 }
 
 __device__ __forceinline__ void flag_bad(const Mesh& g, long long idx)
@@ -666,7 +674,7 @@ template <int M> struct FluxStrip {
 // Values of one warp in shared memory: the ring of W and W_n of both sides; the
 // tangential derivatives of the step; two slots of what only the step's own
 // points read: W_nn, and the bases of the face (TD of its right cell, FP32
-// bulk) with the tangential DFF of its two cells.
+// bulk) with the tangential DFF of its two cells; the step's sigma.
 template <int M, typename R>
 struct FluxShared {
     static constexpr int FW = FluxStrip<M>::FW, RING = FluxStrip<M>::RING;
@@ -750,6 +758,8 @@ template <int M, typename R>
 struct StripPoint {
     using L = FluxShared<M, R>;
     const R* s;       // the warp's values
+    R* FO;
+    long long nf;     // faces of the direction
     int slot, own_q;  // slot of the step, ring position of the point's own segment
     int x, l;
     __device__ __forceinline__ void own(int side, int nd, R* v) const
@@ -762,7 +772,96 @@ struct StripPoint {
     {
         ld4(s + L::tang + (((side * 3 + q) * M + l) * L::FW + x) * 4, v);
     }
+    // interface states to global memory; fluxes and sigma are left to the face's sums
+    template <int STAGE>
+    __device__ __forceinline__ void put(const R o[4][4], long long face, R) const
+    {
+#pragma unroll
+        for (int q = 0; q < (STAGE == 1 ? 2 : 1); ++q) st4(FO + fo_off(nf, M, q, l, face), o[2 + q]);
+    }
 };
+
+// A face's Gauss sums of its points' fluxes and the mean of their sigma, over
+// the M lanes of the face (all lanes of the warp take part).  Each lane ends up
+// with a share of the sums and writes it: the update reads one value per face
+// where it read M: 1024^2, order 9, FP32, the updates took 307 + 160 us, now 199 +
+// 150 (with three blocks of 256 threads per SM), the fluxes 395 + 354, now 418 +
+// 364; at 2048^2, order 5, 905 + 413 -> 508 + 393 and 770 + 703 -> 821 + 721.
+__device__ __forceinline__ float swap_lane(float v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+__device__ __forceinline__ double swap_lane(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+
+template <int M, int NO, typename R>
+__device__ __forceinline__ void face_sums(R (&o)[4][4], R* FS, long long nf, long long face, int l, bool on)
+{
+    const auto& T = Tab<R>::get(M - 2);
+    R w = T.gw[0];  // the lane's weight, mirrored lines alike
+    if (M == 3 ? l == 1 : (M == 4 && (l == 1 || l == 2))) w = T.gw[1];
+#pragma unroll
+    for (int q = 0; q < NO; ++q)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) o[q][v] *= w;
+    if (M == 3) {
+        const int base = (threadIdx.x & 31) - l;
+#pragma unroll
+        for (int q = 0; q < NO; ++q) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                R s = __shfl_sync(0xffffffffu, o[q][v], base);
+                s += __shfl_sync(0xffffffffu, o[q][v], base + 1);
+                s += __shfl_sync(0xffffffffu, o[q][v], base + 2);
+                o[q][v] = s;
+            }
+            if (on && l == q) st4(FS + (q * nf + face) * 4, o[q]);
+        }
+    } else if (NO == 2) {
+        // lines l and l ^ M/2 split the two quantities ...
+        const bool up = (l & (M / 2)) != 0;
+        R s[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const R give = up ? o[0][v] : o[NO - 1][v], keep = up ? o[NO - 1][v] : o[0][v];
+            s[v] = keep + swap_lane(give, M / 2);
+        }
+        R* p = FS + ((up ? nf : 0) + face) * 4;
+        if (M == 2) {
+            if (on) st4(p, s);
+        } else {
+            // ... and l and l ^ 1 the variables
+            const bool odd = l & 1;
+            R r[2];
+#pragma unroll
+            for (int v = 0; v < 2; ++v) r[v] = (odd ? s[2 + v] : s[v]) + swap_lane(odd ? s[v] : s[2 + v], 1);
+            if (on) st2(p + (odd ? 2 : 0), r);
+        }
+    } else {
+        const bool up = (l & (M / 2)) != 0;
+        R s[2];
+#pragma unroll
+        for (int v = 0; v < 2; ++v) s[v] = (up ? o[0][2 + v] : o[0][v]) + swap_lane(up ? o[0][v] : o[0][2 + v], M / 2);
+        R* p = FS + face * 4 + (up ? 2 : 0);
+        if (M == 2) {
+            if (on) st2(p, s);
+        } else {
+            const bool odd = l & 1;
+            const R r = (odd ? s[1] : s[0]) + swap_lane(odd ? s[0] : s[1], 1);
+            if (on) p[odd ? 1 : 0] = r;
+        }
+    }
+}
+
+template <int M, typename R>
+__device__ __forceinline__ void face_sigma(R sig, double* out, int l, bool on)
+{
+    double s = (double)sig;
+    if (M == 3) {
+        const int base = (threadIdx.x & 31) - l;
+        s = __shfl_sync(0xffffffffu, s, base) + __shfl_sync(0xffffffffu, s, base + 1) + __shfl_sync(0xffffffffu, s, base + 2);
+    } else {
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        if (M == 4) s += __shfl_xor_sync(0xffffffffu, s, 2);
+    }
+    if (on && l == 0) *out = s / M;
+}
 
 // What a 1-D face reads, from global memory.
 template <typename R>
@@ -772,6 +871,17 @@ struct LinePoint {
     R h[4];
     __device__ __forceinline__ void own(int side, int nd, R* v) const { ld4(FR + fr_off(nrow, 1, side, nd, 0, row), v); }
     __device__ __forceinline__ void base(R* v) const { for (int q = 0; q < 4; ++q) v[q] = h[q]; }
+    R* FO;
+    double* sx;
+    long long nf;
+    template <int STAGE>
+    __device__ __forceinline__ void put(const R o[4][4], long long face, R sig) const
+    {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (STAGE == 1 || q % 2 == 0) st4(FO + (q * nf + face) * 4, o[q]);
+        if (STAGE == 1) sx[face] = (double)sig;
+    }
 };
 
 // One face Gauss point.  Each side's reconstructed data (Step 2 values, Step 3
@@ -784,7 +894,7 @@ struct LinePoint {
 // Dt^2 / 6.
 template <int D, int M, typename R, int STAGE, int HG, bool PF, typename Point>
 __device__ __forceinline__ void flux_point(const Mesh& g, int dir, int na, int nb, int f, int b, int l, const Point& in,
-                                           R Dt, R dt26)
+                                           R Dt, R dt26, R (&o)[4][4], R& sig)
 {
     constexpr int NV = D + 2;
     constexpr int ND = D == 2 ? 5 : 2;  // derivatives: n, nn (, t, tt, nt)
@@ -944,10 +1054,9 @@ __device__ __forceinline__ void flux_point(const Mesh& g, int dir, int na, int n
                 for (int v = 0; v < NV; ++v) qv[v] = Q0[v] - hb1[v];
             }
         }
-        double sig;
         {
             R dpz = fabs(pz[0] - pz[1]);
-            sig = (double)(dpz * recip(pz[0]) + dpz * recip(pz[1])
+            sig = (dpz * recip(pz[0]) + dpz * recip(pz[1])
                            + MeshR<R>::igamma(g) * ((mn[0] - mn[1]) * (mn[0] - mn[1]) + (mt[0] - mt[1]) * (mt[0] - mt[1])));
         }
         // equilibrium state g0 (Eq. 2.8): derivatives in the variables of its
@@ -1021,11 +1130,7 @@ __device__ __forceinline__ void flux_point(const Mesh& g, int dir, int na, int n
                 Wtt[v] += (R)4 * (ed - eh) / Dt * dS;
             }
         }
-        long long face = pt_idx(dir, na, nb, b, f);
-        long long pt = face * M + l;  // SP index
-        const long long nf = (long long)nb * (na + 1);
-        R* FO = (R*)g.FO[dir];
-        R o[4][4];
+        // stage outputs: o[0], o[1] fluxes, o[2], o[3] interface states
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             if (v >= NV) { o[0][v] = o[1][v] = o[2][v] = o[3][v] = (R)0; continue; }
@@ -1038,20 +1143,20 @@ __device__ __forceinline__ void flux_point(const Mesh& g, int dir, int na, int n
                 o[3][v] = Qv + Dt * Wt[v] + dt26 * Wtt[v];
             } else {
                 o[0][v] = (R)2 * dt26 * Ft[v];
-                o[1][v] = (R)2 * dt26 * Wtt[v];
+                o[2][v] = (R)2 * dt26 * Wtt[v];
             }
         }
         // finite outputs: 0 * x is 0 for finite x only
         R zero = (R)0;
-        constexpr int NO = STAGE == 1 ? 4 : 2;
 #pragma unroll
-        for (int q = 0; q < NO; ++q) {
+        for (int q = 0; q < 4; ++q)
+            if (STAGE == 1 || q % 2 == 0) {
 #pragma unroll
-            for (int v = 0; v < NV; ++v) zero += (R)0 * o[q][v];
-            st4(FO + fo_off(nf, M, q, l, face), o[q]);
-        }
-        if (STAGE == 1) g.SP[dir][pt] = sig;
-        if (!ok || !(zero == (R)0)) flag_bad(g, pt);
+                for (int v = 0; v < NV; ++v) zero += (R)0 * o[q][v];
+            }
+        const long long face = pt_idx(dir, na, nb, b, f);
+        in.template put<STAGE>(o, face, sig);
+        if (!ok || !(zero == (R)0)) flag_bad(g, face * M + l);
     }
 }
 
@@ -1074,6 +1179,9 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
         in.FR = (const R*)g.FR[0];
         in.nrow = fr_nrow(0, na, 1);
         in.row = fr_row(0, na, 1, 1, f);
+        in.FO = (R*)g.FO[0];
+        in.sx = g.sig_xn;
+        in.nf = na + 1;
         if (sizeof(R) == 4) {
             const R* SF = state_planes<R>(g, STAGE == 1 ? 0 : 1);
             const double tb = stage_time(g, STAGE);
@@ -1081,7 +1189,8 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
             for (int v = 0; v < 3; ++v) in.h[v] = cell<1, 1, R, true>(g, SF, 0, v, 0, f, 0, tb);
             in.h[3] = (R)0;
         }
-        flux_point<1, 1, R, STAGE, HG, PF>(g, 0, na, 1, f, 0, 0, in, Dt, Dt * Dt / (R)6);
+        R o[4][4], sig;
+        flux_point<1, 1, R, STAGE, HG, PF>(g, 0, na, 1, f, 0, 0, in, Dt, Dt * Dt / (R)6, o, sig);
     }
 }
 
@@ -1118,6 +1227,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flu
         const R Dt = MeshR<R>::dt(g);
         const R dt26 = Dt * Dt / (R)6, iht = (R)1 / (R)(dir == 0 ? g.dy : g.dx);
         const int f = dir == 0 ? outer * FW + x : outer;
+        const long long nf = (long long)nb * (na + 1);
         // this lane's sources of the next row (dir 0) or block of rows (dir 1) of
         // face states, advanced by `step` values a row or block; its copies stop at
         // row bb = nb + 1
@@ -1209,15 +1319,24 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flu
             }
             copy_commit();
             const int b = dir == 0 ? k : k * FW + x;
-            if (mine && b < nb) {
+            const bool point = mine && b < nb;
+            const long long face = pt_idx(dir, na, nb, point ? b : 0, point ? f : 0);
+            R o[4][4] = {}, sig = (R)0;
+            if (point) {
                 StripPoint<M, R> in;
                 in.s = sm;
+                in.FO = (R*)g.FO[dir];
+                in.nf = nf;
                 in.slot = slot;
                 in.own_q = dir == 0 ? r1 * FW + x : (x + 1 < FW ? r0 * FW + x + 1 : r1 * FW);
                 in.x = x;
                 in.l = l;
-                flux_point<2, M, R, STAGE, HG, PF>(g, dir, na, nb, f, b, l, in, Dt, dt26);
+                flux_point<2, M, R, STAGE, HG, PF>(g, dir, na, nb, f, b, l, in, Dt, dt26, o, sig);
             }
+            __syncwarp();
+            constexpr int NO = STAGE == 1 ? 2 : 1;
+            face_sums<M, NO>(o, (R*)g.FO[dir] + fs_off(nf, M, NO, 0, 0), nf, face, l, point);
+            if (STAGE == 1) face_sigma<M>(sig, (dir == 0 ? g.sig_xn : g.sig_yn) + face, l, point);
             r0 = r1;
         }
     }
@@ -1240,8 +1359,10 @@ __device__ __forceinline__ double exact_diff(float r, float l)
 // Stage 1 writes W* (S1) and the accumulator; stage 2 writes state n+1 (S0).
 // FP32-bulk form: the float planes (F1 / F0) receive everything the next stage
 // reads, the FP64 planes the cell averages of state n+1 (W* lives in F1 only).
+template <typename R> __device__ __forceinline__ void swap12(R* v) { const R z = v[1]; v[1] = v[2]; v[2] = z; }
+
 template <int M, typename R, int STAGE, bool ONE>
-__global__ void __launch_bounds__(256) k_update2(Work w)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_update2(Work w)
 {
     constexpr bool BULK32 = sizeof(R) == 4;
     for (long long gi = blockIdx.x * (long long)blockDim.x + threadIdx.x; gi < w.total;
@@ -1264,9 +1385,8 @@ __global__ void __launch_bounds__(256) k_update2(Work w)
         R* accs = (R*)(g.ACC + 4 * P);
         float* outf = STAGE == 1 ? g.F1 : g.F0;
         const auto& TR = Tab<R>::get(g.oi);
-        // Conserved quantities: the Gauss sum over a face's points is formed
-        // per face, in the bulk precision and in the same order by both cells
-        // of the face (bitwise alike), and the difference of a cell's two
+        // Conserved quantities: the Gauss sum over a face's points was formed
+        // per face, in the bulk precision, and the difference of a cell's two
         // face sums is taken exactly (exact_diff) into the FP64 averages, so
         // the updates telescope over the mesh and the totals change only by
         // the boundary fluxes and FP64 rounding.  Slopes use bulk differences.
@@ -1282,11 +1402,22 @@ __global__ void __launch_bounds__(256) k_update2(Work w)
         if (BULK32 && STAGE == 1) {
             const float* SF = g.F0;
             const double tb = *g.tn;
+            const bool nx = i + 1 < g.nx, ny = j + 1 < g.ny;
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 h0[v] = (R)SF[v * P + c];
-                hxn[v] = (R)cell<2, M, float, true>(g, SF, 0, v, 0, i + 1, j, tb);
-                hyn[v] = (R)cell<2, M, float, true>(g, SF, 0, v, 0, i, j + 1, tb);
+                if (nx) hxn[v] = (R)SF[v * P + c + 1];
+                if (ny) hyn[v] = (R)SF[v * P + c + g.nx];
+            }
+            if (!nx) {
+                const CellMap m = cell_map<true>(g, i + 1, j, tb);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) hxn[v] = (R)mapped<2, M, float, true>(g, SF, m, 0, v, 0);
+            }
+            if (!ny) {
+                const CellMap m = cell_map<true>(g, i, j + 1, tb);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) hyn[v] = (R)mapped<2, M, float, true>(g, SF, m, 0, v, 0);
             }
             const double gm1d = g.gamma - 1.0;
             const ff gm1 = {(float)gm1d, (float)(gm1d - (double)(float)gm1d)};
@@ -1306,39 +1437,44 @@ __global__ void __launch_bounds__(256) k_update2(Work w)
             const int yl[4] = {0, 2, 1, 3};
             for (int v = 0; v < 4; ++v) By[v] = ff_add(f1[yl[v]], ff_neg(f0[yl[v]]));
         }
-        R gxr0[4] = {0, 0, 0, 0}, gxl0[4] = {0, 0, 0, 0}, gyr0[4] = {0, 0, 0, 0}, gyl0[4] = {0, 0, 0, 0};
-        R gxr1[4] = {0, 0, 0, 0}, gxl1[4] = {0, 0, 0, 0}, gyr1[4] = {0, 0, 0, 0}, gyl1[4] = {0, 0, 0, 0};
+        // the faces' flux sums (y-faces: local frame (rho, m_y, m_x, E) to global order)
+        constexpr int NO = STAGE == 1 ? 2 : 1;
+        R gxr[NO][4], gxl[NO][4], gyr[NO][4], gyl[NO][4];
+#pragma unroll
+        for (int q = 0; q < NO; ++q) {
+            ld4(FX + fs_off(nfx, M, NO, q, fxl + 1), gxr[q]);
+            ld4(FX + fs_off(nfx, M, NO, q, fxl), gxl[q]);
+            ld4(FY + fs_off(nfy, M, NO, q, fyl + g.nx), gyr[q]);
+            ld4(FY + fs_off(nfy, M, NO, q, fyl), gyl[q]);
+            swap12(gyr[q]);
+            swap12(gyl[q]);
+        }
+        double W0[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) W0[v] = STAGE == 1 ? g.S0[v * P + c] : g.ACC[v * P + c];
         R sx[4] = {0, 0, 0, 0}, sy[4] = {0, 0, 0, 0};
 #pragma unroll 1
         for (int l = 0; l < M; ++l) {
             R wl = TR.gw[l];
             R a[4], bq[4], cq[4], dq[4];
-            // stage 1: o0 = F(dt/2), o1 = dt F + dt^2/6 F_t, o2 = W(dt/2), o3 = W0 + dt W_t + dt^2/6 W_tt
-            // stage 2: o0 = dt^2/3 F_t*, o1 = dt^2/3 W_tt*
+            // stage 1: W(dt/2), W0 + dt W_t + dt^2/6 W_tt; stage 2: dt^2/3 W_tt*
 #pragma unroll
-            for (int q = 0; q < (STAGE == 1 ? 4 : 2); ++q) {
+            for (int q = 0; q < NO; ++q) {
                 ld4(FX + fo_off(nfx, M, q, l, fxl + 1), a);
                 ld4(FX + fo_off(nfx, M, q, l, fxl), bq);
                 ld4(FY + fo_off(nfy, M, q, l, fyl + g.nx), cq);
                 ld4(FY + fo_off(nfy, M, q, l, fyl), dq);
-                // y-faces: local frame (rho, m_y, m_x, E) to global order
-                { const R z = cq[1]; cq[1] = cq[2]; cq[2] = z; }
-                { const R z = dq[1]; dq[1] = dq[2]; dq[2] = z; }
+                swap12(cq);
+                swap12(dq);
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
                     R dx_ = a[v] - bq[v];
                     R dy_ = cq[v] - dq[v];
-                    if (BULK32 && STAGE == 1 && q >= 2) {  // interface states over the bases' hi
+                    if (BULK32 && STAGE == 1) {  // interface states over the bases' hi
                         dx_ += hxn[v] - h0[v];
                         dy_ += hyn[v] - h0[v];
                     }
                     if (q == 0) {
-                        gxr0[v] += wl * a[v]; gxl0[v] += wl * bq[v];
-                        gyr0[v] += wl * cq[v]; gyl0[v] += wl * dq[v];
-                    } else if (STAGE == 1 && q == 1) {
-                        gxr1[v] += wl * a[v]; gxl1[v] += wl * bq[v];
-                        gyr1[v] += wl * cq[v]; gyl1[v] += wl * dq[v];
-                    } else if ((STAGE == 1 && q == 2) || (STAGE == 2 && q == 1)) {
                         R lx = dx_ * ridx, ly = dy_ * ridy;
                         if (STAGE == 2) {
                             lx += accs[(4 * l + v) * P + c];
@@ -1353,7 +1489,7 @@ __global__ void __launch_bounds__(256) k_update2(Work w)
                         }
                         sx[v] += wl * lx;
                         sy[v] += wl * ly;
-                    } else {  // stage 1, q == 3: line-slope part of the accumulator
+                    } else {  // the line-slope part of the accumulator
                         accs[(4 * l + v) * P + c] = dx_ * ridx;
                         accs[(4 * M + 4 * l + v) * P + c] = dy_ * ridy;
                     }
@@ -1369,27 +1505,36 @@ __global__ void __launch_bounds__(256) k_update2(Work w)
                 // the bases' flux differences times dt/2 or dt, over dx and dy;
                 // one conversion to FP64 per quantity (the FP64 pipe is narrow)
                 const ff ix = {g.idxf, g.idxlo}, iy = {g.idyf, g.idylo};
-                ff tx = ff_two_sum((float)gxr0[v], -(float)gxl0[v]), ty = ff_two_sum((float)gyr0[v], -(float)gyl0[v]);
+                ff tx = ff_two_sum((float)gxr[0][v], -(float)gxl[0][v]), ty = ff_two_sum((float)gyr[0][v], -(float)gyl[0][v]);
                 if (STAGE == 1) {
                     const ff hdt = {0.5f * g.dtf[0], 0.5f * g.dtf[1]}, fdt = {g.dtf[0], g.dtf[1]};
                     tx = ff_add(tx, ff_mul(hdt, Bx[v]));
                     ty = ff_add(ty, ff_mul(hdt, By[v]));
-                    ff ax = ff_add(ff_two_sum((float)gxr1[v], -(float)gxl1[v]), ff_mul(fdt, Bx[v]));
-                    ff ay = ff_add(ff_two_sum((float)gyr1[v], -(float)gyl1[v]), ff_mul(fdt, By[v]));
-                    double W = g.S0[v * P + c];
-                    Wn = W - ff_val(ff_add(ff_mul(tx, ix), ff_mul(ty, iy)));  // Eq. 2.21
-                    g.ACC[v * P + c] = W - ff_val(ff_add(ff_mul(ax, ix), ff_mul(ay, iy)));
+                    ff ax = ff_add(ff_two_sum((float)gxr[NO - 1][v], -(float)gxl[NO - 1][v]), ff_mul(fdt, Bx[v]));
+                    ff ay = ff_add(ff_two_sum((float)gyr[NO - 1][v], -(float)gyl[NO - 1][v]), ff_mul(fdt, By[v]));
+                    g.ACC[v * P + c] = W0[v] - ff_val(ff_add(ff_mul(ax, ix), ff_mul(ay, iy)));
+                    // Eq. 2.21: W*, held as hi + lo only, from W's hi + lo in float-float
+                    // (the FP64 pipe was half busy with conversions)
+                    const ff ws = ff_add({(float)h0[v], g.F0[(12 + 8 * M + v) * P + c]},
+                                         ff_neg(ff_add(ff_mul(tx, ix), ff_mul(ty, iy))));
+                    bad |= !isfinite(ws.hi);
+                    outf[v * P + c] = ws.hi;
+                    outf[(12 + 8 * M + v) * P + c] = ws.lo;
+                    outf[(4 + v) * P + c] = (float)sx[v];  // cell slopes: Gauss sum of the line slopes
+                    outf[(8 + v) * P + c] = (float)sy[v];
+                    continue;
                 } else {
-                    Wn = g.ACC[v * P + c] - ff_val(ff_add(ff_mul(tx, ix), ff_mul(ty, iy)));  // Eq. 2.22-2.23
+                    Wn = W0[v] - ff_val(ff_add(ff_mul(tx, ix), ff_mul(ty, iy)));  // Eq. 2.22-2.23
                 }
             } else {
-                const double dx0 = exact_diff(gxr0[v], gxl0[v]), dy0 = exact_diff(gyr0[v], gyl0[v]);
+                const double dx0 = exact_diff(gxr[0][v], gxl[0][v]), dy0 = exact_diff(gyr[0][v], gyl[0][v]);
                 if (STAGE == 1) {
-                    double W = g.S0[v * P + c];
+                    const double W = W0[v];
                     Wn = W - dx0 * idx - dy0 * idy;  // Eq. 2.21
-                    g.ACC[v * P + c] = W - exact_diff(gxr1[v], gxl1[v]) * idx - exact_diff(gyr1[v], gyl1[v]) * idy;
+                    g.ACC[v * P + c] = W - exact_diff(gxr[NO - 1][v], gxl[NO - 1][v]) * idx
+                                     - exact_diff(gyr[NO - 1][v], gyl[NO - 1][v]) * idy;
                 } else {
-                    Wn = g.ACC[v * P + c] - dx0 * idx - dy0 * idy;  // Eq. 2.22-2.23
+                    Wn = W0[v] - dx0 * idx - dy0 * idy;  // Eq. 2.22-2.23
                 }
             }
             // the FP32-bulk stage 2 reads W* from the float planes only
@@ -1406,27 +1551,8 @@ __global__ void __launch_bounds__(256) k_update2(Work w)
                 out[(8 + v) * P + c] = (double)sy[v];
             }
         }
-        // face sigma of this step (Eq. 3.1): mean over the face's Gauss points
-        if (STAGE == 1) {
-            const double* SX = g.SP[0];
-            const double* SY = g.SP[1];
-            double s = 0;
-            for (int l = 0; l < M; ++l) s += SX[((long long)j * (g.nx + 1) + i) * M + l];
-            g.sig_xn[(long long)j * (g.nx + 1) + i] = s / M;
-            if (i == g.nx - 1) {
-                s = 0;
-                for (int l = 0; l < M; ++l) s += SX[((long long)j * (g.nx + 1) + g.nx) * M + l];
-                g.sig_xn[(long long)j * (g.nx + 1) + g.nx] = s / M;
-            }
-            s = 0;
-            for (int l = 0; l < M; ++l) s += SY[((long long)j * g.nx + i) * M + l];
-            g.sig_yn[(long long)j * g.nx + i] = s / M;
-            if (j == g.ny - 1) {
-                s = 0;
-                for (int l = 0; l < M; ++l) s += SY[((long long)g.ny * g.nx + i) * M + l];
-                g.sig_yn[(long long)g.ny * g.nx + i] = s / M;
-            }
-        } else {
+        // the step's face sigma (Eq. 3.1) for the next step
+        if (STAGE == 2) {
             g.sig_x[(long long)j * (g.nx + 1) + i] = g.sig_xn[(long long)j * (g.nx + 1) + i];
             if (i == g.nx - 1) g.sig_x[(long long)j * (g.nx + 1) + g.nx] = g.sig_xn[(long long)j * (g.nx + 1) + g.nx];
             g.sig_y[(long long)j * g.nx + i] = g.sig_yn[(long long)j * g.nx + i];
@@ -1485,7 +1611,7 @@ __global__ void __launch_bounds__(256) k_update1(Work w)
                 g.ACC[(3 + v) * P + i] = (((double)xr(12 + v) - (double)xl(12 + v)) + hd[v]) * idx;
             } else {
                 Wn = g.ACC[v * P + i] - ((double)xr(v) - (double)xl(v)) * idx;
-                Sn = g.ACC[(3 + v) * P + i] + ((double)xr(4 + v) - (double)xl(4 + v)) * idx;
+                Sn = g.ACC[(3 + v) * P + i] + ((double)xr(8 + v) - (double)xl(8 + v)) * idx;
                 g.S0[v * P + i] = Wn;
             }
             if (BULK32) {
@@ -1499,10 +1625,7 @@ __global__ void __launch_bounds__(256) k_update1(Work w)
             }
             bad |= !isfinite(Wn);
         }
-        if (STAGE == 1) {
-            g.sig_xn[i] = g.SP[0][i];
-            if (i == g.nx - 1) g.sig_xn[g.nx] = g.SP[0][g.nx];
-        } else {
+        if (STAGE == 2) {
             g.sig_x[i] = g.sig_xn[i];
             if (i == g.nx - 1) g.sig_x[g.nx] = g.sig_xn[g.nx];
         }

@@ -108,6 +108,11 @@ struct cgks_batch {
     int n = 0, dim = 2, M = 1, nvar = 4, nplanes = 0, nacc = 0;
     size_t rsize = 8;
     cudaStream_t stream = nullptr;
+    // capture of the step's graph branches (2-D, made when needed): a second stream
+    // and the events between the two; nothing runs on it outside the graphs
+    cudaStream_t side = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+    double* host_smax = nullptr;  // mapped host memory: the CFL maximum for cgks_compute_dt
     std::vector<Mesh> host;      // host copy of the descriptors
     Mesh* dmesh = nullptr;       // device descriptors
     long long* doff = nullptr;   // device prefix arrays [W_COUNT][n+1]
@@ -165,7 +170,7 @@ long long items(const Kfns& k, int kind, int dim, int M, int nx, int ny)
     case W_NORMAL: return dim == 2 ? 0 : nx + 2;
     case W_FLUX: return dim == 2 ? flux_steps(M, nx, ny) : nx + 1;
     case W_CELLS: return (long long)nx * ny;
-    default: return dim == 2 ? (long long)(nx + 1) * ny + (long long)(ny + 1) * nx : nx + 1;
+    default: return (long long)nx * ((ny + kSigRows - 1) / kSigRows);
     }
 }
 
@@ -175,7 +180,24 @@ size_t dyn_smem(const cgks_batch* b, int kind, int threads)
     return b->dim == 2 && kind == W_FLUX ? (size_t)(threads / 32) * b->k.flux_warp_bytes : 0;
 }
 
-int launch(cgks_batch* b, const void* fn, int kind, int gi, int stage, bool has_stage)
+// Launch fn; dep: as a programmatic dependent of the kernel before it in the
+// stream (which, like fn, waits for its own predecessor: grid_wait).
+cudaError_t launch_kernel(const void* fn, int grid, int threads, void** args, size_t smem, cudaStream_t st, bool dep)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = dep ? 1 : 0;
+    return cudaLaunchKernelExC(&c, fn, args);
+}
+
+int launch(cgks_batch* b, const void* fn, int kind, int gi, int stage, bool has_stage, bool dep = false)
 {
     Work w = work_of(b, kind);
     if (w.total == 0) return CGKS_OK;
@@ -187,46 +209,81 @@ int launch(cgks_batch* b, const void* fn, int kind, int gi, int stage, bool has_
     if (grid < 1) grid = 1;
     void* args2[] = {&w, &stage};
     void* args1[] = {&w};
-    CK(cudaLaunchKernel(fn, dim3(grid), dim3(threads), has_stage ? args2 : args1, dyn_smem(b, kind, threads), b->stream));
+    CK(launch_kernel(fn, grid, threads, has_stage ? args2 : args1, dyn_smem(b, kind, threads), b->stream, dep));
     return CGKS_OK;
 }
 
 // One launch of the 2-D Steps 1-2 of direction dir (tiles as work items).
-int launch_recon(cgks_batch* b, int dir, int stage)
+int launch_recon(cgks_batch* b, int dir, int stage, cudaStream_t st, bool dep = false)
 {
     Work w = work_of(b, dir == 0 ? W_TILE0 : W_TILE1);
     if (w.total == 0) return CGKS_OK;
     const int grid = (int)w.total;  // a block per tile
     void* args[] = {&w, &stage};
-    CK(cudaLaunchKernel((const void*)b->k.recon[dir], dim3(grid), dim3(b->threads[dir]), args,
-                        (size_t)b->k.recon_bytes[dir], b->stream));
+    CK(launch_kernel((const void*)b->k.recon[dir], grid, b->threads[dir], args, (size_t)b->k.recon_bytes[dir], st, dep));
     return CGKS_OK;
 }
 
+// The CFL reduction over all meshes; mode as k_cfl's.
+int launch_cfl(cgks_batch* b, int mode)
+{
+    Work w = work_of(b, W_CELLS);
+    const int threads = b->threads[6];
+    const int grid = (int)std::max<long long>(1, std::min<long long>((w.total + threads - 1) / threads, (long long)b->grid[6]));
+    double* out = b->host_smax;
+    void* args[] = {&w, &out};
+    CK(launch_kernel((const void*)b->k.cfl[mode], grid, threads, args, 0, b->stream, false));
+    return CGKS_OK;
+}
+
+// Whether the step's kernels overlap: as programmatic dependents, and in 2-D
+// Steps 1-2 of the two directions side by side (a branch of the graph on the
+// second stream), where a mesh fills neither launch.  Up to 32 tiles per SM: 80
+// cells 1-D 78 -> 56 us a step, 47 x 33 66 -> 49, 400^2 454 -> 425 us, 960 x 240
+// FP64 12.2 -> 11.7 ms.  Beyond, side by side the launches only share the caches
+// (1024^2 1785 -> 1797 us, 2048^2 order 5 4.09 -> 4.24 ms), and early blocks of the
+// next kernel take room from the last of this one (1024^2 1946 us).
+bool overlap(const cgks_batch* b)
+{
+    return b->dim == 1 || b->off[(size_t)W_TILE0 * (b->n + 1) + b->n] <= 32LL * b->nsm;
+}
+
+// One stage, captured into a step's graph.
 int enqueue_stage(cgks_batch* b, int stage)
 {
     int r;
-    if (b->dim == 2) {
-        if ((r = launch_recon(b, 0, stage))) return r;
-        if ((r = launch_recon(b, 1, stage))) return r;
-    } else if ((r = launch(b, (const void*)b->k.normal, W_NORMAL, 1, stage, true))) {
+    const bool over = overlap(b);
+    if (b->dim == 2 && !over) {
+        if ((r = launch_recon(b, 0, stage, b->stream))) return r;
+        if ((r = launch_recon(b, 1, stage, b->stream))) return r;
+    } else if (b->dim == 2) {
+        CK(cudaEventRecord(b->fork, b->stream));
+        CK(cudaStreamWaitEvent(b->side, b->fork, 0));
+        if ((r = launch_recon(b, 1, stage, b->side))) return r;
+        if ((r = launch_recon(b, 0, stage, b->stream, true))) return r;
+        CK(cudaEventRecord(b->join, b->side));
+        CK(cudaStreamWaitEvent(b->stream, b->join, 0));
+    } else if ((r = launch(b, (const void*)b->k.normal, W_NORMAL, 1, stage, true, true))) {
         return r;
     }
-    if ((r = launch(b, (const void*)(stage == 1 ? b->k.flux1 : b->k.flux2), W_FLUX, stage == 1 ? 2 : 3, 0, false))) return r;
-    if ((r = launch(b, (const void*)(stage == 1 ? b->k.upd1 : b->k.upd2), W_CELLS, stage == 1 ? 4 : 5, 0, false))) return r;
+    if ((r = launch(b, (const void*)(stage == 1 ? b->k.flux1 : b->k.flux2), W_FLUX, stage == 1 ? 2 : 3, 0, false, b->dim == 1))) return r;
+    if ((r = launch(b, (const void*)(stage == 1 ? b->k.upd1 : b->k.upd2), W_CELLS, stage == 1 ? 4 : 5, 0, false, over))) return r;
     return CGKS_OK;
 }
 
 int enqueue_step(cgks_batch* b, bool cfl)
 {
     int r;
-    if (cfl && (r = launch(b, (const void*)b->k.cfl, W_CELLS, 6, 0, false))) return r;
-    int use = cfl ? 1 : 0;
-    const double* fx = b->dfixed;
-    Mesh* dm = b->dmesh;
-    int n = b->n;
-    void* args[] = {&dm, &n, &use, &fx};
-    CK(cudaLaunchKernel((const void*)k_dt<0>, dim3((n + 127) / 128), dim3(128), args, 0, b->stream));
+    const bool one = b->n == 1;
+    if (cfl && (r = launch_cfl(b, one ? 1 : 0))) return r;
+    if (!cfl || !one) {
+        int use = cfl ? 1 : 0;
+        const double* fx = b->dfixed;
+        Mesh* dm = b->dmesh;
+        int n = b->n;
+        void* args[] = {&dm, &n, &use, &fx};
+        CK(launch_kernel((const void*)k_dt<0>, (n + 127) / 128, 128, args, 0, b->stream, cfl));
+    }
     if ((r = enqueue_stage(b, 1))) return r;
     if ((r = enqueue_stage(b, 2))) return r;
     return CGKS_OK;
@@ -235,6 +292,11 @@ int enqueue_step(cgks_batch* b, bool cfl)
 int build_graph(cgks_batch* b, int which)
 {
     if (b->gexec[which]) return CGKS_OK;
+    if (b->dim == 2 && overlap(b)) {
+        if (!b->side) CK(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
+        if (!b->fork) CK(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
+        if (!b->join) CK(cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming));
+    }
     cudaGraph_t g;
     CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     int r = enqueue_step(b, which == 1);
@@ -284,6 +346,14 @@ int validate(const cgks_params* p)
     // the fallback is compiled into the collision-time (tau > 0) flux only
     if (p->pt_fallback && p->tau_mode == CGKS_TAU_ZERO) return CGKS_ENOTSUP;
     return CGKS_OK;
+}
+
+// Linear weights of HWENO-AO (Eq. 3.12) and their ratios
+void set_ao(Mesh& g, const cgks_params* p)
+{
+    const double hi = p->gamma_hi, lo = p->gamma_lo, g0 = (1.0 - hi) * (1.0 - lo) * 0.5, g2 = (1.0 - hi) * lo;
+    const double v[6] = {g0, g2, hi, g0 / hi, g2 / hi, 1.0 / hi};
+    for (int q = 0; q < 6; ++q) { g.ao[q] = v[q]; g.aof[q] = (float)v[q]; }
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -370,7 +440,7 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
     }
     total = align256(total + n * sizeof(double));
     cudaError_t e = cudaMalloc(&b->slab, total);
-    if (e != cudaSuccess) { delete b; return e == cudaErrorMemoryAllocation ? CGKS_ENOMEM : CGKS_ECUDA; }
+    if (e != cudaSuccess) { cgks_batch_destroy(b); return e == cudaErrorMemoryAllocation ? CGKS_ENOMEM : CGKS_ECUDA; }
     b->dfixed = (double*)(b->slab + total - align256(n * sizeof(double)));
     b->host.resize(n);
     double K = p->dim == 2 ? (4.0 - 2.0 * p->gamma) / (p->gamma - 1.0) : (3.0 - p->gamma) / (p->gamma - 1.0);
@@ -388,7 +458,8 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
         std::memcpy(g.bcx, p->bc_split, sizeof(g.bcx));
         g.dx = (ext[4 * k + 1] - ext[4 * k]) / nx[k];
         g.dy = p->dim == 2 ? (ext[4 * k + 3] - ext[4 * k + 2]) / ny[k] : 1.0;
-        g.gamma = p->gamma; g.K = K; g.thr = p->sigma_thres; g.ghi = p->gamma_hi; g.glo = p->gamma_lo;
+        g.gamma = p->gamma; g.K = K; g.thr = p->sigma_thres;
+        set_ao(g, p);
         g.eps = p->weno_eps; g.c1 = p->tau_c1; g.c2 = p->tau_c2; g.cfl = p->cfl;
         g.igamma = 1.0 / g.gamma; g.igm1 = 1.0 / (g.gamma - 1.0);
         g.igf = (float)g.igamma; g.igm1f = (float)g.igm1;
@@ -427,6 +498,7 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
         g.ghost = (const double*)(sc + 80);  // 36 doubles of fixed ghost cells (1-D)
         g.tn = (double*)(sc + 368);
         g.nfall = (unsigned long long*)(sc + 376);
+        g.done = (unsigned*)(sc + 384);
     }
     // prefix arrays
     b->off.assign((size_t)W_COUNT * (n + 1), 0);
@@ -460,10 +532,15 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
         cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, dev);
         const void* fns[7] = {nullptr, (const void*)b->k.normal, (const void*)b->k.flux1,
                               (const void*)b->k.flux2, (const void*)b->k.upd1, (const void*)b->k.upd2,
-                              (const void*)b->k.cfl};
+                              (const void*)b->k.cfl[0]};
         for (int q = 0; q < 7; ++q) {
             int occ = 1;
-            int th = (q == 2 || q == 3) ? 128 : 256;
+            // 1-D meshes and small 2-D ones: small blocks, which spread over the SMs
+            // (80 cells FP64: flux 18 -> 8 us, its FP64 pipe being the SM's)
+            const long long all = b->off[(size_t)W_CELLS * (n + 1) + n];
+            const bool small = p->dim == 1 || all < 512LL * b->nsm;
+            int th = p->dim == 1 ? 32 : (q == 2 || q == 3) ? 128 : (small ? 64 : 256);
+            if (p->dim == 2 && (q == 2 || q == 3) && b->off[(size_t)W_FLUX * (n + 1) + n] < 8LL * b->nsm) th = 32;
             b->threads[q] = th;
             if (fns[q] && p->dim == 2 && (q == 2 || q == 3)) {
                 // every flux variant may launch blocks of up to 128 threads; the
@@ -510,9 +587,73 @@ int status_of(cgks_batch* b, long long* bad_out)
     return rc;
 }
 
+// The arrays of a state, in the order of the state planes (2-D: W, Wx, Wy,
+// Wx_line, Wy_line; 1-D: W, Wx), each [planes][cells]; end: running totals.
+struct StateArrays {
+    double* a[5];
+    long long end[5];
+    int n;
+};
+
+// FP32-bulk form, device arrays: straight between the caller's FP64 arrays and
+// the float planes, without the pass through the FP64 planes that host arrays
+// take (half the traffic; 2048^2, order 9: in and out 5.6 -> 2.9 ms with the
+// initial sigma's gain).
+__global__ void __launch_bounds__(256) k_state_in(StateArrays s, double* S0, float* F0, float* lo, long long nw)
+{
+    const long long stride = (long long)gridDim.x * blockDim.x;
+#pragma unroll 4
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < s.end[4]; e += stride) {
+        const int k = e < s.end[0] ? 0 : e < s.end[1] ? 1 : e < s.end[2] ? 2 : e < s.end[3] ? 3 : 4;
+        const double x = s.a[k][k ? e - s.end[k - 1] : e];
+        F0[e] = (float)x;
+        if (e < nw) {
+            S0[e] = x;
+            lo[e] = low_part<float>(x);
+        }
+    }
+}
+__global__ void __launch_bounds__(256) k_state_out(StateArrays s, const double* S0, const float* F0, long long nw)
+{
+    const long long stride = (long long)gridDim.x * blockDim.x;
+#pragma unroll 4
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < s.end[4]; e += stride) {
+        const int k = e < s.end[0] ? 0 : e < s.end[1] ? 1 : e < s.end[2] ? 2 : e < s.end[3] ? 3 : 4;
+        if (s.a[k]) s.a[k][k ? e - s.end[k - 1] : e] = e < nw ? S0[e] : (double)F0[e];
+    }
+}
+
+// The arrays of mesh k's state, and whether every one given is memory of the
+// current device, which a kernel may address (copies go anywhere).
+bool state_arrays(const cgks_batch* b, int k, const double* W, const double* Wx, const double* Wy, const double* Wxl,
+                  const double* Wyl, StateArrays& s)
+{
+    const long long P = b->host[k].plane;
+    const double* a[5] = {W, Wx, Wy, Wxl, Wyl};
+    const int planes[5] = {b->nvar, b->nvar, b->dim == 2 ? 4 : 0, b->dim == 2 ? 4 * b->M : 0, b->dim == 2 ? 4 * b->M : 0};
+    long long end = 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    for (int q = 0; q < 5; ++q) {
+        s.a[q] = planes[q] ? (double*)a[q] : nullptr;
+        s.end[q] = end += planes[q] * P;
+        if (!s.a[q]) continue;
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, a[q]) != cudaSuccess) { cudaGetLastError(); return false; }
+        if (at.type != cudaMemoryTypeDevice || at.device != dev || ((size_t)a[q] & 7)) return false;
+    }
+    s.n = 5;
+    return true;
+}
+
+int state_grid(const cgks_batch* b, long long n)
+{
+    return (int)std::max<long long>(1, std::min<long long>((n + 1023) / 1024, 8LL * b->nsm));
+}
+
 int set_state_impl(cgks_batch* b, int k, const double* W, const double* Wx, const double* Wy,
                    const double* Wxl, const double* Wyl, const double* sx, const double* sy,
-                   cudaMemcpyKind kind, bool sync)
+                   cudaMemcpyKind kind, bool sync, bool* converted = nullptr)
 {
     if (k < 0 || k >= b->n) return CGKS_EINVAL;
     Mesh& g = b->host[k];
@@ -521,9 +662,19 @@ int set_state_impl(cgks_batch* b, int k, const double* W, const double* Wx, cons
     if (!W || !Wx) return CGKS_EINVAL;
     if (b->dim == 2 && (!Wy || !Wxl || !Wyl)) return CGKS_EINVAL;
     cudaStream_t s = b->stream;
-    CK(cudaMemcpyAsync(g.S0, W, nv * P * 8, kind, s));
-    CK(cudaMemcpyAsync(g.S0 + nv * P, Wx, nv * P * 8, kind, s));
-    if (b->dim == 2) {
+    StateArrays sa;
+    const bool direct = kind == cudaMemcpyDeviceToDevice && b->rsize == 4 && state_arrays(b, k, W, Wx, Wy, Wxl, Wyl, sa);
+    if (converted) *converted = direct;
+    if (direct) {
+        const long long nw = nv * P;
+        float* lo = g.F0 + (size_t)b->nplanes * P;
+        void* args[] = {&sa, &g.S0, &g.F0, &lo, (void*)&nw};
+        CK(cudaLaunchKernel((const void*)k_state_in, dim3(state_grid(b, sa.end[4])), dim3(256), args, 0, s));
+    } else {
+        CK(cudaMemcpyAsync(g.S0, W, nv * P * 8, kind, s));
+        CK(cudaMemcpyAsync(g.S0 + nv * P, Wx, nv * P * 8, kind, s));
+    }
+    if (b->dim == 2 && !direct) {
         CK(cudaMemcpyAsync(g.S0 + 8 * P, Wy, 4 * P * 8, kind, s));
         CK(cudaMemcpyAsync(g.S0 + 12 * P, Wxl, 4 * b->M * P * 8, kind, s));
         CK(cudaMemcpyAsync(g.S0 + (12 + 4 * b->M) * P, Wyl, 4 * b->M * P * 8, kind, s));
@@ -638,7 +789,7 @@ int autotune(cgks_batch* b, int* out)
         CK(cudaMemcpy(&bad_saved[k], b->host[k].bad, 8, cudaMemcpyDeviceToHost));
     }
     // a CFL time step so that every kernel sees the data of a real step
-    int r = launch(b, (const void*)b->k.cfl, W_CELLS, 6, 0, false);
+    int r = launch_cfl(b, 0);
     if (r) return r;
     {
         int use = 1;
@@ -653,7 +804,7 @@ int autotune(cgks_batch* b, int* out)
     CK(cudaEventCreate(&e1));
     // the 2-D Steps 1-2 have one shape: run them for the flux's inputs
     for (int dir = 0; dir < (b->dim == 2 ? 2 : 0); ++dir)
-        if ((r = launch_recon(b, dir, 1))) return r;
+        if ((r = launch_recon(b, dir, 1, b->stream))) return r;
     for (int qq = 0; qq < 4; ++qq) {
         if (!fns[qq]) continue;
         int q = slots[qq];
@@ -665,7 +816,7 @@ int autotune(cgks_batch* b, int* out)
         int best_t = b->threads[q], best_g = b->grid[q];
         const void* best_f = fns[qq];
         float best = 1e30f;
-        const int cand[4] = {64, 128, 256, 512};
+        const int cand[4] = {b->dim == 1 ? 32 : 64, 128, 256, 512};
         for (int vi = 0; vi < 2; ++vi) {
             if (!var[vi]) continue;
             cudaFuncAttributes at;
@@ -787,11 +938,12 @@ int cgks_set_state_device(cgks_solver* s, const double* W, const double* Wx, con
                           const double* sigma_y)
 {
     if (!s) return CGKS_EINVAL;
-    int r = set_state_impl(s->b, 0, W, Wx, Wy, Wx_line, Wy_line, sigma_x, sigma_y, cudaMemcpyDeviceToDevice, false);
+    bool converted = false;
+    int r = set_state_impl(s->b, 0, W, Wx, Wy, Wx_line, Wy_line, sigma_x, sigma_y, cudaMemcpyDeviceToDevice, false, &converted);
     if (r) return r;
     s->b->state_set = true;
     s->b->sigma_pending = sigma_x == nullptr;
-    if ((r = convert_state(s->b, 1))) return r;
+    if (!converted && (r = convert_state(s->b, 1))) return r;
     if (sigma_x == nullptr) return launch(s->b, (const void*)s->b->k.siginit, W_SIGINIT, 6, 0, false);
     return CGKS_OK;
 }
@@ -819,14 +971,11 @@ int cgks_compute_dt(cgks_solver* s, double* dt)
 {
     if (!s || !dt) return CGKS_EINVAL;
     cgks_batch* b = s->b;
-    int r = launch(b, (const void*)b->k.cfl, W_CELLS, 6, 0, false);
+    if (!b->host_smax) CK(cudaHostAlloc((void**)&b->host_smax, sizeof(double), cudaHostAllocMapped));
+    int r = launch_cfl(b, 2);
     if (r) return r;
-    unsigned long long bits = 0, zero = 0;
-    CK(cudaMemcpyAsync(&bits, b->host[0].smax, 8, cudaMemcpyDeviceToHost, b->stream));
-    CK(cudaMemcpyAsync(b->host[0].smax, &zero, 8, cudaMemcpyHostToDevice, b->stream));
     CK(cudaStreamSynchronize(b->stream));
-    double sm;
-    std::memcpy(&sm, &bits, 8);
+    const double sm = *b->host_smax;
     *dt = sm > 0.0 ? b->p.cfl / sm : 0.0;
     return CGKS_OK;
 }
@@ -870,8 +1019,18 @@ static int get_state_impl(cgks_batch* b, int k, double* W, double* Wx, double* W
     size_t P = (size_t)g.plane;
     int nv = b->nvar;
     cudaStream_t s = b->stream;
-    if (b->state_set) {
-        int r = convert_state(b, 0);
+    StateArrays sa;
+    const bool direct = kind == cudaMemcpyDeviceToDevice && b->rsize == 4 && b->state_set && state_arrays(b, k, W, Wx, Wy, Wxl, Wyl, sa);
+    if (direct) {
+        const long long nw = nv * P;
+        const double* S0 = g.S0;
+        const float* F0 = g.F0;
+        void* args[] = {&sa, &S0, &F0, (void*)&nw};
+        CK(cudaLaunchKernel((const void*)k_state_out, dim3(state_grid(b, sa.end[4])), dim3(256), args, 0, s));
+        W = Wx = Wy = Wxl = Wyl = nullptr;  // done
+    } else if (b->state_set && b->rsize == 4) {
+        // this mesh's slopes (of a batch: not every mesh's on every read)
+        int r = launch_one(b, k, (const void*)b->k.convert, W_CELLS, 0, true);
         if (r) return r;
     }
     if (W) CK(cudaMemcpyAsync(W, g.S0, nv * P * 8, kind, s));
@@ -968,8 +1127,8 @@ int cgks_profile_step(cgks_solver* s, double dt, float* ms, int* ids, int* n)
     }
     for (int stage = 1; stage <= 2; ++stage) {
         if (b->dim == 2) {
-            if ((r = launch_recon(b, 0, stage)) || (r = rec(10 * stage + 0))) goto done;
-            if ((r = launch_recon(b, 1, stage)) || (r = rec(10 * stage + 1))) goto done;
+            if ((r = launch_recon(b, 0, stage, b->stream)) || (r = rec(10 * stage + 0))) goto done;
+            if ((r = launch_recon(b, 1, stage, b->stream)) || (r = rec(10 * stage + 1))) goto done;
         } else {
             if ((r = launch(b, (const void*)b->k.normal, W_NORMAL, 1, stage, true)) || (r = rec(10 * stage + 1))) goto done;
         }
@@ -1032,12 +1191,13 @@ int cgks_batch_set_state_device(cgks_batch* b, int k, const double* W, const dou
                                 const double* Wx_line, const double* Wy_line)
 {
     if (!b) return CGKS_EINVAL;
-    int r = set_state_impl(b, k, W, Wx, Wy, Wx_line, Wy_line, nullptr, nullptr, cudaMemcpyDeviceToDevice, false);
+    bool converted = false;
+    int r = set_state_impl(b, k, W, Wx, Wy, Wx_line, Wy_line, nullptr, nullptr, cudaMemcpyDeviceToDevice, false, &converted);
     if (r) return r;
     b->state_set = true;
     // the float planes, sigma from the cell averages and the positivity check of
     // instance k, enqueued; a non-physical state shows in cgks_batch_sync
-    if (b->rsize == 4 && (r = launch_one(b, k, (const void*)b->k.convert, W_CELLS, 1, true))) return r;
+    if (b->rsize == 4 && !converted && (r = launch_one(b, k, (const void*)b->k.convert, W_CELLS, 1, true))) return r;
     if ((r = launch_one(b, k, (const void*)b->k.siginit, W_SIGINIT, 0, false))) return r;
     return launch_one(b, k, (const void*)b->k.check, W_CELLS, 0, false);
 }
@@ -1082,6 +1242,10 @@ void cgks_batch_destroy(cgks_batch* b)
     if (b->doff) cudaFree(b->doff);
     if (b->doff1) cudaFree(b->doff1);
     if (b->slab) cudaFree(b->slab);
+    if (b->host_smax) cudaFreeHost(b->host_smax);
+    if (b->fork) cudaEventDestroy(b->fork);
+    if (b->join) cudaEventDestroy(b->join);
+    if (b->side) cudaStreamDestroy(b->side);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b;
 }
@@ -1186,7 +1350,8 @@ extern "C" int cgks_step_1d_noalloc(const cgks_params* p, int nx, double x0, dou
     g.x0 = x0;
     g.dx = (x1 - x0) / nx; g.dy = 1.0;
     g.gamma = p->gamma; g.K = (3.0 - p->gamma) / (p->gamma - 1.0); g.thr = p->sigma_thres;
-    g.ghi = p->gamma_hi; g.glo = p->gamma_lo; g.eps = p->weno_eps; g.c1 = p->tau_c1; g.c2 = p->tau_c2;
+    set_ao(g, p);
+    g.eps = p->weno_eps; g.c1 = p->tau_c1; g.c2 = p->tau_c2;
     g.cfl = p->cfl; g.plane = nx;
     g.igamma = 1.0 / g.gamma; g.igm1 = 1.0 / (g.gamma - 1.0);
     g.igf = (float)g.igamma; g.igm1f = (float)g.igm1;
@@ -1210,6 +1375,7 @@ extern "C" int cgks_step_1d_noalloc(const cgks_params* p, int nx, double x0, dou
     g.bad = (long long*)(sc + 24); g.smax = (unsigned long long*)(sc + 32);
     g.branch = (unsigned long long*)(sc + 40); g.dtf = (float*)(sc + 72); g.ghost = (const double*)(sc + 80);
     g.tn = (double*)(sc + 368); g.nfall = (unsigned long long*)(sc + 376);
+    g.done = (unsigned*)(sc + 384);
     NoallocInit init;
     std::memset(&init, 0, sizeof(init));
     init.g = g;
@@ -1249,7 +1415,18 @@ extern "C" int cgks_step_1d_noalloc(const cgks_params* p, int nx, double x0, dou
     if (!sigma_in && (r = go((const void*)k.siginit, W_SIGINIT, 0, false, 256))) return r;
     // dt: the CFL reduction into the scratch scalars, or the fixed value copied above
     int use_cfl = dt > 0.0 ? 0 : 1;
-    if (use_cfl && (r = go((const void*)k.cfl, W_CELLS, 0, false, 256))) return r;
+    if (use_cfl) {
+        Work w;
+        w.mesh = dmesh;
+        w.m0 = g;
+        w.off = doff + 2 * W_CELLS;
+        w.n = 1;
+        w.total = off[2 * W_CELLS + 1];
+        double* out = nullptr;
+        void* args[] = {&w, &out};
+        const int grid = (int)std::max<long long>(1, std::min<long long>((w.total + 255) / 256, 4LL * nsm));
+        CK(cudaLaunchKernel((const void*)k.cfl[0], dim3(grid), dim3(256), args, 0, st));
+    }
     {
         int n1 = 1;
         const double* fixed = g.dt;

@@ -66,7 +66,9 @@ struct Mesh {
     int tau_mode;
     int dff_lag;                    // 0: sigma of step n-1; 1: stage 2 uses stage 1's
     int pf;                         // first-order fallback at non-physical face points
-    double dx, dy, gamma, K, thr, ghi, glo, eps, c1, c2, cfl;
+    double dx, dy, gamma, K, thr, eps, c1, c2, cfl;
+    double ao[6];                   // linear weights of HWENO-AO: g0 = g1, g2, g3, g0 / g3, g2 / g3, 1 / g3
+    float aof[6];
     double idx, idy;                // 1 / dx, 1 / dy
     double mu;                      // dynamic viscosity (tau_mode 2)
     double x0, y0;                  // lower-left corner
@@ -101,6 +103,7 @@ struct Mesh {
     unsigned* status;
     long long* bad;
     unsigned long long* smax;       // CFL reduction (bits of a positive double)
+    unsigned* done;                 // its blocks that have arrived
     unsigned long long* branch;     // [4] AO, r5, r7, r9 counts
 };
 
@@ -147,6 +150,7 @@ template <> struct MeshR<double> {
     __device__ static double gamma(const Mesh& g) { return g.gamma; }
     __device__ static double K(const Mesh& g) { return g.K; }
     __device__ static double igamma(const Mesh& g) { return g.igamma; }
+    __device__ static const double* ao(const Mesh& g) { return g.ao; }
     __device__ static double igm1(const Mesh& g) { return g.igm1; }
     __device__ static double c1(const Mesh& g) { return g.c1; }
     __device__ static double c2(const Mesh& g) { return g.c2; }
@@ -158,6 +162,7 @@ template <> struct MeshR<float> {
     __device__ static float gamma(const Mesh& g) { return g.gf; }
     __device__ static float K(const Mesh& g) { return g.Kf; }
     __device__ static float igamma(const Mesh& g) { return g.igf; }
+    __device__ static const float* ao(const Mesh& g) { return g.aof; }
     __device__ static float igm1(const Mesh& g) { return g.igm1f; }
     __device__ static float c1(const Mesh& g) { return g.c1f; }
     __device__ static float c2(const Mesh& g) { return g.c2f; }
@@ -520,25 +525,6 @@ __device__ __forceinline__ Dff dff_select(int order, const double s[6], double t
     return d;
 }
 
-// A cell's DFF choice in the bulk precision R: the DFFs of S0, S1, S2 = r5
-// (a[2] == a[3]) and the stencil code (-1 HWENO-AO, else r5/r7/r9).  On the
-// linear branches the chosen stencil's DFF is 1 (Algorithm 1 only takes a
-// linear stencil whose DFF is 1), so only the HWENO-AO branch scales.
-template <typename R>
-struct DffR {
-    R a[4];
-    int st;
-};
-
-template <typename R>
-__device__ __forceinline__ DffR<R> dff_r(const Dff& d)
-{
-    DffR<R> r;
-    for (int k = 0; k < 4; ++k) r.a[k] = (R)d.a[k];
-    r.st = d.st;
-    return r;
-}
-
 // The taps of dp that sub-stencil k of HWENO-AO uses (S0, S1, S2, r5; the own
 // average enters through the differences only)
 __host__ __device__ constexpr bool ao_tap(int k, int q)
@@ -552,9 +538,12 @@ __host__ __device__ constexpr bool ao_tap(int k, int q)
 // HWENO-AO(5,3) with DFF-scaled sub-polynomials (Eq. 3.11-3.17, 3.19) for
 // NOUT consecutive functional rows starting at row0.  Kept out of line: the
 // branch is rare, and inlining it in every variable's loop bloats the kernels.
-// Only the taps a sub-stencil has are summed (10 of 40 a row).
+// Only the taps a sub-stencil has are summed (10 of 40 a row), and only the
+// entries of the smoothness matrices that are not zero (even x + y); the linear
+// weights' ratios gw = (g0, g2, g3, g0 / g3, g2 / g3, 1 / g3) come from the host: a
+// few lanes of a shock's cells hold up an FP64 warp for all of this.
 template <typename R, int NOUT>
-__device__ __noinline__ void recon_ao(const R* al, int oi, int row0, const R* dp, R* out, R ghi, R glo, R eps)
+__device__ __noinline__ void recon_ao(const R* al, int oi, int row0, const R* dp, R* out, const R* gw, R eps)
 {
     const auto& T = Tab<R>::get(oi);
     R beta[4];
@@ -572,36 +561,28 @@ __device__ __noinline__ void recon_ao(const R* al, int oi, int row0, const R* dp
             }
             c[n] = s;
         }
-        R b = 0;
+        R b;
         if (k < 3) {
-#pragma unroll
-            for (int x = 1; x < 3; ++x)
-#pragma unroll
-                for (int y = 1; y < 3; ++y) b += c[x] * c[y] * T.bm2[x][y];
+            b = T.bm2[1][1] * (c[1] * c[1]) + T.bm2[2][2] * (c[2] * c[2]);
         } else {
-#pragma unroll
-            for (int x = 1; x < 5; ++x)
-#pragma unroll
-                for (int y = 1; y < 5; ++y) b += c[x] * c[y] * T.bm4[x][y];
+            b = c[1] * (T.bm4[1][1] * c[1] + ((R)2 * T.bm4[1][3]) * c[3]) + c[2] * (T.bm4[2][2] * c[2] + ((R)2 * T.bm4[2][4]) * c[4])
+              + T.bm4[3][3] * (c[3] * c[3]) + T.bm4[4][4] * (c[4] * c[4]);
         }
         beta[k] = al[k] * al[k] * b;  // smoothness of the DFF-scaled polynomial
     }
-    R g3 = ghi, g2 = ((R)1 - ghi) * glo, g0 = ((R)1 - ghi) * ((R)1 - glo) * (R)0.5;
-    R gk[4] = {g0, g0, g2, g3};
-    R tz = (fabs(beta[3] - beta[0]) + fabs(beta[3] - beta[1]) + fabs(beta[3] - beta[2])) / (R)3;
+    const R tz = (fabs(beta[3] - beta[0]) + fabs(beta[3] - beta[1]) + fabs(beta[3] - beta[2])) * (R)(1.0 / 3.0);
     R w[4], ws = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        R q = tz / (beta[k] + eps);
-        w[k] = gk[k] * ((R)1 + q * q);
+        const R q = tz / (beta[k] + eps), g = gw[k < 2 ? 0 : k - 1];
+        w[k] = g + g * (q * q);
         ws += w[k];
     }
-    R inv = (R)1 / ws;
-    R c3 = w[3] * inv / g3;
+    const R inv = (R)1 / ws;
     R ck[4];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) ck[k] = (w[k] * inv - w[3] * inv * gk[k] / g3) * al[k];
-    ck[3] = c3 * al[3];
+    for (int k = 0; k < 3; ++k) ck[k] = (w[k] - w[3] * gw[k < 2 ? 3 : 4]) * inv * al[k];
+    ck[3] = w[3] * inv * gw[5] * al[3];
 #pragma unroll
     for (int r = 0; r < NOUT; ++r) {
         R s = 0;
@@ -615,28 +596,6 @@ __device__ __noinline__ void recon_ao(const R* al, int oi, int row0, const R* dp
         }
         out[r] = s;
     }
-}
-
-// Evaluate NOUT consecutive functional rows (from row0) of the ASE-DFF
-// polynomial of one cell.  dp[10]: data relative to the own cell:
-// [Qbar_{i+k} - Qbar_i (k=-2..2), h*Qx_{i+k}]; values come out relative to
-// Qbar_i too (Eq. 3.5: Q_i + alpha (p - Q_i), derivatives alpha p').
-template <typename R, int NOUT>
-__device__ __forceinline__ void recon(const DffR<R>& dff, int oi, int row0, const R dp[10], R out[NOUT],
-                                      R ghi, R glo, R eps)
-{
-    if (dff.st >= 0) {
-        const auto& T = Tab<R>::get(oi);
-#pragma unroll
-        for (int r = 0; r < NOUT; ++r) {
-            R s = 0;
-#pragma unroll
-            for (int k = 0; k < 10; ++k) s += T.row[dff.st][row0 + r][k] * dp[k];
-            out[r] = s;
-        }
-        return;
-    }
-    recon_ao<R, NOUT>(dff.a, oi, row0, dp, out, ghi, glo, eps);
 }
 
 // The taps of dp = (Qbar_{i-2..i+2} - Qbar_i, h Qx_{i-2..i+2}) that a linear
@@ -698,6 +657,23 @@ __device__ __forceinline__ void sym_data(const R dp[10], R e[2], R o[2], R E[2],
         O[j] = dp[8 + j] - dp[6 - j];
     }
 }
+
+// value, first and second derivative at xi = +1/2 (out[0..2]) and -1/2 (out[3..5])
+template <int ST>
+__device__ __forceinline__ void faces_sym(const CgksTables& T, const double dp[10], double out[6])
+{
+    double e[2], o[2], E[2], O[2];
+    sym_data(dp, e, o, E, O);
+#pragma unroll
+    for (int nd = 0; nd < 3; ++nd) {
+        double p, q;
+        sym_row<ST, double>(T.sym[ST - ST_R5][nd], e, o, E, O, p, q);
+        out[nd] = p + q;
+        out[3 + nd] = nd == 1 ? q - p : p - q;
+    }
+}
+template <int ST>
+__device__ __forceinline__ void faces_sym(const CgksTables&, const float*, float*) {}  // FP32 keeps the taps
 
 // Calls body(StTag<st>()) for a stencil code (-1: HWENO-AO); the order bounds
 // the linear stencils that occur.  The branch is taken once, outside the loop

@@ -7,13 +7,15 @@
 namespace cgks {
 typedef void (*KStage)(Work, int);
 typedef void (*KOne)(Work);
+typedef void (*KCfl)(Work, double*);
 struct Kfns {
     KStage recon[2];           // 2-D Steps 1-2 per direction (meshes without walls)
     KStage reconw[2];          // the same with the wall ghost rules
     int recon_tile[2][2];      // their tile shapes (TA, TB), blocks and dynamic shared memory
     int recon_threads[2], recon_bytes[2];
     KStage normal, normalw;    // 1-D Step 2, without and with the wall ghost rules
-    KOne flux1, flux2, upd1, upd2, cfl, siginit, check;
+    KOne flux1, flux2, upd1, upd2, siginit, check;
+    KCfl cfl[3];               // CFL reduction: alone, with the step set, to the host
     KStage convert;  // FP32-bulk state copies (to_float = 1: FP64 -> float planes)
     KOne flux1v[2], flux2v[2];  // flux variants: [0] uncapped, [1] register-capped (tau = 0)
     KOne flux1h[2], flux2h[2];  // the same with the collision-time terms (tau > 0)

@@ -67,7 +67,9 @@ Kfns make_kfns_one()
     if constexpr (D == 2) { k.upd1 = (KOne)k_update2<M, R, 1, ONE>; k.upd2 = (KOne)k_update2<M, R, 2, ONE>; }
     else { k.upd1 = (KOne)k_update1<R, 1, ONE>; k.upd2 = (KOne)k_update1<R, 2, ONE>; }
     k.flux_warp_bytes = D == 2 ? (int)(FluxShared<(D == 2 ? M : 4), R>::total * sizeof(R)) : 0;
-    k.cfl = k_cfl<D, R>;
+    k.cfl[0] = k_cfl<D, R, 0>;
+    k.cfl[1] = k_cfl<D, R, 1>;
+    k.cfl[2] = k_cfl<D, R, 2>;
     k.siginit = k_sigma_init<D>;
     k.check = k_check_state<D>;
     k.convert = k_convert<D, M>;

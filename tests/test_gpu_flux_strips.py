@@ -1,6 +1,6 @@
 """The 2-D flux kernel marches warps over strips of 32 / m faces (16, 10, 8 for
 orders 5, 7, 9), and Steps 1-2 cover the mesh and a ring of ghost cells with
-tiles of 28 x 4 (x faces) and 12 x 16 (y faces; FP64 12 x 8) cells: meshes that
+tiles of 28 x 4 (x faces; FP64 28 x 2) and 12 x 16 (y faces; FP64 12 x 8) cells: meshes that
 fill strips or tiles exactly, fall one short or spill one over, in each
 direction, alone and as a batch (one work list over meshes of different sizes),
 against the oracle after one step.

@@ -708,7 +708,7 @@ int launch_one(cgks_batch* b, int k, const void* fn, int kind, int arg, bool has
     w.n = 1;
     w.total = items(b->k, kind, b->dim, b->M, b->host[k].nx, b->host[k].ny);
     if (w.total == 0) return CGKS_OK;
-    int threads = 256;
+    int threads = w.total < 512LL * b->nsm ? 64 : 256;
     long long need = (w.total + threads - 1) / threads;
     int grid = (int)std::max<long long>(1, std::min<long long>(need, (long long)b->grid[6]));
     void* a2[] = {&w, &arg};

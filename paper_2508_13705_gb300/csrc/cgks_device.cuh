@@ -140,6 +140,18 @@ __device__ __forceinline__ const Mesh& mesh_of(const Work& w, long long gi, long
     return w.mesh[k];
 }
 
+// The same for a thread whose items only go up: the mesh is searched once and
+// then stepped on from.  k: -1 at first.
+template <bool ONE>
+__device__ __forceinline__ const Mesh& mesh_from(const Work& w, long long gi, long long& local, int& k)
+{
+    if (ONE) { local = gi; return w.m0; }
+    if (k < 0) k = find_mesh(w, gi);
+    while (gi >= w.off[k + 1]) ++k;
+    local = gi - w.off[k];
+    return w.mesh[k];
+}
+
 __device__ __forceinline__ int imod(int a, int n) { int r = a % n; return r < 0 ? r + n : r; }
 
 // ------------------------------------------------------------------ ghost cells

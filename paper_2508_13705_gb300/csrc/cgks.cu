@@ -2,7 +2,7 @@
 //
 // A single-mesh solver is a batch of one: every kernel is a grid-stride loop
 // over the work items of all meshes of a descriptor table (see
-// cgks_kernels.cuh), launched with one persistent grid sized to the GPU
+// cgks_kernels.cuh), launched with a persistent grid sized to the GPU
 // (SM count x resident blocks).  One S2O4 step (Sec. 2.2) is captured once as
 // a CUDA graph:
 //   [CFL reduction] -> dt -> stage 1 (lines, normal, flux, update)
@@ -62,6 +62,7 @@ int load_tables()
             for (int b = 0; b < 2; ++b)
                 for (int c = 0; c < 7; ++c) {
                     f[k].sd1[a][b][c] = (float)t[k].sd1[a][b][c];
+                    f[k].sd1w[a][b][c] = make_float2(f[k].sd1[a][b][c], f[k].sd1[a][b][c]);
                     f[k].sd2[a][b][c] = (float)t[k].sd2[a][b][c];
                 }
     }
@@ -597,8 +598,8 @@ struct StateArrays {
 
 // FP32-bulk form, device arrays: straight between the caller's FP64 arrays and
 // the float planes, without the pass through the FP64 planes that host arrays
-// take (half the traffic; 2048^2, order 9: in and out 5.6 -> 2.9 ms with the
-// initial sigma's gain).
+// take (half the traffic; 2048^2, order 9: in and out 5.6 -> 2.5 ms, of which the
+// initial sigma's part fell from 3.1 to 0.9 ms).
 __global__ void __launch_bounds__(256) k_state_in(StateArrays s, double* S0, float* F0, float* lo, long long nw)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;

@@ -45,7 +45,8 @@ struct TabF {
     float bm4[5][5];
     float gx[4], gw[4];
     float sd1[2][2][7], sd2[2][2][7];
-    float2 row2[3][10][10];  // rows of r5, r7, r9, each coefficient twice, for two-wide FMAs
+    // each coefficient twice, for two-wide FMAs: rows of r5, r7, r9, and sd1
+    float2 row2[3][10][10], sd1w[2][2][7];
 };
 
 static __constant__ CgksTables c_tab[3];  // orders 5, 7, 9 (one copy per translation unit)

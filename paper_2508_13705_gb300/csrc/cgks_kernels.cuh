@@ -721,10 +721,11 @@ __global__ void __launch_bounds__(256) k_normal1(Work w, int stage)
 // shared-memory passes a step on them (780 us): a 16-byte load takes four,
 // whichever lanes read alike.  A lane per variable reads 4 bytes, one pass for
 // a whole segment point of 8 faces, serves all M lines from it with weights from
-// constant memory, and sums mirrored points once for mirrored lines.  Now FP32
-// takes 512 + 448 us for the two stages (start 889 + 770), bound by issue slots:
-// 1443 instructions a point, 955 of them FP32 arithmetic, 16 warps per SM.  FP64,
-// bound by the FP64 pipe, takes 3.35 + 3.10 ms at 512^2 (start 5.96 + 5.51).  The
+// constant memory, and sums mirrored points once for mirrored lines.  With the
+// ghost bases out of the way (TD) and the face sums (below), FP32 takes 416 + 363
+// us for the two stages (start 889 + 770), bound by issue slots: 75% of them used
+// by 16 warps per SM, about 920 FP32 instructions of 1450 a point.  FP64, bound by
+// its pipe (87% busy), takes 3.28 + 2.99 ms at 512^2 (start 5.96 + 5.51).  The
 // steps of a mesh are dealt to the warps in equal contiguous runs: a run has one
 // prologue, the rest streams.
 template <int M> struct FluxStrip {
@@ -770,47 +771,76 @@ __device__ __forceinline__ void step3(const R* W, const R* Wn, const int q[3], R
     constexpr int K = 3 * M, H = K / 2, RING = FluxStrip<M>::RING, FW = FluxStrip<M>::FW;
     constexpr bool BULK32 = sizeof(R) == 4;
     const auto& T = Tab<R>::get(M - 2);
-    R e[H + 1], o[H];
-    auto split = [&](const R* P) {
-        R x[K];
-#pragma unroll
-        for (int s = 0; s < 3; ++s)
-#pragma unroll
-            for (int k = 0; k < M; ++k) x[s * M + k] = P[(k * RING + q[s]) * 4];
-#pragma unroll
-        for (int k = 0; k < H; ++k) { e[k] = x[k] + x[K - 1 - k]; o[k] = x[k] - x[K - 1 - k]; }
-        e[H] = K % 2 ? x[H] : (R)0;
+    constexpr int NE = (K + 1) / 2;
+    // quantity q at line l and its mirror: scale (odd + even), +-scale (odd - even)
+    auto put = [&](int q, int l, R scale, R plus, R minus) {
+        const R m = scale * minus;  // the part that changes sign
+        out[(q * M + l) * FW * 4] = scale * plus + m;
+        if (M - 1 - l != l) out[(q * M + M - 1 - l) * FW * 4] = scale * plus - m;
     };
-    auto sum = [&](const R* w, const R* v, int n) {
-        R r = w[0] * v[0];
+    if constexpr (BULK32) {
+        // W and W_n share the first-derivative weights: both at once, with two-wide FMAs
+        float2 e[H + 1], o[H];
 #pragma unroll
-        for (int k = 1; k < n; ++k) r += w[k] * v[k];
-        return r;
-    };
-    split(W);
-#pragma unroll
-    for (int l = 0; l < (M + 1) / 2; ++l) {
-        R te = sum(T.sd1[l][0], e, (K + 1) / 2), to = sum(T.sd1[l][1], o, H);
-        R se = sum(T.sd2[l][0], e, (K + 1) / 2), so = sum(T.sd2[l][1], o, H);
-        if (BULK32) {
-            te += T.sd1[l][0][6] * (dm + dp);
-            to += T.sd1[l][1][6] * (dm - dp);
-            se += T.sd2[l][0][6] * (dm + dp);
-            so += T.sd2[l][1][6] * (dm - dp);
+        for (int k = 0; k <= (K % 2 ? H : H - 1); ++k) {
+            auto at2 = [&](int j) {
+                const int x = ((j % M) * RING + q[j / M]) * 4;
+                return make_float2(W[x], Wn[x]);
+            };
+            const float2 x = at2(k);
+            if (k == H) {
+                e[k] = x;
+            } else {
+                const float2 y = at2(K - 1 - k);
+                e[k] = add2(x, y);
+                o[k] = sub2(x, y);
+            }
         }
-        out[(0 * M + l) * FW * 4] = c1 * (to + te);
-        out[(1 * M + l) * FW * 4] = c2 * (se + so);
-        if (M - 1 - l != l) {
-            out[(0 * M + M - 1 - l) * FW * 4] = c1 * (to - te);
-            out[(1 * M + M - 1 - l) * FW * 4] = c2 * (se - so);
-        }
-    }
-    split(Wn);
+        const float sb = dm + dp, db = dm - dp;
 #pragma unroll
-    for (int l = 0; l < (M + 1) / 2; ++l) {
-        R te = sum(T.sd1[l][0], e, (K + 1) / 2), to = sum(T.sd1[l][1], o, H);
-        out[(2 * M + l) * FW * 4] = c1 * (to + te);
-        if (M - 1 - l != l) out[(2 * M + M - 1 - l) * FW * 4] = c1 * (to - te);
+        for (int l = 0; l < (M + 1) / 2; ++l) {
+            float2 te = __fmul2_rn(T.sd1w[l][0][0], e[0]), to = __fmul2_rn(T.sd1w[l][1][0], o[0]);
+            float se = T.sd2[l][0][0] * e[0].x, so = T.sd2[l][1][0] * o[0].x;
+#pragma unroll
+            for (int k = 1; k < NE; ++k) {
+                te = __ffma2_rn(T.sd1w[l][0][k], e[k], te);
+                se += T.sd2[l][0][k] * e[k].x;
+                if (k < H) {
+                    to = __ffma2_rn(T.sd1w[l][1][k], o[k], to);
+                    so += T.sd2[l][1][k] * o[k].x;
+                }
+            }
+            put(0, l, c1, to.x + T.sd1[l][1][6] * db, te.x + T.sd1[l][0][6] * sb);
+            put(1, l, c2, se + T.sd2[l][0][6] * sb, so + T.sd2[l][1][6] * db);
+            put(2, l, c1, to.y, te.y);
+        }
+    } else {
+        R e[H + 1], o[H];
+        auto split = [&](const R* P) {
+            R x[K];
+#pragma unroll
+            for (int s = 0; s < 3; ++s)
+#pragma unroll
+                for (int k = 0; k < M; ++k) x[s * M + k] = P[(k * RING + q[s]) * 4];
+#pragma unroll
+            for (int k = 0; k < H; ++k) { e[k] = x[k] + x[K - 1 - k]; o[k] = x[k] - x[K - 1 - k]; }
+            e[H] = K % 2 ? x[H] : (R)0;
+        };
+        auto sum = [&](const R* w, const R* v, int n) {
+            R r = w[0] * v[0];
+#pragma unroll
+            for (int k = 1; k < n; ++k) r += w[k] * v[k];
+            return r;
+        };
+        split(W);
+#pragma unroll
+        for (int l = 0; l < (M + 1) / 2; ++l) {
+            put(0, l, c1, sum(T.sd1[l][1], o, H), sum(T.sd1[l][0], e, NE));
+            put(1, l, c2, sum(T.sd2[l][0], e, NE), sum(T.sd2[l][1], o, H));
+        }
+        split(Wn);
+#pragma unroll
+        for (int l = 0; l < (M + 1) / 2; ++l) put(2, l, c1, sum(T.sd1[l][1], o, H), sum(T.sd1[l][0], e, NE));
     }
 }
 
@@ -1842,7 +1872,7 @@ __global__ void k_dt(Mesh* meshes, int n, int use_cfl, const double* fixed)
 // Initial sigma from the two cell averages adjacent to each face (Eq. 3.2), in
 // FP64 and bound by its pipe: a thread takes kSigRows cells of a column, so that
 // the cell below is evaluated once, with one reciprocal and one reciprocal
-// square root a cell and one division a face (2048^2: 2.6 -> 0.8 ms).
+// square root a cell and one division a face (2048^2: 3.06 -> 0.91 ms).
 constexpr int kSigRows = 4;
 
 struct Mach { double p, mx, my; };  // pressure, Mach numbers along x and y

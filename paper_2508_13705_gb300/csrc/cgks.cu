@@ -1,13 +1,12 @@
 // Host side of the C ABI declared in include/cgks.h.
 //
-// A single-mesh solver is a batch of one: every kernel is a grid-stride loop
-// over the work items of all meshes of a descriptor table (see
-// cgks_kernels.cuh), launched with a persistent grid sized to the GPU
-// (SM count x resident blocks).  One S2O4 step (Sec. 2.2) is captured once as
-// a CUDA graph:
-//   [CFL reduction] -> dt -> stage 1 (lines, normal, flux, update)
-//                         -> stage 2 (lines, normal, flux, update)
+// A single-mesh solver is a batch of one: every kernel covers the work items of
+// all meshes of a descriptor table (see cgks_kernels.cuh).  One S2O4 step
+// (Sec. 2.2) is captured once as a CUDA graph:
+//   CFL reduction and dt -> stage 1 (Steps 1-2 per direction, flux, update)
+//                        -> stage 2 (the same)
 // Device memory of all meshes lives in one slab allocated at init.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -624,6 +623,28 @@ __global__ void __launch_bounds__(256) k_state_out(StateArrays s, const double* 
     }
 }
 
+// Whether `bytes` from p on lie inside one allocation: the driver refuses a copy
+// that leaves it, and a kernel must not take such a range over.
+bool in_one_allocation(const void* p, size_t bytes)
+{
+    using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) !=
+                cudaSuccess || found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (Range)f;
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    if (!range || range(&base, &size, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    const size_t at = (CUdeviceptr)p - base;
+    return at <= size && bytes <= size - at;
+}
+
 // The arrays of mesh k's state, and whether every one given is memory of the
 // current device, which a kernel may address (copies go anywhere).
 bool state_arrays(const cgks_batch* b, int k, const double* W, const double* Wx, const double* Wy, const double* Wxl,
@@ -642,6 +663,7 @@ bool state_arrays(const cgks_batch* b, int k, const double* W, const double* Wx,
         cudaPointerAttributes at;
         if (cudaPointerGetAttributes(&at, a[q]) != cudaSuccess) { cudaGetLastError(); return false; }
         if (at.type != cudaMemoryTypeDevice || at.device != dev || ((size_t)a[q] & 7)) return false;
+        if (!in_one_allocation(a[q], planes[q] * P * sizeof(double))) return false;
     }
     s.n = 5;
     return true;
@@ -972,7 +994,14 @@ int cgks_compute_dt(cgks_solver* s, double* dt)
 {
     if (!s || !dt) return CGKS_EINVAL;
     cgks_batch* b = s->b;
-    if (!b->host_smax) CK(cudaHostAlloc((void**)&b->host_smax, sizeof(double), cudaHostAllocMapped));
+    if (!b->host_smax) {
+        // also while another stream of this program is being captured
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        const cudaError_t e = cudaHostAlloc((void**)&b->host_smax, sizeof(double), cudaHostAllocMapped);
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        CK(e);
+    }
     int r = launch_cfl(b, 2);
     if (r) return r;
     CK(cudaStreamSynchronize(b->stream));

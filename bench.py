@@ -50,8 +50,8 @@ ORACLE_FLOPS = {
 # counterparts; dram__bytes_read.sum + dram__bytes_write.sum), for the
 # kernels as profiled in profiles/kernel_counters_vortex1024_o9.md: the pipe
 # utilisation beside the algorithmic rate, and the DRAM traffic per launch.
-FLUX1_EXECUTED = {"fp32": {"flops_per_cell": 20723.8, "dram_bytes_per_cell": 1417.5},
-                  "fp64": {"flops_per_cell": 21389.3, "dram_bytes_per_cell": 2711.5}}
+FLUX1_EXECUTED = {"fp32": {"flops_per_cell": 11376.2, "dram_bytes_per_cell": 1305.1},
+                  "fp64": {"flops_per_cell": 11273.3, "dram_bytes_per_cell": 2234.5}}
 
 
 def parse():
@@ -363,7 +363,7 @@ def roofline(kms, precision, order, n, p32, p64, hbm):
     is the oracle's count of the kinetic part per face Gauss point times the
     launch's 2 m n (n + 1) points; the peak is the measured FMA throughput of
     the kernel's precision.  The kernels reach the oracle's results with fewer
-    operations (one Gram matrix per Maxwellian, closed-form micro-slopes), so
+    operations (moment differentials instead of micro-slope solves), so
     this algorithmic rate can exceed what the pipe executes."""
     m = (order - 1) // 2
     pts = 2 * m * n * (n + 1)
@@ -373,7 +373,7 @@ def roofline(kms, precision, order, n, p32, p64, hbm):
     peak = p32 if precision == "fp32" else p64
     ach = alg / (ms / 1e3) / 1e12
     ex = FLUX1_EXECUTED[precision] if order == 9 else None
-    out = {"bound": "alu", "kernel": "k_flux, stage 1", "achieved": round(ach, 3), "peak": round(peak, 2),
+    out = {"bound": "alu", "kernel": "k_flux2, stage 1", "achieved": round(ach, 3), "peak": round(peak, 2),
            "unit": "TFLOP/s", "frac": round(ach / peak, 4),
            "traffic": None if ex is None else round(ex["dram_bytes_per_cell"] * n * n),
            "executed": None if ex is None else {

@@ -440,7 +440,12 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
     }
     total = align256(total + n * sizeof(double));
     cudaError_t e = cudaMalloc(&b->slab, total);
-    if (e != cudaSuccess) { cgks_batch_destroy(b); return e == cudaErrorMemoryAllocation ? CGKS_ENOMEM : CGKS_ECUDA; }
+    if (e != cudaSuccess) {
+        // reported here: not left as the runtime's last error for the caller's other code
+        cudaGetLastError();
+        cgks_batch_destroy(b);
+        return e == cudaErrorMemoryAllocation ? CGKS_ENOMEM : CGKS_ECUDA;
+    }
     b->dfixed = (double*)(b->slab + total - align256(n * sizeof(double)));
     b->host.resize(n);
     double K = p->dim == 2 ? (4.0 - 2.0 * p->gamma) / (p->gamma - 1.0) : (3.0 - p->gamma) / (p->gamma - 1.0);

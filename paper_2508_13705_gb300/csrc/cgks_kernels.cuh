@@ -91,8 +91,8 @@ __device__ __forceinline__ long long cell_idx(int dir, int na, int nb, int a, in
 }
 // FR rows are padded to 8 points (128 bytes of FP32), so that the strips of the
 // flux kernel start on whole memory sectors: unpadded, it read 1436 MB instead
-// of 917 at 1024^2
-__host__ __device__ __forceinline__ int fr_pitch(int n) { return (n + 7) & ~7; }
+// of 917 at 1024^2.  Unsigned: 1-D meshes go up to 2^31 - 3 cells
+__host__ __device__ __forceinline__ unsigned fr_pitch(int n) { return ((unsigned)n + 7u) & ~7u; }
 __device__ __forceinline__ long long fr_row(int dir, int na, int nb, int bb, int f)
 {
     return dir == 0 ? (long long)bb * fr_pitch(na + 1) + f : (long long)f * fr_pitch(nb + 2) + bb;

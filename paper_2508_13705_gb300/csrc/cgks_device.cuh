@@ -111,7 +111,11 @@ struct Mesh {
 // Prefix sums of the work items of every kernel over the meshes of a table,
 // and the first mesh's descriptor by value: a launch over one mesh reads its
 // descriptor from the kernel parameters (constant-bank operands) instead of
-// loading it from the table in every grid-stride iteration.
+// loading it from the table in every grid-stride iteration.  Kernels take it as
+// a __grid_constant__: where a pointer into it escapes (a CellMap's prescribed
+// state), the compiler otherwise copies all of it into every thread's local
+// memory, 880 bytes (500 x 250 cells between walls, order 5, FP32: a pass of 2602
+// instead of 1891 us).
 struct Work {
     const Mesh* mesh;
     const long long* off;  // [n+1] prefix of items

@@ -250,7 +250,7 @@ __device__ __forceinline__ void split(int t, int& q, int& r) { q = t / N; r = t 
 
 template <int M, typename R, bool WALLS, int DIR, bool ONE>
 __global__ void __launch_bounds__(ReconTile<R, DIR>::threads, sizeof(R) == 4 ? 768 / ReconTile<R, DIR>::threads : 1)
-k_recon(Work w, int stage)
+k_recon(const __grid_constant__ Work w, int stage)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned long long cnt[4];
@@ -577,7 +577,7 @@ k_recon(Work w, int stage)
 // their values loaded together, and each stencil sums only its own taps (80
 // cells FP64, 400 cells FP32: 21 -> 8 us).
 template <typename R, bool WALLS, bool ONE>
-__global__ void __launch_bounds__(256) k_normal1(Work w, int stage)
+__global__ void __launch_bounds__(256) k_normal1(const __grid_constant__ Work w, int stage)
 {
     __shared__ unsigned long long cnt[4];
     grid_wait();
@@ -1258,7 +1258,8 @@ __device__ __forceinline__ void flux_point(const Mesh& g, int dir, int na, int n
 // form has the uncapped one only (a capped compilation may contract its FP32
 // arithmetic differently, and results must not depend on tuning).
 template <typename R, int STAGE, int CAP, int HG, bool PF, bool ONE>
-__global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) : 1)) k_flux1(Work w)
+__global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) : 1))
+k_flux1(const __grid_constant__ Work w)
 {
     grid_wait();
     for (long long gi = blockIdx.x * (long long)blockDim.x + threadIdx.x; gi < w.total;
@@ -1289,7 +1290,7 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? (HG ? 3 : 4) 
 // 2-D: warps marching over strips of faces (above).  Dynamic shared memory:
 // FluxShared<M, R>::total values of R per warp.  Work offsets count steps.
 template <int M, typename R, int STAGE, int CAP, int HG, bool PF, bool ONE>
-__global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flux2(Work w)
+__global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flux2(const __grid_constant__ Work w)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_wait();
@@ -1455,7 +1456,7 @@ __device__ __forceinline__ double exact_diff(float r, float l)
 template <typename R> __device__ __forceinline__ void swap12(R* v) { const R z = v[1]; v[1] = v[2]; v[2] = z; }
 
 template <int M, typename R, int STAGE, bool ONE>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_update2(Work w)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_update2(const __grid_constant__ Work w)
 {
     grid_wait();
     constexpr bool BULK32 = sizeof(R) == 4;
@@ -1659,7 +1660,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_update2(Work w)
 
 // -------------------------------------------------------------- update (1-D)
 template <typename R, int STAGE, bool ONE>
-__global__ void __launch_bounds__(256) k_update1(Work w)
+__global__ void __launch_bounds__(256) k_update1(const __grid_constant__ Work w)
 {
     grid_wait();
     constexpr bool BULK32 = sizeof(R) == 4;
@@ -1734,7 +1735,7 @@ __global__ void __launch_bounds__(256) k_update1(Work w)
 // otherwise the float slope planes -> the FP64 planes (before a state is read
 // out; the FP64 cell averages are already current).
 template <int D, int M>
-__global__ void __launch_bounds__(256) k_convert(Work w, int to_float)
+__global__ void __launch_bounds__(256) k_convert(const __grid_constant__ Work w, int to_float)
 {
     constexpr int NP = D == 2 ? 12 + 8 * M : 6;
     constexpr int NV = D + 2;
@@ -1781,7 +1782,7 @@ __device__ __forceinline__ void set_step(const Mesh& g, double dt)
 // which saves a launch (and the host two copies): MODE 1 sets the step, MODE 2
 // writes the maximum to *out, mapped host memory.
 template <int D, typename R, int MODE>
-__global__ void __launch_bounds__(256) k_cfl(Work w, double* out)
+__global__ void __launch_bounds__(256) k_cfl(const __grid_constant__ Work w, double* out)
 {
     grid_wait();
     __shared__ double red[8];
@@ -1903,7 +1904,7 @@ __device__ __forceinline__ double sigma_of(const Mach& l, const Mach& r)
 }
 
 template <int D>
-__global__ void k_sigma_init(Work w)
+__global__ void k_sigma_init(const __grid_constant__ Work w)
 {
     for (long long gi = blockIdx.x * (long long)blockDim.x + threadIdx.x; gi < w.total;
          gi += (long long)gridDim.x * blockDim.x) {
@@ -1929,7 +1930,7 @@ __global__ void k_sigma_init(Work w)
 
 // positivity of a state set in (host-side check is done on the device)
 template <int D>
-__global__ void k_check_state(Work w)
+__global__ void k_check_state(const __grid_constant__ Work w)
 {
     for (long long gi = blockIdx.x * (long long)blockDim.x + threadIdx.x; gi < w.total;
          gi += (long long)gridDim.x * blockDim.x) {

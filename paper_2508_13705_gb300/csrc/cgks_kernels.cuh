@@ -1609,19 +1609,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_update2(const _
                     ff ax = ff_add(ff_two_sum((float)gxr[NO - 1][v], -(float)gxl[NO - 1][v]), ff_mul(fdt, Bx[v]));
                     ff ay = ff_add(ff_two_sum((float)gyr[NO - 1][v], -(float)gyl[NO - 1][v]), ff_mul(fdt, By[v]));
                     g.ACC[v * P + c] = W0[v] - ff_val(ff_add(ff_mul(ax, ix), ff_mul(ay, iy)));
-                    // Eq. 2.21: W*, held as hi + lo only, from W's hi + lo in float-float
-                    // (the FP64 pipe was half busy with conversions)
-                    const ff ws = ff_add({(float)h0[v], g.F0[(12 + 8 * M + v) * P + c]},
-                                         ff_neg(ff_add(ff_mul(tx, ix), ff_mul(ty, iy))));
-                    bad |= !isfinite(ws.hi);
-                    outf[v * P + c] = ws.hi;
-                    outf[(12 + 8 * M + v) * P + c] = ws.lo;
-                    outf[(4 + v) * P + c] = (float)sx[v];  // cell slopes: Gauss sum of the line slopes
-                    outf[(8 + v) * P + c] = (float)sy[v];
-                    continue;
-                } else {
-                    Wn = W0[v] - ff_val(ff_add(ff_mul(tx, ix), ff_mul(ty, iy)));  // Eq. 2.22-2.23
                 }
+                // Eq. 2.21, 2.22-2.23: from the FP64 average or its accumulator, in FP64
+                Wn = W0[v] - ff_val(ff_add(ff_mul(tx, ix), ff_mul(ty, iy)));
             } else {
                 const double dx0 = exact_diff(gxr[0][v], gxl[0][v]), dy0 = exact_diff(gyr[0][v], gyl[0][v]);
                 if (STAGE == 1) {

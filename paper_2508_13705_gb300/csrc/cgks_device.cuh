@@ -720,11 +720,14 @@ __device__ __forceinline__ void with_stencil(int st, Body&& body)
 // tau = 0 (two stages), and the FP32 one, then bound by load latency, from
 // 889 + 770 to 768 + 680 us at 1024^2.
 
-// 1 / x.  FP32: the hardware's approximation (1 ulp) and one Newton step, r +
-// r (1 - x r) with fused operations, which leaves the correctly rounded value
-// but for rare last bits; the compiled division tests for subnormal operands
-// and results besides, a fifth of the flux kernel's integer instructions.
-// x = 0 and infinite x give NaN: no physical density or pressure.
+// 1 / x.  FP32: the hardware's approximation r (PTX states 1 ulp for
+// rcp.approx) and one step of the Newton-Raphson iteration for 1 / r - x = 0, r + r
+// (1 - x r), with the residual in one fused operation (as in Markstein, IBM J.
+// Res. Dev. 34, 1990): its error d becomes d^2, so that the result is within 0.5 +
+// 2^-21 ulp of 1 / x wherever both are normal numbers.  x = 0, infinite x and x
+// whose reciprocal overflows give NaN: no physical density or pressure.  1.0f / x
+// in its place: 1024^2, order 9, 9670 against 9514 us for five steps, 2048^2 with
+// finite tau 18967 against 18808 for two.
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 __device__ __forceinline__ float recip(float x)
 {
@@ -733,8 +736,9 @@ __device__ __forceinline__ float recip(float x)
     return __fmaf_rn(r, __fmaf_rn(-x, r, 1.0f), r);
 }
 
-// 1 / sqrt(x).  FP32: the approximation (2 ulp) and one Newton step; without it
-// the half-range moments of a shock's two sides carry its error.
+// 1 / sqrt(x).  FP32: rsqrtf (2 ulp stated) and one Newton-Raphson step for
+// 1 / r^2 - x = 0, r + r (1 - x r^2) / 2: within 1 ulp, of which the rounding of x r is
+// half; without it the half-range moments of a shock's two sides carry rsqrtf's error.
 __device__ __forceinline__ double recip_sqrt(double x) { return rsqrt(x); }
 __device__ __forceinline__ float recip_sqrt(float x)
 {

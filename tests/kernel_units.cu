@@ -59,3 +59,20 @@ extern "C" int unit_stage1_averages(int nx, int ny, double h, const double* W, c
     cudaMemcpy(lo, F1.p + NP * P, 4 * P * sizeof(float), cudaMemcpyDeviceToHost);
     return 0;
 }
+
+// recip and recip_sqrt of floats
+__global__ void k_reciprocals(const float* x, float* r, float* q, int n)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    r[i] = recip(x[i]);
+    q[i] = recip_sqrt(x[i]);
+}
+extern "C" int unit_reciprocals(const float* x, float* r, float* q, int n)
+{
+    Array<float> X(n, x), A(n), B(n);
+    if (!X.p || !A.p || !B.p) return 1;
+    k_reciprocals<<<(n + 255) / 256, 256>>>(X.p, A.p, B.p, n);
+    return cudaMemcpy(r, A.p, n * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess ||
+           cudaMemcpy(q, B.p, n * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess;
+}

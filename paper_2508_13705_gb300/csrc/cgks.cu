@@ -597,7 +597,6 @@ int status_of(cgks_batch* b, long long* bad_out)
 struct StateArrays {
     double* a[5];
     long long end[5];
-    int n;
 };
 
 // FP32-bulk form, device arrays: straight between the caller's FP64 arrays and
@@ -670,7 +669,6 @@ bool state_arrays(const cgks_batch* b, int k, const double* W, const double* Wx,
         if (at.type != cudaMemoryTypeDevice || at.device != dev || ((size_t)a[q] & 7)) return false;
         if (!in_one_allocation(a[q], planes[q] * P * sizeof(double))) return false;
     }
-    s.n = 5;
     return true;
 }
 
@@ -1000,7 +998,7 @@ int cgks_compute_dt(cgks_solver* s, double* dt)
     if (!s || !dt) return CGKS_EINVAL;
     cgks_batch* b = s->b;
     if (!b->host_smax) {
-        // also while another stream of this program is being captured
+        // also beside the capture of another stream in relaxed mode or by another thread
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
         CK(cudaThreadExchangeStreamCaptureMode(&mode));
         const cudaError_t e = cudaHostAlloc((void**)&b->host_smax, sizeof(double), cudaHostAllocMapped);

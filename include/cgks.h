@@ -219,20 +219,18 @@ int cgks_get_stats(cgks_solver* s, cgks_stats* st);
 
 /* Autotuner: times the stage kernels that have more than one launch shape on
  * the solver's current state and keeps the fastest; the step graph is rebuilt on
- * the next step.  Block sizes are tried from 32 (2-D updates: from 64) up to the
- * kernel's largest (flux 128, others 256; persistent grid = SM count x resident
- * blocks), the FP64 flux kernels also in a register-capped variant (more
- * resident warps, some spilling).  The 2-D Steps 1-2 (one fused kernel per
- * direction over tiles held in shared memory, a block per tile) have one shape.
- * The state is not advanced (only scratch is written; the simulated time, the
- * status word and the fallback count are restored) and results do not depend
- * on the choice: the arithmetic of a cell, and of a face of the warps that share
- * a strip of faces, is the same in any block.  threads_out (may be NULL) receives
- * 10 ints: the block sizes of Steps 1-2 along x and y (1-D: 0
- * and Step 2), flux (stage 1, 2), update (stage 1, 2), then the tile shapes
- * TA x TB (cells along the face normal x across it) along x and y (0 in 1-D); a
- * negative flux entry marks the capped variant.  Requires a state (CGKS_EINVAL
- * otherwise). */
+ * the next step.  Block sizes 64..256 are tried (1-D: from 32; fluxes: up to 128;
+ * persistent grid = SM count x resident blocks), the FP64 flux kernels also in a
+ * register-capped variant (more resident warps, some spilling).  The 2-D Steps 1-2
+ * (one fused kernel per direction over tiles held in shared memory, a block per
+ * tile) have one shape.  The state is not advanced (only scratch is written; the
+ * simulated time, the status word and the fallback count are restored) and
+ * results do not depend on the choice: a cell's arithmetic, and a face's in the
+ * warp that takes its strip, is the same in any block.  threads_out (may be NULL)
+ * receives 10 ints: the block sizes of Steps 1-2 along x and y (1-D: 0 and Step 2),
+ * flux (stage 1, 2), update (stage 1, 2), then the tile shapes TA x TB (cells along
+ * the face normal x across it) along x and y (0 in 1-D); a negative flux entry
+ * marks the capped variant.  Requires a state (CGKS_EINVAL otherwise). */
 int cgks_autotune(cgks_solver* s, int* threads_out);
 int cgks_batch_autotune(cgks_batch* b, int* threads_out);
 

@@ -23,8 +23,9 @@
 //
 // Precision: R is the type of the reconstruction and kinetic arithmetic
 // (double, or float for the FP32-bulk form).  Cell averages and their
-// accumulation, the DFF (sigma, alpha, branch tests) and the positivity
-// tests are always FP64.
+// accumulation, the DFF (the sums of sigma, alpha and the branch tests), the check
+// of a state that is set and the point fallback's test are always FP64; a face's
+// sigma and the flux kernels' positivity flag are evaluated in R.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -856,7 +857,11 @@ template <typename R, int NM>
 struct Range { R m[NM]; R k, hk; };
 
 // erfc(x) / 2 for x >= 0, e = exp(-x^2).  FP64: the scaled function takes the
-// exponential that f(0) needs anyway; FP32: erfcf alone is the shorter.
+// exponential that f(0) needs anyway, which then scales m_0 and f(0) alike: where
+// they cancel in m_1 and m_2 (x > 1/2) those are as accurate as with erfc(x) or up to a
+// quarter better, below they carry 1-3 ulp more; the fields' errors against 64
+// bits are the same to 1%, and erfc(x) takes 17597 -> 18145 us at 512^2, order 9 (two
+// steps).  FP32: erfcf alone is the shorter.
 __device__ __forceinline__ double half_erfc(double x, double e) { return 0.5 * e * erfcx(x); }
 __device__ __forceinline__ float half_erfc(float x, float) { return 0.5f * erfcf(x); }
 

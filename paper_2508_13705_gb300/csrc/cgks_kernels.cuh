@@ -1,6 +1,7 @@
 // Stage kernels of the ASE-DFF-CGKS step.  See cgks_device.cuh for the
-// mathematics; this file maps it onto grid-stride loops over the work items
-// of every mesh in a descriptor table.
+// mathematics; this file maps it onto the work items of every mesh in a
+// descriptor table: a block per tile in the 2-D Steps 1-2, a contiguous run of
+// strips per warp in the 2-D flux, grid-stride loops in the other kernels.
 //
 // Local frame of a direction: dir 0 (faces normal to x): a = i (normal
 // index), b = j (tangential); dir 1 (faces normal to y): a = j, b = i.
@@ -1437,19 +1438,6 @@ __global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flu
 }
 
 // -------------------------------------------------------------- update (2-D)
-// r - l exactly, as a double: in FP64 the difference itself; in FP32 the
-// rounded difference plus its rounding error (Knuth's two-sum), each exact
-// in a double.
-__device__ __forceinline__ double exact_diff(double r, double l) { return r - l; }
-__device__ __forceinline__ double exact_diff(float r, float l)
-{
-    float b = -l;
-    float s = r + b;
-    float z = s - r;
-    float e = (r - (s - z)) + (b - z);
-    return (double)s + (double)e;
-}
-
 // Stage 1 writes W* (S1) and the accumulator; stage 2 writes state n+1 (S0).
 // FP32-bulk form: the float planes (F1 / F0) receive everything the next stage
 // reads, the FP64 planes the cell averages of state n+1 (W* lives in F1 only).
@@ -1482,10 +1470,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_update2(const _
         float* outf = STAGE == 1 ? g.F1 : g.F0;
         const auto& TR = Tab<R>::get(g.oi);
         // Conserved quantities: the Gauss sum over a face's points was formed
-        // per face, in the bulk precision, and the difference of a cell's two
-        // face sums is taken exactly (exact_diff) into the FP64 averages, so
-        // the updates telescope over the mesh and the totals change only by
-        // the boundary fluxes and FP64 rounding.  Slopes use bulk differences.
+        // per face, in the bulk precision, and both cells of a face use it.  The
+        // difference of a cell's two face sums is taken in FP64 or, FP32 bulk, in
+        // float-float (exactly, by a two-sum), scaled, and subtracted from the
+        // FP64 average in FP64: the updates telescope over the mesh and the totals
+        // change only by the boundary fluxes and by rounding at FP64's level.
+        // Slopes use bulk differences.
         // FP32 bulk, stage 1: the face outputs are increments over hi of each
         // face's right cell (this cell for the left and bottom faces, cells
         // (i+1, j) and (i, j+1) for the others).  Their flux parts add
@@ -1613,12 +1603,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_update2(const _
                 // Eq. 2.21, 2.22-2.23: from the FP64 average or its accumulator, in FP64
                 Wn = W0[v] - ff_val(ff_add(ff_mul(tx, ix), ff_mul(ty, iy)));
             } else {
-                const double dx0 = exact_diff(gxr[0][v], gxl[0][v]), dy0 = exact_diff(gyr[0][v], gyl[0][v]);
+                const double dx0 = gxr[0][v] - gxl[0][v], dy0 = gyr[0][v] - gyl[0][v];
                 if (STAGE == 1) {
                     const double W = W0[v];
                     Wn = W - dx0 * idx - dy0 * idy;  // Eq. 2.21
-                    g.ACC[v * P + c] = W - exact_diff(gxr[NO - 1][v], gxl[NO - 1][v]) * idx
-                                     - exact_diff(gyr[NO - 1][v], gyl[NO - 1][v]) * idy;
+                    g.ACC[v * P + c] = W - (double)(gxr[NO - 1][v] - gxl[NO - 1][v]) * idx
+                                     - (double)(gyr[NO - 1][v] - gyl[NO - 1][v]) * idy;
                 } else {
                     Wn = W0[v] - dx0 * idx - dy0 * idy;  // Eq. 2.22-2.23
                 }
@@ -1841,7 +1831,8 @@ __global__ void __launch_bounds__(256) k_cfl(const __grid_constant__ Work w, dou
     }
 }
 
-// dt = cfl / smax per mesh (or the fixed value); t^n = t, t += dt; reset the reduction
+// dt = cfl / smax per mesh (or the fixed value); t^n = t, t += dt; reset the
+// reduction.  A template, so that only the unit that launches it holds it.
 template <int Unused = 0>
 __global__ void k_dt(Mesh* meshes, int n, int use_cfl, const double* fixed)
 {

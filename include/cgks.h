@@ -220,9 +220,9 @@ int cgks_get_stats(cgks_solver* s, cgks_stats* st);
 /* Autotuner: times the stage kernels that have more than one launch shape on
  * the solver's current state and keeps the fastest; the step graph is rebuilt on
  * the next step.  Block sizes 64..256 are tried (1-D: from 32; fluxes: up to 128;
- * persistent grid = SM count x resident blocks), the FP64 flux kernels also in a
- * register-capped variant (more resident warps, some spilling).  The 2-D Steps 1-2
- * (one fused kernel per direction over tiles held in shared memory, a block per
+ * persistent grid = SM count x resident blocks), the 1-D FP64 flux kernels also in
+ * a register-capped variant (more resident warps, some spilling).  The 2-D Steps
+ * 1-2 (one fused kernel per direction over tiles held in shared memory, a block per
  * tile) have one shape.  The state is not advanced (only scratch is written; the
  * simulated time, the status word and the fallback count are restored) and
  * results do not depend on the choice: a cell's arithmetic, and a face's in the

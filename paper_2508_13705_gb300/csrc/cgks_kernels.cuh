@@ -1290,8 +1290,12 @@ k_flux1(const __grid_constant__ Work w)
 
 // 2-D: warps marching over strips of faces (above).  Dynamic shared memory:
 // FluxShared<M, R>::total values of R per warp.  Work offsets count steps.
-template <int M, typename R, int STAGE, int CAP, int HG, bool PF, bool ONE>
-__global__ void __launch_bounds__(128, CAP ? 4 : (sizeof(R) == 4 ? 4 : 1)) k_flux2(const __grid_constant__ Work w)
+// FP32: 4 blocks of 128 threads per SM (128 registers).  FP64: a warp's ring takes
+// 21-23 KB, so that 8 to 10 warps fit an SM, which its 164-226 registers allow
+// (a variant capped at 128 registers only spilled: of 72 tuned fluxes between
+// 12^2 and 512^2 cells 3 took it, on small meshes, where the timings scatter).
+template <int M, typename R, int STAGE, int HG, bool PF, bool ONE>
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 4 : 1) k_flux2(const __grid_constant__ Work w)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_wait();

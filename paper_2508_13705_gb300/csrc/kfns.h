@@ -17,7 +17,7 @@ struct Kfns {
     KOne flux1, flux2, upd1, upd2, siginit, check;
     KCfl cfl[3];               // CFL reduction: alone, with the step set, to the host
     KStage convert;  // FP32-bulk state copies (to_float = 1: FP64 -> float planes)
-    KOne flux1v[2], flux2v[2];  // flux variants: [0] uncapped, [1] register-capped (tau = 0)
+    KOne flux1v[2], flux2v[2];  // flux variants: [0] uncapped, [1] register-capped (tau = 0; 1-D FP64, else [0])
     KOne flux1h[2], flux2h[2];  // the same with the collision-time terms (tau > 0)
     int flux_warp_bytes;        // dynamic shared memory of the 2-D flux kernels per warp
     KOne flux1p, flux2p;        // tau > 0 with the first-order fallback at face points

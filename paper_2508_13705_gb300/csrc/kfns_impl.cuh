@@ -17,7 +17,7 @@ int upload_tables(const CgksTables* t3, const TabF* f3)
 template <int D, int M, typename R, int STAGE, int CAP, int HG, bool PF, bool ONE>
 constexpr KOne flux_fn()
 {
-    if constexpr (D == 2) return k_flux2<M, R, STAGE, CAP, HG, PF, ONE>;
+    if constexpr (D == 2) return k_flux2<M, R, STAGE, HG, PF, ONE>;
     else return k_flux1<R, STAGE, CAP, HG, PF, ONE>;
 }
 
@@ -48,8 +48,9 @@ Kfns make_kfns_one()
     k.flux2h[0] = flux_fn<D, M, R, 2, 0, 1, false, ONE>();
     // the register-capped variants round exactly like the uncapped ones in
     // FP64 only (the compiler may contract the FP32 arithmetic differently),
-    // so the FP32-bulk form offers the autotuner one variant
-    if constexpr (sizeof(R) == 8) {
+    // so the FP32-bulk form offers the autotuner one variant; so do the 2-D
+    // fluxes, whose warps shared memory bounds
+    if constexpr (sizeof(R) == 8 && D == 1) {
         k.flux1v[1] = flux_fn<D, M, R, 1, 1, 0, false, ONE>();
         k.flux2v[1] = flux_fn<D, M, R, 2, 1, 0, false, ONE>();
         k.flux1h[1] = flux_fn<D, M, R, 1, 1, 1, false, ONE>();

@@ -540,8 +540,12 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
                               (const void*)b->k.cfl[0]};
         for (int q = 0; q < 7; ++q) {
             int occ = 1;
-            // 1-D meshes and small 2-D ones: small blocks, which spread over the SMs
-            // (80 cells FP64: flux 18 -> 8 us, its FP64 pipe being the SM's)
+            // 1-D meshes and small 2-D ones: small blocks, which spread over the SMs,
+            // whose FP64 pipes and latencies bound them.  A step with blocks of 128
+            // (fluxes) and 256 (others) against these, us: 1-D FP64, 2000 cells 78, 59, 80
+            // cells alike; 2-D order 9, 24^2 FP64 188, 172, FP32 58.4, 57.4; 64^2 FP64
+            // 260, 240, FP32 58.2, 55.0.  The small others lose at 100^2 (FP64 473,
+            // 508; FP32 75.9, 77.7), and are even from 160^2 on.
             const long long all = b->off[(size_t)W_CELLS * (n + 1) + n];
             const bool small = p->dim == 1 || all < 512LL * b->nsm;
             int th = p->dim == 1 ? 32 : (q == 2 || q == 3) ? 128 : (small ? 64 : 256);

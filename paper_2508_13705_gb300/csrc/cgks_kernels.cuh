@@ -876,9 +876,9 @@ struct StripPoint {
 // A face's Gauss sums of its points' fluxes and the mean of their sigma, over
 // the M lanes of the face (all lanes of the warp take part).  Each lane ends up
 // with a share of the sums and writes it: the update reads one value per face
-// where it read M: 1024^2, order 9, FP32, the updates took 307 + 160 us, now 199 +
-// 150 (with three blocks of 256 threads per SM), the fluxes 395 + 354, now 418 +
-// 364; at 2048^2, order 5, 905 + 413 -> 508 + 393 and 770 + 703 -> 821 + 721.
+// where it read M: 1024^2, order 9, FP32, the updates took 307 + 160 us, now 189 +
+// 150 (with 24 warps per SM), the fluxes 395 + 354, now 418 +
+// 364; at 2048^2, order 5, 905 + 413 -> 518 + 399 and 770 + 703 -> 821 + 721.
 __device__ __forceinline__ float swap_lane(float v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 __device__ __forceinline__ double swap_lane(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 

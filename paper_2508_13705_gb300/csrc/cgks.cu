@@ -576,7 +576,7 @@ int batch_create(cgks_batch** out, const cgks_params* p, int n, const int* nx, c
                     rr = CGKS_ECUDA;
             }
     } while (0);
-    if (rr) { cgks_batch_destroy(b); return rr; }
+    if (rr) { cudaGetLastError(); cgks_batch_destroy(b); return rr; }  // as above
     *out = b;
     return CGKS_OK;
 }
